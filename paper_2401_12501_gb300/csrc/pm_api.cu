@@ -12,6 +12,7 @@
 #include "pm_internal.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdlib>
@@ -45,6 +46,11 @@ extern "C" const char* pm_status_str(pm_status st) {
         case PM_ERR_NO_COEFF: return "no coefficient set";
     }
     return "unknown status";
+}
+
+long long pm_new_epoch() {
+    static std::atomic<long long> next{1};
+    return next.fetch_add(1, std::memory_order_relaxed);
 }
 
 extern "C" void pm_default_opts(pm_opts* o) {
@@ -576,7 +582,7 @@ extern "C" pm_status pm_surface_tune(pm_surface* s, int direct_tpt, int direct_b
     }
     s->opts.direct_tpt = direct_tpt;
     s->opts.direct_blocks_per_sm = direct_blocks_per_sm;
-    s->graph_epoch++;
+    s->graph_epoch = pm_new_epoch();
     return PM_OK;
 }
 
@@ -639,7 +645,7 @@ extern "C" pm_status pm_surface_set_coeff(pm_surface* s, const double* a, const 
     PM_CUDA_TRY(cudaStreamSynchronize(st));
     s->has_coeff = true;
     s->has_c = 0;
-    s->graph_epoch++;
+    s->graph_epoch = pm_new_epoch();
     s->coeff_epoch++;
     return PM_OK;
 }

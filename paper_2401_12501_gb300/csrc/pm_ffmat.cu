@@ -655,7 +655,7 @@ extern "C" pm_status pm_surface_store_ff(pm_surface* s, int which) {
     PM_CUDA_TRY(cudaDeviceSynchronize());
     if (which == 0) {
         pm_ffmat_free(s);
-        s->graph_epoch++;
+        s->graph_epoch = pm_new_epoch();
         return PM_OK;
     }
     if (!s->has_coeff) {
@@ -667,7 +667,7 @@ extern "C" pm_status pm_surface_store_ff(pm_surface* s, int which) {
         return PM_ERR_INVALID_ARG;
     }
     pm_ffmat_free(s);
-    s->graph_epoch++;
+    s->graph_epoch = pm_new_epoch();
     const size_t need = pm_ffmat_bytes(s, which);
     const size_t fr = pm_free_hbm_bytes();
     size_t total = 0, fr_real = 0;

@@ -422,7 +422,7 @@ extern "C" pm_status pm_surface_set_coeff_c(pm_surface* s, const double* a, cons
     }
     PM_TRY(pm_near_build_c(s));
     s->has_c = 1;
-    s->graph_epoch++;
+    s->graph_epoch = pm_new_epoch();
     s->coeff_epoch++;
     return PM_OK;
 }

@@ -117,6 +117,9 @@ struct PmSharedBuffers {
     ~PmSharedBuffers();
 };
 
+// a value no earlier call of the process returned (pm_api.cu)
+long long pm_new_epoch();
+
 struct PmSolveWork;
 struct PmFmmTree;
 struct PmBatchWork;
@@ -215,7 +218,10 @@ struct pm_surface {
 
     // per-phase timing (events recorded around launches while enabled)
     bool profiling = false;
-    long long graph_epoch = 0;    // bumped when buffers or launch shapes captured in graphs change
+    // renewed when buffers or launch shapes captured in graphs change; no two surfaces ever
+    // share a value, so a workspace that remembers (address, epoch) cannot take a new surface
+    // for a destroyed one at the same address
+    long long graph_epoch = pm_new_epoch();
     long long coeff_epoch = 0;    // bumped by every coefficient change (set_coeff, set_coeff_c)
     std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> prof_events;
     double prof_ms[PM_PHASE_COUNT] = {};

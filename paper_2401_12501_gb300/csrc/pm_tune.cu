@@ -48,7 +48,7 @@ void apply_knobs(pm_surface* s, const pm_knobs& k) {
     s->batch_bps = k.batch_blocks_per_sm;
     s->opts.fmm_depth = k.fmm_depth;
     s->fmm_streams = k.fmm_streams;
-    s->graph_epoch++;      // captured solve graphs hold launch shapes
+    s->graph_epoch = pm_new_epoch();      // captured solve graphs hold launch shapes
 }
 
 struct TuneBuffers {

@@ -111,3 +111,24 @@ def test_multi_argument_checks(ctx):
         assert abs(info[0][0].removed_mean - 1.0) < 1e-9 and info[0][0].residual <= 1e-9
     finally:
         s.close()
+
+
+def test_workspace_follows_recreated_operators(ctx):
+    """Operators destroyed and created again in one context, often at the same host
+    address, with the same coefficient history: the batch solves the new ones."""
+    import paper_2401_12501_gb300 as pm
+    from workloads import cubed_sphere
+    from workloads.rhs import random_harmonic_rhs
+    for k in range(6):
+        s = cubed_sphere(1, 6, axes=(1.0, 1.0 + 0.1 * k, 2.0))
+        f = random_harmonic_rhs(s, k)
+        ops = [pm.Surface.from_fixture(ctx, s)]
+        ops[0].set_coeff(np.full(s.N, 1.0 + k))
+        ops.append(ops[0].clone())
+        ops[1].set_coeff(np.full(s.N, 2.0 + k))
+        us, _ = pm.solve_multi(ops, [f, f], tol=1e-10)
+        for op, u in zip(ops, us):
+            ref, _ = op.solve(f, tol=1e-10)
+            assert np.abs(u - ref).max() <= 1e-8 * np.abs(ref).max()
+        for op in ops:
+            op.close()
