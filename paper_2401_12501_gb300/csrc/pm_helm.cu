@@ -8,8 +8,10 @@
 // -K0(kappa r)/(2 pi) is real, but one path serves both signs, a c whose sign
 // changes over the surface and complex c, whose kernels take K0, K1 at complex
 // argument, pm_green.cuh).  Arithmetic is float64 throughout:
-//   - smooth sums: one thread per target, sources staged through shared memory,
-//     split over gridDim.y, g, g', g'' from pm_green.cuh at every pair;
+//   - smooth sums of an apply: one thread per target, sources staged through shared
+//     memory, split over gridDim.y, g, g', g'' from pm_green.cuh at every pair;
+//   - a solve evaluates the pairs once, into dense matrices of both operators (corrections
+//     included) that its Krylov steps stream, where 32 N^2 bytes fit; else the sums above;
 //   - near field: complex corrections from pm_nearfield.cu (pm_near_build_c);
 //   - GMRES(m) with classical Gram-Schmidt applied twice; the Krylov vectors and
 //     the orthogonalisation stay on the device, the (m+1) x m Hessenberg matrix and
@@ -96,6 +98,100 @@ k_direct_c64(const double* __restrict__ x, const double* __restrict__ n,
         }
     }
     if (i < N) partial[(size_t)blockIdx.y * N + i] = make_double2(are, aim);
+}
+
+// The operators of one solve as dense matrices: MR[i][j] = w_j R(x_i, x_j) and MK likewise
+// (the density's factors, j != i; 0 on the diagonal), both from one evaluation of the
+// Green's function.  Block: kHT sources (one a thread, so rows are written coalesced) x
+// kFillRows targets staged in shared memory.  Bound by the float64 pipe like k_direct_c64,
+// which a solve without the matrices runs once per Krylov step and residual.
+constexpr int kFillRows = 32;
+__global__ void __launch_bounds__(kHT)
+k_fill_c64(const double* __restrict__ x, const double* __restrict__ n,
+           const double* __restrict__ H, const double* __restrict__ a,
+           const double* __restrict__ g, const double2* __restrict__ c,
+           const double2* __restrict__ qn, const double* __restrict__ wa, int N,
+           double2* __restrict__ MR, double2* __restrict__ MK) {
+    __shared__ double st[kFillRows][13];   // x, n, grad a, H, a, Re c, Im c
+    const int i0 = blockIdx.y * kFillRows, rows = min(kFillRows, N - i0);
+    for (int e = threadIdx.x; e < rows * 13; e += kHT) {
+        const int r = e / 13, k = e - r * 13, i = i0 + r;
+        st[r][k] = k < 3 ? x[3 * i + k] : k < 6 ? n[3 * i + k - 3] : k < 9 ? g[3 * i + k - 6]
+                 : k == 9 ? H[i] : k == 10 ? a[i] : k == 11 ? c[i].x : c[i].y;
+    }
+    __syncthreads();
+    const int j = blockIdx.x * kHT + threadIdx.x;
+    if (j >= N) return;
+    const double xj0 = x[3 * j], xj1 = x[3 * j + 1], xj2 = x[3 * j + 2], wj = wa[j];
+    const pm_green::cplx_d qj = {qn[j].x, qn[j].y};
+    for (int r = 0; r < rows; ++r) {
+        const double* t = st[r];
+        double out[4] = {0.0, 0.0, 0.0, 0.0};
+        if (i0 + r != j)
+            pm_green::pair_rk_cz(t[0] - xj0, t[1] - xj1, t[2] - xj2, t[3], t[4], t[5], t[9], t[10],
+                                 t[6], t[7], t[8], pm_green::cplx_d{t[11], t[12]}, qj, cHG16,
+                                 cHG16 + PM_GL16, out);
+        const size_t o = (size_t)(i0 + r) * N + j;
+        MR[o] = make_double2(wj * out[0], wj * out[1]);
+        MK[o] = make_double2(wj * out[2], wj * out[3]);
+    }
+}
+
+// the near-field corrections added into the matrices (every entry of a block is its own)
+__global__ void k_fill_near_c(int nblk, int pp, const int* __restrict__ blk_row,
+                              const int* __restrict__ blk_patch, const double2* __restrict__ cR,
+                              const double2* __restrict__ cK, int N, double2* __restrict__ MR,
+                              double2* __restrict__ MK) {
+    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= (size_t)nblk * pp) return;
+    const int b = (int)(e / pp), k = (int)(e - (size_t)b * pp);
+    const size_t o = (size_t)blk_row[b] * N + (size_t)blk_patch[b] * pp + k;
+    const double2 r = MR[o], q = MK[o];
+    MR[o] = make_double2(r.x + cR[e].x, r.y + cR[e].y);
+    MK[o] = make_double2(q.x + cK[e].x, q.y + cK[e].y);
+}
+
+// out = M v (+ v when add): kGemvRowsC rows a block, so that each v_j is read once for them
+constexpr int kGemvRowsC = 4;
+__global__ void __launch_bounds__(kHT)
+k_dense_c64(const double2* __restrict__ M, const double2* __restrict__ v, int add, int N,
+            double2* __restrict__ out) {
+    __shared__ double2 sh[kGemvRowsC][kHT / 32];
+    const int i0 = blockIdx.x * kGemvRowsC;
+    const double2* row[kGemvRowsC];
+    double2 acc[kGemvRowsC];
+    for (int r = 0; r < kGemvRowsC; ++r) {
+        row[r] = M + (size_t)min(i0 + r, N - 1) * N;
+        acc[r] = make_double2(0.0, 0.0);
+    }
+#pragma unroll 2
+    for (int j = threadIdx.x; j < N; j += kHT) {
+        const double2 vj = v[j];
+#pragma unroll
+        for (int r = 0; r < kGemvRowsC; ++r) {
+            const double2 m = row[r][j];
+            acc[r].x = fma(m.x, vj.x, fma(-m.y, vj.y, acc[r].x));
+            acc[r].y = fma(m.x, vj.y, fma(m.y, vj.x, acc[r].y));
+        }
+    }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int r = 0; r < kGemvRowsC; ++r) {
+        for (int o = 16; o > 0; o >>= 1) {
+            acc[r].x += __shfl_down_sync(0xffffffffu, acc[r].x, o);
+            acc[r].y += __shfl_down_sync(0xffffffffu, acc[r].y, o);
+        }
+        if (lane == 0) sh[r][wid] = acc[r];
+    }
+    __syncthreads();
+    const int r = threadIdx.x, i = i0 + r;
+    if (r < kGemvRowsC && i < N) {
+        double2 t = add ? v[i] : make_double2(0.0, 0.0);
+        for (int k = 0; k < kHT / 32; ++k) {
+            t.x += sh[r][k].x;
+            t.y += sh[r][k].y;
+        }
+        out[i] = t;
+    }
 }
 
 // out_i = sum_s partial[s][i] + sum_{b in row i} sum_k C[b][k] sigma[patch_b][k] (warp per row)
@@ -330,11 +426,55 @@ pm_status helm_apply(pm_surface* s, int which_K, const double2* sigma, double2* 
     return PM_OK;
 }
 
+// Both dense matrices of one solve, given back when it ends; empty (MR null) where the
+// device has no room for them beside a margin.
+struct HelmDense {
+    double2 *MR = nullptr, *MK = nullptr;
+    cudaStream_t st = 0;
+    ~HelmDense() {
+        if (MR) cudaFreeAsync(MR, st);
+    }
+    // 32 N^2 bytes.  One evaluation of the pairs serves every step, residual and the
+    // representation; the pair sums evaluate all of them each time.  A solve to 1e-12 on the
+    // GB300: 3,456 nodes with c/a > 0 206 -> 14.7 ms, 864 nodes with complex c 878 -> 28.7 ms.
+    pm_status fill(pm_surface* s) {
+        const size_t N = s->N, need = 2 * sizeof(double2) * N * N;
+        size_t fr = 0, total = 0;
+        PM_CUDA_TRY(cudaMemGetInfo(&fr, &total));
+        if (need + std::max<size_t>(1ull << 30, total / 50) > pm_free_hbm_bytes()) return PM_OK;
+        if (cudaMallocAsync((void**)&MR, need, st) != cudaSuccess) {
+            cudaGetLastError();
+            MR = nullptr;
+            return PM_OK;
+        }
+        MK = MR + N * N;
+        PhaseTimer t(s, PM_PHASE_DIRECT64, st);
+        dim3 grid(pm_ceil_div(s->N, kHT), pm_ceil_div(s->N, kFillRows));
+        k_fill_c64<<<grid, kHT, 0, st>>>(s->x, s->n, s->H, s->a, s->g, s->cc, s->qn, s->wa, s->N,
+                                         MR, MK);
+        k_fill_near_c<<<pm_ceil_div((long long)s->nblk * s->pp, 256), 256, 0, st>>>(
+            s->nblk, s->pp, s->blk_row, s->blk_patch, s->cRc, s->cKc, s->N, MR, MK);
+        PM_CUDA_TRY(cudaGetLastError());
+        s->launch_total += 2;
+        return PM_OK;
+    }
+};
+
 struct HelmSolver {
     pm_surface* s;
     PmHelmWork& W;
     cudaStream_t st;
     int grid;
+    HelmDense D;
+
+    // out = M v (+ v when add) from a dense matrix
+    pm_status dense(const double2* M, const double2* v, int add, double2* out) {
+        PhaseTimer t(s, PM_PHASE_NEAR, st);
+        k_dense_c64<<<pm_ceil_div(W.N, kGemvRowsC), kHT, 0, st>>>(M, v, add, W.N, out);
+        PM_CUDA_TRY(cudaGetLastError());
+        s->launch_total++;
+        return PM_OK;
+    }
 
     // dst[0..ncols) = V_j^H b on the device
     pm_status dots(const double2* V, long long ldv, int ncols, const double2* b, double2* dst) {
@@ -354,6 +494,7 @@ struct HelmSolver {
 
     // out = (I + R~) v
     pm_status apply_A(const double2* v, double2* out) {
+        if (D.MR) return dense(D.MR, v, 1, out);
         PM_TRY(helm_apply(s, 0, v, W.tmp, st));
         k_cadd<<<grid, kRT, 0, st>>>(v, 1.0, W.tmp, 1.0, out, W.N);
         PM_CUDA_TRY(cudaGetLastError());
@@ -472,7 +613,7 @@ extern "C" pm_status pm_solve_c(pm_surface* s, const double* f, double* u, doubl
     PmHelmWork& W = *Wp;
     const int N = s->N;
     cudaStream_t st = 0;
-    HelmSolver S{s, W, st, pm_ceil_div(N, kRT)};
+    HelmSolver S{s, W, st, pm_ceil_div(N, kRT), {}};
     const size_t bytes = sizeof(double2) * N;
     PM_CUDA_TRY(cudaMemcpyAsync(W.f, f, bytes, cudaMemcpyHostToDevice, st));
     PM_CUDA_TRY(cudaMemsetAsync(W.x, 0, bytes, st));
@@ -482,6 +623,7 @@ extern "C" pm_status pm_solve_c(pm_surface* s, const double* f, double* u, doubl
     double relres = 0.0;
     pm_status result = PM_OK;
     if (fnorm > 0.0) {
+        PM_TRY(S.D.fill(s));
         PM_CUDA_TRY(cudaMemcpyAsync(W.r, W.f, bytes, cudaMemcpyDeviceToDevice, st));
         std::vector<cplx> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
         const long long ldv = N;
@@ -571,7 +713,8 @@ extern "C" pm_status pm_solve_c(pm_surface* s, const double* f, double* u, doubl
         }
     }
     // u = K~ sigma (eq. representation; no projection for c != 0)
-    PM_TRY(helm_apply(s, 1, W.x, W.u, st));
+    if (S.D.MR) PM_TRY(S.dense(S.D.MK, W.x, 0, W.u));
+    else PM_TRY(helm_apply(s, 1, W.x, W.u, st));
     PM_CUDA_TRY(cudaMemcpyAsync(u, W.u, bytes, cudaMemcpyDeviceToHost, st));
     if (sigma_out) PM_CUDA_TRY(cudaMemcpyAsync(sigma_out, W.x, bytes, cudaMemcpyDeviceToHost, st));
     PM_CUDA_TRY(cudaStreamSynchronize(st));
