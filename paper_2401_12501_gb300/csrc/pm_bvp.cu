@@ -40,7 +40,8 @@
 // * K'_Gamma: the smooth rule over all surface nodes plus corrections on the patches near
 //   each edge node (pm_nearfield.cu k_bvp_kp_quad: polar rule about the edge point on its
 //   own patch, the quadtree near rule on the others).
-// Everything runs in float64; the solver is restarted GMRES with classical Gram-Schmidt
+// Everything runs in float64; a solve applies the system through its dense matrix where
+// that fits the device (else pair by pair); the solver is restarted GMRES with classical Gram-Schmidt
 // and one reorthogonalisation, the Hessenberg system on the host.
 #include "pm_internal.cuh"
 
@@ -66,7 +67,7 @@ struct pm_bvp {
     int *interp_off = nullptr;           // [ncurves + 1] offsets into interp
     int *curve_of = nullptr;             // [Fo] curve of an oversampled point
     double *Kpg = nullptr;               // [Me][Me] K'_gamma (Neumann) or N_gamma (Dirichlet), weighted
-    int *kp_ptr = nullptr, *kp_patch = nullptr;
+    int *kp_ptr = nullptr, *kp_patch = nullptr, *kp_edge = nullptr;
     double *kp_C = nullptr;              // [nblk][pp] K'_Gamma (K_Gamma) corrections
     int kp_nblk = 0;
     double *mu_o = nullptr;              // [Fo]
@@ -101,6 +102,54 @@ __global__ void k_bvp_interp(const double* __restrict__ I, const int* __restrict
 // nu' . grad' R for constant a (the a's cancel), 3 the double layer
 // -nu' . r / (2 pi a r^2)
 enum { kEdgeR = 0, kEdgeK = 1, kEdgeT = 2, kEdgeN = 3 };
+
+// a target's data (n, H, a and g for the remainder kinds only)
+struct EdgeTarget {
+    double x[3], n[3], g[3], H, a;
+};
+
+template <int KIND>
+__device__ __forceinline__ EdgeTarget edge_target(int i, const double* x, const double* n,
+                                                  const double* H, const double* a, const double* g) {
+    EdgeTarget t{};
+    for (int d = 0; d < 3; ++d) t.x[d] = x[3 * i + d];
+    if (KIND == kEdgeR || KIND == kEdgeT) {
+        for (int d = 0; d < 3; ++d) {
+            t.n[d] = n[3 * i + d];
+            t.g[d] = g[3 * i + d];
+        }
+        t.H = H[i];
+        t.a = a[i];
+    }
+    return t;
+}
+
+// the kernel of one (target, oversampled point y with binormal u) pair, all its constants in
+// (R and K without 1 / a(x'), which the strength carries)
+template <int KIND>
+__device__ __forceinline__ double edge_pair(const EdgeTarget& t, double y0, double y1, double y2,
+                                            double u0, double u1, double u2) {
+    const double r0 = t.x[0] - y0, r1 = t.x[1] - y1, r2 = t.x[2] - y2;
+    const double rr = r0 * r0 + r1 * r1 + r2 * r2;
+    if (KIND == kEdgeK) return log(rr) * (0.25 / M_PI);
+    const double inv = 1.0 / rr;
+    if (KIND == kEdgeN) return -(u0 * r0 + u1 * r1 + u2 * r2) * inv * (0.5 / M_PI);
+    const double nr = t.n[0] * r0 + t.n[1] * r1 + t.n[2] * r2;
+    if (KIND == kEdgeR) {
+        const double qn = nr * inv;
+        return t.a * (qn * qn - t.H * qn) * (1.0 / M_PI) +
+               (t.g[0] * r0 + t.g[1] * r1 + t.g[2] * r2) * inv * (0.5 / M_PI);
+    }
+    // -(1/pi) [2 (n.r)(n.nu')/r^4 - 4 (n.r)^2 (r.nu')/r^6 - H (n.nu')/r^2
+    //          + 2 H (n.r)(r.nu')/r^4]
+    const double nnu = t.n[0] * u0 + t.n[1] * u1 + t.n[2] * u2;
+    const double rnu = r0 * u0 + r1 * u1 + r2 * u2;
+    return -(1.0 / M_PI) * inv * (2.0 * nr * nnu * inv - 4.0 * nr * nr * rnu * inv * inv -
+                                  t.H * nnu + 2.0 * t.H * nr * rnu * inv);
+}
+
+// A warp a target, its lanes over the oversampled points: float64-pipe work, for which a
+// thread a target left most SMs without any (9.6 ms for 2,048 targets x 4,096 points).
 template <int KIND>
 __global__ void __launch_bounds__(kT)
 k_bvp_edge_to_surface(int N, const double* __restrict__ x, const double* __restrict__ n,
@@ -109,66 +158,154 @@ k_bvp_edge_to_surface(int N, const double* __restrict__ x, const double* __restr
                       const double* __restrict__ wo, const double* __restrict__ ao,
                       const double* __restrict__ nuo, const double* __restrict__ mu_o,
                       double* __restrict__ out) {
-    constexpr bool WHICH_K = KIND == kEdgeK || KIND == kEdgeN;
-    __shared__ double sx[kTile], sy[kTile], sz[kTile], ss[kTile];
-    __shared__ double su[KIND >= kEdgeT ? kTile : 1], sv[KIND >= kEdgeT ? kTile : 1],
-        sw[KIND >= kEdgeT ? kTile : 1];
-    const int i = blockIdx.x * kT + threadIdx.x;
-    double xi0 = 0, xi1 = 0, xi2 = 0, n0 = 0, n1 = 0, n2 = 0, Hi = 0, ai = 0, g0 = 0, g1 = 0, g2 = 0;
-    if (i < N) {
-        xi0 = x[3 * i]; xi1 = x[3 * i + 1]; xi2 = x[3 * i + 2];
-        if (KIND == kEdgeR || KIND == kEdgeT) {
-            n0 = n[3 * i]; n1 = n[3 * i + 1]; n2 = n[3 * i + 2];
-            Hi = H[i]; ai = a[i];
-            g0 = g[3 * i]; g1 = g[3 * i + 1]; g2 = g[3 * i + 2];
-        }
-    }
+    const int i = (blockIdx.x * kT + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (i >= N) return;
+    const EdgeTarget t = edge_target<KIND>(i, x, n, H, a, g);
     double acc = 0.0;
-    for (int base = 0; base < Fo; base += kTile) {
-        __syncthreads();
+    for (int j = lane; j < Fo; j += 32) {
+        const double s = KIND == kEdgeT ? wo[j] * mu_o[j] : wo[j] * mu_o[j] / ao[j];
+        acc += s * edge_pair<KIND>(t, xo[3 * j], xo[3 * j + 1], xo[3 * j + 2], nuo[3 * j],
+                                   nuo[3 * j + 1], nuo[3 * j + 2]);
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if (lane == 0) out[i] += acc;
+}
+
+// ------------------------------------------------------------------ the dense system
+// A solve forms the system's matrix once, A [n][n] over z = [sigma; mu] (n = N + Me), and
+// its Krylov steps stream it: 8 n^2 bytes a step instead of the float64 pair sums of
+// apply_sys.  Dirichlet, 2,048 nodes and 128 edge nodes (a matrix of 38 MB, so it stays in
+// L2): a solve of 15 steps 176 -> 4.7 ms.
+
+// surface rows, sigma columns: delta_ij + w_j R(x_i, x_j) / a_j (kDI targets x kDJ sources a block)
+constexpr int kDI = 32, kDJ = 128;
+__global__ void __launch_bounds__(kDJ)
+k_bvp_fill_surface(int N, const double* __restrict__ x, const double* __restrict__ nrm,
+                   const double* __restrict__ H, const double* __restrict__ a,
+                   const double* __restrict__ g, const double* __restrict__ wa, int ld,
+                   double* __restrict__ A) {
+    __shared__ double st[kDI][9];        // x, sqrt(a/pi) n, -(a H/pi) n + grad a/(2 pi)
+    const int i0 = blockIdx.y * kDI, rows = min(kDI, N - i0);
+    for (int e = threadIdx.x; e < rows * 3; e += kDJ) {
+        const int r = e / 3, d = e - r * 3, i = i0 + r;
+        st[r][d] = x[3 * i + d];
+        st[r][3 + d] = sqrt(a[i] / M_PI) * nrm[3 * i + d];
+        st[r][6 + d] = -a[i] * H[i] / M_PI * nrm[3 * i + d] + 0.5 / M_PI * g[3 * i + d];
+    }
+    __syncthreads();
+    const int j = blockIdx.x * kDJ + threadIdx.x;
+    if (j >= N) return;
+    const double y0 = x[3 * j], y1 = x[3 * j + 1], y2 = x[3 * j + 2], w = wa[j];
+    for (int r = 0; r < rows; ++r) {
+        const double* t = st[r];
+        const double r0 = t[0] - y0, r1 = t[1] - y1, r2 = t[2] - y2;
+        const double inv = 1.0 / (r0 * r0 + r1 * r1 + r2 * r2);
+        const double nr = t[3] * r0 + t[4] * r1 + t[5] * r2;
+        const double mr = t[6] * r0 + t[7] * r1 + t[8] * r2;
+        A[(size_t)(i0 + r) * ld + j] = i0 + r == j ? 1.0 : w * inv * (nr * nr * inv + mr);
+    }
+}
+
+// corrections of surface rows (row_of = blk_row) or edge rows (the edge node of each block)
+__global__ void k_bvp_fill_near(int nblk, int pp, const int* __restrict__ row_of, int row0,
+                                const int* __restrict__ blk_patch, const double* __restrict__ C,
+                                int ld, double* __restrict__ A) {
+    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= (size_t)nblk * pp) return;
+    const int b = (int)(e / pp), k = (int)(e - (size_t)b * pp);
+    A[(size_t)(row0 + row_of[b]) * ld + (size_t)blk_patch[b] * pp + k] += C[e];
+}
+
+// surface rows, mu columns: sum over curve c's oversampled points of the pair kernel times the
+// interpolation row.  Block: kEI targets x 128 edge nodes of one curve; the points pass in
+// tiles of 128, a thread evaluating its point for every target, then its edge node's sums.
+constexpr int kEI = 4;
+template <int KIND>
+__global__ void __launch_bounds__(128)
+k_bvp_fill_edge_columns(int N, const double* __restrict__ x, const double* __restrict__ n,
+                        const double* __restrict__ H, const double* __restrict__ a,
+                        const double* __restrict__ g, int ncurves, const double* __restrict__ xo,
+                        const double* __restrict__ wo, const double* __restrict__ ao,
+                        const double* __restrict__ nuo, const double* __restrict__ I,
+                        const int* __restrict__ ioff, int ld, double* __restrict__ A) {
+    __shared__ double sk[kEI][128];
+    const int c = blockIdx.y, nc1 = ncurves + 1;
+    const int o0 = ioff[nc1 + c], o1 = ioff[nc1 + c + 1], off = ioff[2 * nc1 + c], M = ioff[3 * nc1 + c];
+    const int e = blockIdx.z * 128 + threadIdx.x;
+    if (blockIdx.z * 128 >= M) return;
+    const int i0 = blockIdx.x * kEI;
+    EdgeTarget t[kEI];
+    for (int r = 0; r < kEI; ++r) t[r] = edge_target<KIND>(min(i0 + r, N - 1), x, n, H, a, g);
+    double acc[kEI] = {};
+    for (int base = o0; base < o1; base += 128) {
         const int j = base + threadIdx.x;
-        if (j < Fo) {
-            sx[threadIdx.x] = xo[3 * j];
-            sy[threadIdx.x] = xo[3 * j + 1];
-            sz[threadIdx.x] = xo[3 * j + 2];
-            ss[threadIdx.x] = KIND == kEdgeT ? wo[j] * mu_o[j] : wo[j] * mu_o[j] / ao[j];
-            if (KIND >= kEdgeT) {
-                su[threadIdx.x] = nuo[3 * j];
-                sv[threadIdx.x] = nuo[3 * j + 1];
-                sw[threadIdx.x] = nuo[3 * j + 2];
+        if (j < o1) {
+            const double w = KIND == kEdgeT ? wo[j] : wo[j] / ao[j];
+            for (int r = 0; r < kEI; ++r)
+                sk[r][threadIdx.x] = w * edge_pair<KIND>(t[r], xo[3 * j], xo[3 * j + 1], xo[3 * j + 2],
+                                                         nuo[3 * j], nuo[3 * j + 1], nuo[3 * j + 2]);
+        }
+        __syncthreads();
+        if (e < M) {
+            const double* row = I + ioff[c] + (size_t)(base - o0) * M + e;
+            const int cnt = min(128, o1 - base);
+            for (int q = 0; q < cnt; ++q) {
+                const double v = row[(size_t)q * M];
+                for (int r = 0; r < kEI; ++r) acc[r] = fma(v, sk[r][q], acc[r]);
             }
         }
         __syncthreads();
-        const int cnt = min(kTile, Fo - base);
-        if (i < N)
-            for (int q = 0; q < cnt; ++q) {
-                const double r0 = xi0 - sx[q], r1 = xi1 - sy[q], r2 = xi2 - sz[q];
-                const double rr = r0 * r0 + r1 * r1 + r2 * r2;
-                if (KIND == kEdgeK) {
-                    acc += ss[q] * log(rr);
-                } else if (KIND == kEdgeR) {
-                    const double inv = 1.0 / rr;
-                    const double qn = (n0 * r0 + n1 * r1 + n2 * r2) * inv;
-                    acc += ss[q] * (ai * (qn * qn - Hi * qn) * (1.0 / M_PI) +
-                                    (g0 * r0 + g1 * r1 + g2 * r2) * inv * (0.5 / M_PI));
-                } else if (KIND == kEdgeN) {
-                    acc -= ss[q] * (su[q] * r0 + sv[q] * r1 + sw[q] * r2) / rr;
-                } else {
-                    // -(1/pi) [2 (n.r)(n.nu')/r^4 - 4 (n.r)^2 (r.nu')/r^6 - H (n.nu')/r^2
-                    //          + 2 H (n.r)(r.nu')/r^4]
-                    const double inv = 1.0 / rr;
-                    const double nr = n0 * r0 + n1 * r1 + n2 * r2;
-                    const double nnu = n0 * su[q] + n1 * sv[q] + n2 * sw[q];
-                    const double rnu = r0 * su[q] + r1 * sv[q] + r2 * sw[q];
-                    acc -= ss[q] * inv * (2.0 * nr * nnu * inv - 4.0 * nr * nr * rnu * inv * inv -
-                                          Hi * nnu + 2.0 * Hi * nr * rnu * inv);
-                }
-            }
     }
-    if (i < N)
-        out[i] += KIND == kEdgeK ? acc * (0.25 / M_PI)
-                  : KIND == kEdgeN ? acc * (0.5 / M_PI)
-                  : KIND == kEdgeT ? acc * (1.0 / M_PI) : acc;
+    if (e < M)
+        for (int r = 0; r < kEI && i0 + r < N; ++r) A[(size_t)(i0 + r) * ld + N + off + e] = acc[r];
+}
+
+// edge rows (as k_bvp_edge_row, without the corrections)
+__global__ void k_bvp_fill_edge_rows(int dirichlet, int N, int Me, const double* __restrict__ x,
+                                     const double* __restrict__ wa, const double* __restrict__ xe,
+                                     const double* __restrict__ nue, const double* __restrict__ ae,
+                                     const double* __restrict__ we, const double* __restrict__ Kpg,
+                                     int ld, double* __restrict__ A) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x, e = blockIdx.y;
+    if (j >= N + Me) return;
+    double v;
+    if (j < N) {
+        const double r0 = xe[3 * e] - x[3 * j], r1 = xe[3 * e + 1] - x[3 * j + 1],
+                     r2 = xe[3 * e + 2] - x[3 * j + 2];
+        const double rr = r0 * r0 + r1 * r1 + r2 * r2;
+        v = wa[j] * (0.5 / M_PI) *
+            (dirichlet ? 0.5 * log(rr)
+                       : (nue[3 * e] * r0 + nue[3 * e + 1] * r1 + nue[3 * e + 2] * r2) / rr);
+    } else {
+        const int k = j - N;
+        v = Kpg[(size_t)e * Me + k] + (dirichlet ? 0.0 : we[k]);
+        if (k == e) v += (dirichlet ? 0.5 : -0.5) / ae[e];
+    }
+    A[(size_t)(N + e) * ld + j] = v;
+}
+
+// out = A z, four rows a block
+__global__ void __launch_bounds__(128)
+k_bvp_gemv(int n, const double* __restrict__ A, const double* __restrict__ z, double* __restrict__ out) {
+    __shared__ double sh[4][4];
+    const int i0 = blockIdx.x * 4;
+    const double* row[4];
+    double acc[4] = {};
+    for (int r = 0; r < 4; ++r) row[r] = A + (size_t)min(i0 + r, n - 1) * n;
+#pragma unroll 4
+    for (int j = threadIdx.x; j < n; j += 128) {
+        const double v = z[j];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[r] = fma(row[r][j], v, acc[r]);
+    }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int r = 0; r < 4; ++r) {
+        for (int o = 16; o > 0; o >>= 1) acc[r] += __shfl_down_sync(0xffffffffu, acc[r], o);
+        if (lane == 0) sh[r][wid] = acc[r];
+    }
+    __syncthreads();
+    const int r = threadIdx.x;
+    if (r < 4 && i0 + r < n) out[i0 + r] = (sh[r][0] + sh[r][1]) + (sh[r][2] + sh[r][3]);
 }
 
 __device__ double block_sum(double v, double* red) {
@@ -294,15 +431,48 @@ pm_status apply_sys(pm_bvp* b, const double* z, double* out) {
             b->interp_off + 2 * (b->ncurves + 1), b->interp_off + 3 * (b->ncurves + 1), z + N,
             b->mu_o, b->Fo);
         if (b->kind)
-            k_bvp_edge_to_surface<kEdgeT><<<pm_ceil_div(N, kT), kT, 0, st>>>(
+            k_bvp_edge_to_surface<kEdgeT><<<pm_ceil_div((long long)N * 32, kT), kT, 0, st>>>(
                 N, s->x, s->n, s->H, s->a, s->g, b->Fo, b->xo, b->wo, b->ao, b->nuo, b->mu_o, out);
         else
-            k_bvp_edge_to_surface<kEdgeR><<<pm_ceil_div(N, kT), kT, 0, st>>>(
+            k_bvp_edge_to_surface<kEdgeR><<<pm_ceil_div((long long)N * 32, kT), kT, 0, st>>>(
                 N, s->x, s->n, s->H, s->a, s->g, b->Fo, b->xo, b->wo, b->ao, b->nuo, b->mu_o, out);
         k_bvp_edge_row<<<b->Me, kT, 0, st>>>(b->kind, N, b->Me, s->pp, s->x, s->wa, b->xe, b->nue, b->ae,
                                              b->we, b->kp_ptr, b->kp_patch, b->kp_C, b->Kpg, z,
                                              z + N, out + N);
     }
+    PM_CUDA_TRY(cudaGetLastError());
+    return PM_OK;
+}
+
+// The system's matrix into A [n][n] (device).
+pm_status fill_sys(pm_bvp* b, double* A) {
+    pm_surface* s = b->s;
+    const int N = b->N, Me = b->Me, ld = N + Me;
+    cudaStream_t st = b->st;
+    k_bvp_fill_surface<<<dim3(pm_ceil_div(N, kDJ), pm_ceil_div(N, kDI)), kDJ, 0, st>>>(
+        N, s->x, s->n, s->H, s->a, s->g, s->wa, ld, A);
+    k_bvp_fill_near<<<pm_ceil_div((long long)s->nblk * s->pp, kT), kT, 0, st>>>(
+        s->nblk, s->pp, s->blk_row, 0, s->blk_patch, s->cR64, ld, A);
+    if (Me > 0) {
+        const int mmax = *std::max_element(b->M.begin(), b->M.end());
+        dim3 grid(pm_ceil_div(N, kEI), b->ncurves, pm_ceil_div(mmax, 128));
+        (b->kind ? k_bvp_fill_edge_columns<kEdgeT> : k_bvp_fill_edge_columns<kEdgeR>)
+            <<<grid, 128, 0, st>>>(N, s->x, s->n, s->H, s->a, s->g, b->ncurves, b->xo, b->wo, b->ao,
+                                   b->nuo, b->interp, b->interp_off, ld, A);
+        k_bvp_fill_edge_rows<<<dim3(pm_ceil_div(ld, kT), Me), kT, 0, st>>>(
+            b->kind, N, Me, s->x, s->wa, b->xe, b->nue, b->ae, b->we, b->Kpg, ld, A);
+        k_bvp_fill_near<<<pm_ceil_div((long long)b->kp_nblk * s->pp, kT), kT, 0, st>>>(
+            b->kp_nblk, s->pp, b->kp_edge, N, b->kp_patch, b->kp_C, ld, A);
+    }
+    PM_CUDA_TRY(cudaGetLastError());
+    return PM_OK;
+}
+
+// the operator through its matrix where the solve holds one
+pm_status apply_any(pm_bvp* b, const double* A, const double* z, double* out) {
+    if (!A) return apply_sys(b, z, out);
+    const int n = b->N + b->Me;
+    k_bvp_gemv<<<pm_ceil_div(n, 4), 128, 0, b->st>>>(n, A, z, out);
     PM_CUDA_TRY(cudaGetLastError());
     return PM_OK;
 }
@@ -318,10 +488,10 @@ pm_status represent(pm_bvp* b, const double* z, double* u) {
             b->interp_off + 2 * (b->ncurves + 1), b->interp_off + 3 * (b->ncurves + 1), z + N,
             b->mu_o, b->Fo);
         if (b->kind)
-            k_bvp_edge_to_surface<kEdgeN><<<pm_ceil_div(N, kT), kT, 0, st>>>(
+            k_bvp_edge_to_surface<kEdgeN><<<pm_ceil_div((long long)N * 32, kT), kT, 0, st>>>(
                 N, s->x, s->n, s->H, s->a, s->g, b->Fo, b->xo, b->wo, b->ao, b->nuo, b->mu_o, u);
         else
-            k_bvp_edge_to_surface<kEdgeK><<<pm_ceil_div(N, kT), kT, 0, st>>>(
+            k_bvp_edge_to_surface<kEdgeK><<<pm_ceil_div((long long)N * 32, kT), kT, 0, st>>>(
                 N, s->x, s->n, s->H, s->a, s->g, b->Fo, b->xo, b->wo, b->ao, b->nuo, b->mu_o, u);
     }
     PM_CUDA_TRY(cudaGetLastError());
@@ -335,7 +505,7 @@ void free_bvp(pm_bvp* b) {
     pm_dfree(b->xo); pm_dfree(b->wo); pm_dfree(b->ao); pm_dfree(b->nuo); pm_dfree(b->interp);
     pm_dfree(b->interp_off);
     pm_dfree(b->curve_of); pm_dfree(b->Kpg); pm_dfree(b->kp_ptr); pm_dfree(b->kp_patch);
-    pm_dfree(b->kp_C); pm_dfree(b->mu_o); pm_dfree(b->part);
+    pm_dfree(b->kp_C); pm_dfree(b->kp_edge); pm_dfree(b->mu_o); pm_dfree(b->part);
     delete b;
 }
 
@@ -432,7 +602,7 @@ pm_status create_impl(pm_bvp* b, const double* edge_x, const double* edge_d1,
         kp_ptr[e + 1] = (int)kp_patch.size();
     }
     b->kp_nblk = (int)kp_patch.size();
-    int *d_be = nullptr, *d_own = nullptr;
+    int* d_own = nullptr;
     PM_TRY(upload(&b->xe, edge_x, 3 * (size_t)Me));
     PM_TRY(upload(&b->nue, edge_nu, 3 * (size_t)Me));
     PM_TRY(upload(&b->we, b->h_we.data(), (size_t)Me));
@@ -451,20 +621,19 @@ pm_status create_impl(pm_bvp* b, const double* edge_x, const double* edge_d1,
     PM_TRY(pm_dmalloc(&b->kp_C, (size_t)b->kp_nblk * pp));
     PM_TRY(pm_dmalloc(&b->mu_o, (size_t)std::max(Fo, 1)));
     PM_TRY(pm_dmalloc(&b->part, (size_t)kDotBlocks * 128));
-    pm_status stt = upload(&d_be, blk_edge.data(), blk_edge.size());
+    pm_status stt = upload(&b->kp_edge, blk_edge.data(), blk_edge.size());
     if (stt == PM_OK) stt = upload(&d_own, blk_own.data(), blk_own.size());
     if (stt == PM_OK)
-        stt = pm_bvp_kp_weights(s, b->kp_nblk, d_be, b->kp_patch, d_own, b->xe, b->nue, b->uv,
+        stt = pm_bvp_kp_weights(s, b->kp_nblk, b->kp_edge, b->kp_patch, d_own, b->xe, b->nue, b->uv,
                                 b->kind, b->kp_C);
     if (stt == PM_OK && b->kp_nblk > 0) {
         k_bvp_combine<<<pm_ceil_div((long long)b->kp_nblk * pp, kT), kT>>>(
-            b->kind, b->kp_nblk, pp, d_be, b->kp_patch, s->x, s->a, s->w, b->xe, b->nue, b->kp_C);
+            b->kind, b->kp_nblk, pp, b->kp_edge, b->kp_patch, s->x, s->a, s->w, b->xe, b->nue, b->kp_C);
         if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
             pm_set_error("pm_bvp_create: correction kernel failed");
             stt = PM_ERR_CUDA;
         }
     }
-    pm_dfree(d_be);
     pm_dfree(d_own);
     return stt;
 }
@@ -620,6 +789,7 @@ extern "C" pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_ga
     const int n = b->N + b->Me;
     const int m = std::max(2, std::min(b->s->opts.gmres_restart, 120));
     double *V = nullptr, *w = nullptr, *rhs = nullptr, *x = nullptr, *hd = nullptr, *ud = nullptr;
+    double* A = nullptr;                 // the system's matrix, where the device has room for it
     pm_status st = pm_dmalloc(&V, (size_t)(m + 1) * n);
     if (st == PM_OK) st = pm_dmalloc(&w, (size_t)n);
     if (st == PM_OK) st = pm_dmalloc(&rhs, (size_t)n);
@@ -628,6 +798,7 @@ extern "C" pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_ga
     if (st == PM_OK) st = pm_dmalloc(&ud, (size_t)b->N);
     auto cleanup = [&]() {
         pm_dfree(V); pm_dfree(w); pm_dfree(rhs); pm_dfree(x); pm_dfree(hd); pm_dfree(ud);
+        if (A) cudaFreeAsync(A, b->st);
     };
     if (st != PM_OK) { cleanup(); return st; }
     const auto t0 = std::chrono::steady_clock::now();
@@ -650,9 +821,19 @@ extern "C" pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_ga
     int iters = 0;
     double relres = bnorm > 0 ? 1.0 : 0.0;
     std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
+    if (bnorm > 0) {
+        size_t fr = 0, total = 0;
+        const size_t need = sizeof(double) * (size_t)n * n;
+        if (cudaMemGetInfo(&fr, &total) == cudaSuccess &&
+            need + std::max<size_t>(1ull << 30, total / 50) <= pm_free_hbm_bytes() &&
+            cudaMallocAsync((void**)&A, need, b->st) != cudaSuccess)
+            A = nullptr;
+        cudaGetLastError();
+        if (A && (st = fill_sys(b, A)) != PM_OK) { cleanup(); return st; }
+    }
     while (st == PM_OK && bnorm > 0 && relres > tol && iters < maxit) {
         // r = b - A x
-        st = apply_sys(b, x, w);
+        st = apply_any(b, A, x, w);
         if (st != PM_OK) break;
         k_bvp_scale<<<grid, kT, 0, b->st>>>(n, -1.0, w, w);
         k_bvp_axpy<<<grid, kT, 0, b->st>>>(n, 1.0, rhs, w);
@@ -666,7 +847,7 @@ extern "C" pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_ga
         int k = 0;
         for (; k < m && iters < maxit; ++k, ++iters) {
             double* vk1 = V + (size_t)(k + 1) * n;
-            if ((st = apply_sys(b, V + (size_t)k * n, vk1)) != PM_OK) break;
+            if ((st = apply_any(b, A, V + (size_t)k * n, vk1)) != PM_OK) break;
             // classical Gram-Schmidt with one reorthogonalisation
             std::vector<double> h(k + 1, 0.0);
             for (int pass = 0; pass < 2 && st == PM_OK; ++pass) {
@@ -708,7 +889,7 @@ extern "C" pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_ga
         for (int j = 0; j < k; ++j) k_bvp_axpy<<<grid, kT, 0, b->st>>>(n, y[j], V + (size_t)j * n, x);
         if (relres <= tol) {
             // the true residual confirms the estimate
-            if ((st = apply_sys(b, x, w)) != PM_OK) break;
+            if ((st = apply_any(b, A, x, w)) != PM_OK) break;
             k_bvp_scale<<<grid, kT, 0, b->st>>>(n, -1.0, w, w);
             k_bvp_axpy<<<grid, kT, 0, b->st>>>(n, 1.0, rhs, w);
             if ((st = dots(b, w, 1, w, n, d)) != PM_OK) break;

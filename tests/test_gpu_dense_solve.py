@@ -1,0 +1,80 @@
+"""Solves of the c != 0 and open-surface systems form a dense matrix where the device has room
+for it, and go pair by pair where it has not (PM_FAKE_HBM_BYTES = 0): both give the same
+solution.  Each stops at a relative residual of 1e-12, so with the operators' inverses below
+about 10 in norm the two agree to 1e-10 with room to spare."""
+
+import numpy as np
+import pytest
+
+from workloads import cubed_sphere
+from workloads import bvp as bands
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-10
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2401_12501_gb300 as pm
+    c = pm.Context(0)
+    yield c
+    c.close()
+
+
+def both(monkeypatch, solve):
+    dense = solve()
+    monkeypatch.setenv("PM_FAKE_HBM_BYTES", "0")
+    pairs = solve()
+    monkeypatch.delenv("PM_FAKE_HBM_BYTES")
+    for d, p in zip(dense, pairs):
+        assert np.abs(d - p).max() <= TOL * np.abs(p).max()
+
+
+# 54 to 600 nodes: less than a block's rows and sources, one more, and a remainder of both
+@pytest.mark.parametrize("m,p,kind", [(1, 3, "real"), (1, 5, "negative"), (1, 5, "complex"),
+                                      (1, 7, "mixed"), (2, 5, "real")])
+def test_wave_solve(ctx, monkeypatch, m, p, kind):
+    import paper_2401_12501_gb300 as pm
+    s = cubed_sphere(m, p, axes=(1.0, 1.5, 2.0))
+    x = s.nodes
+    c = {"real": 4.0 + x[:, 1], "negative": -4.0 - x[:, 0] ** 2, "complex": 4.0 + 1j * x[:, 2],
+         "mixed": np.where(x[:, 2] > 0, 3.0, 2.0 + 0.5j)}[kind]
+    S = pm.Surface.from_fixture(ctx, s)
+    S.set_coeff_c(1.0 + 0.2 * x[:, 2] ** 2, None, c)
+    f = np.cos(x[:, 0]) + 1j * x[:, 1]
+
+    def solve():
+        u, _, sigma = S.solve_c(f, tol=1e-12, return_sigma=True)
+        return u, sigma
+
+    both(monkeypatch, solve)
+    S.close()
+
+
+@pytest.mark.parametrize("kind,n,p,M", [("neumann", 4, 5, 12), ("dirichlet", 4, 6, 36),
+                                        ("dirichlet", 3, 7, 135), ("neumann", 3, 6, 129)])
+def test_edge_solve(ctx, monkeypatch, kind, n, p, M):
+    import paper_2401_12501_gb300 as pm
+    F = 4
+    band = bands.torus_band(2, n, p, M, F)
+    co = (bands.band_coefficient(band) if kind == "neumann" else bands.constant_band_coefficient(band))
+    S = pm.Surface.from_fixture(ctx, band.surface)
+    S.set_coeff(co.a, co.grad_a)
+    patch, uv = bands.edge_patches(band)
+    ae, ao = ((bands.edge_a(band), bands.edge_a(band, True)) if kind == "neumann"
+              else (np.ones(band.M), np.ones(F * band.M)))
+    b = pm.BoundaryValueProblem(S, band.curves, ae, ao, patch, uv, kind=kind)
+    rng = np.random.default_rng(5)
+    sigma, mu = rng.standard_normal(S.N), rng.standard_normal(b.Me)
+    f, fg = b.apply(sigma, mu)          # consistent data: the solution is (sigma, mu)
+
+    def solve():
+        u, _, s, m = b.solve(f, fg, tol=1e-12)
+        return s, m
+
+    both(monkeypatch, solve)
+    b.close()
+    S.close()
