@@ -26,8 +26,11 @@
 // target lies within 2*eta*(corner radius) of its centre image, 16 x 16 Gauss
 // rule on each leaf (a geometric a-priori criterion standing in for the
 // adaptive error test of Sec. 6.1.2).
+// Both rules' points depend on the reference square alone, so the weights are sums over
+// tabulated basis values (pm_quadmm.cu); this file fills the tables and finds the leaves.
 #include "pm_green.cuh"
 #include "pm_internal.cuh"
+#include "pm_quadmm.cuh"
 
 #include <algorithm>
 #include <cstring>
@@ -162,126 +165,8 @@ __global__ void k_near_fill(const double* __restrict__ x, const double* __restri
         }
 }
 
-// ------------------------------------------------------------------ self quadrature
-// One block per target; shared memory (doubles): D [3*pp], Jn [pp],
-// lu [128*p], lv [128*p], f [5*128].
-__global__ void __launch_bounds__(kQThreads)
-k_self_quad(int N, int p, const double* __restrict__ x, const double* __restrict__ J,
-            const double* __restrict__ nn, const double* __restrict__ H,
-            const int* __restrict__ th_off, const double* __restrict__ th_ang,
-            const double* __restrict__ th_w, const double* __restrict__ th_L,
-            const int* __restrict__ row_ptr, int nblk, double* __restrict__ W_lb,
-            double* __restrict__ W_g, double* __restrict__ W_k) {
-    extern __shared__ double sm[];
-    const int pp = p * p;
-    double* sD = sm;                       // [3][pp]
-    double* sJ = sD + 3 * pp;              // [pp]
-    double* sLu = sJ + pp;                 // [128][p]
-    double* sLv = sLu + kQThreads * p;     // [128][p]
-    double* sF = sLv + kQThreads * p;      // [5][128]
-    const int i = blockIdx.x;
-    const int tid = threadIdx.x;
-    const int P = i / pp, loc = i - P * pp;
-    const double u0 = cT.t[loc / p], v0 = cT.t[loc % p];
-    const double xi0 = x[3 * i], xi1 = x[3 * i + 1], xi2 = x[3 * i + 2];
-    for (int k = tid; k < pp; k += kQThreads) {
-        const size_t gk = (size_t)P * pp + k;
-        sD[k] = x[3 * gk] - xi0;
-        sD[pp + k] = x[3 * gk + 1] - xi1;
-        sD[2 * pp + k] = x[3 * gk + 2] - xi2;
-        sJ[k] = J[gk];
-    }
-    const double n0 = nn[3 * i], n1 = nn[3 * i + 1], n2 = nn[3 * i + 2];
-    const double Hi = H[i];
-    const int t0 = th_off[loc], t1 = th_off[loc + 1];
-    const int npts = (t1 - t0) * (PM_RADIAL_PANELS * PM_GL16);
-    const double lo_f[4] = {0.0, 0.125, 0.25, 0.5};
-    const double hi_f[4] = {0.125, 0.25, 0.5, 1.0};
-    double acc_lb = 0, acc_g0 = 0, acc_g1 = 0, acc_g2 = 0, acc_k = 0;
-    const int a_own = tid / p, b_own = tid - (tid / p) * p;
-    __syncthreads();
-    for (int base = 0; base < npts; base += kQThreads) {
-        const int q = base + tid;
-        double* lu = sLu + tid * p;
-        double* lv = sLv + tid * p;
-        double f_lb = 0, f_g0 = 0, f_g1 = 0, f_g2 = 0, f_k = 0;
-        if (q < npts) {
-            const int kth = t0 + q / (PM_RADIAL_PANELS * PM_GL16);
-            const int rj = q % (PM_RADIAL_PANELS * PM_GL16);
-            const int panel = rj / PM_GL16, node = rj % PM_GL16;
-            const double L = th_L[kth];
-            const double h = (hi_f[panel] - lo_f[panel]) * L;
-            const double r = lo_f[panel] * L + 0.5 * h * (cT.g16t[node] + 1.0);
-            const double wr = 0.5 * h * cT.g16w[node];
-            double sn, cs;
-            sincos(th_ang[kth], &sn, &cs);
-            const double u = u0 + r * cs, v = v0 + r * sn;
-            lagrange(u, p, lu);
-            lagrange(v, p, lv);
-            double d0 = 0, d1 = 0, d2 = 0, jj = 0;
-            for (int a = 0; a < p; ++a) {
-                double z0 = 0, z1 = 0, z2 = 0, zj = 0;
-                for (int b = 0; b < p; ++b) {
-                    const double l = lv[b];
-                    const int k = a * p + b;
-                    z0 += sD[k] * l;
-                    z1 += sD[pp + k] * l;
-                    z2 += sD[2 * pp + k] * l;
-                    zj += sJ[k] * l;
-                }
-                d0 += lu[a] * z0;
-                d1 += lu[a] * z1;
-                d2 += lu[a] * z2;
-                jj += lu[a] * zj;
-            }
-            // r_vec = x_i - y~ = -(sum of offsets)
-            const double rx = -d0, ry = -d1, rz = -d2;
-            const double r2 = rx * rx + ry * ry + rz * rz;
-            const double inv = 1.0 / r2;
-            const double qq = (n0 * rx + n1 * ry + n2 * rz) * inv;
-            const double base_w = th_w[kth] * wr * r * jj;
-            f_lb = base_w * (qq * qq - Hi * qq) * (1.0 / M_PI);
-            const double gfac = base_w * inv * (0.5 / M_PI);
-            f_g0 = gfac * rx;
-            f_g1 = gfac * ry;
-            f_g2 = gfac * rz;
-            double lg = 0.5 * log(r2);
-            if (panel == 0) lg += cT.logE[node];
-            f_k = base_w * lg * (0.5 / M_PI);
-        } else {
-            for (int a = 0; a < p; ++a) { lu[a] = 0.0; lv[a] = 0.0; }
-        }
-        sF[tid] = f_lb;
-        sF[kQThreads + tid] = f_g0;
-        sF[2 * kQThreads + tid] = f_g1;
-        sF[3 * kQThreads + tid] = f_g2;
-        sF[4 * kQThreads + tid] = f_k;
-        __syncthreads();
-        if (tid < pp) {
-            const int lim = min(kQThreads, npts - base);
-            for (int qq = 0; qq < lim; ++qq) {
-                const double c = sLu[qq * p + a_own] * sLv[qq * p + b_own];
-                acc_lb += sF[qq] * c;
-                acc_g0 += sF[kQThreads + qq] * c;
-                acc_g1 += sF[2 * kQThreads + qq] * c;
-                acc_g2 += sF[3 * kQThreads + qq] * c;
-                acc_k += sF[4 * kQThreads + qq] * c;
-            }
-        }
-        __syncthreads();
-    }
-    if (tid < pp) {
-        const size_t b0 = (size_t)row_ptr[i];   // own patch is the row's first block
-        W_lb[b0 * pp + tid] = acc_lb;
-        W_g[(0 * (size_t)nblk + b0) * pp + tid] = acc_g0;
-        W_g[(1 * (size_t)nblk + b0) * pp + tid] = acc_g1;
-        W_g[(2 * (size_t)nblk + b0) * pp + tid] = acc_g2;
-        W_k[b0 * pp + tid] = acc_k;
-    }
-}
-
 // ------------------------------------------------------------------ near quadrature
-// One block per (target, non-self near patch).  Square codes: level (4 bits),
+// Square codes: level (4 bits),
 // iu (12 bits), iv (12 bits); square = [-1 + 2 iu/2^l, -1 + 2 (iu+1)/2^l] x (same for v).
 __device__ __forceinline__ int sq_code(int lev, int iu, int iv) { return (lev << 24) | (iu << 12) | iv; }
 __device__ __forceinline__ void sq_box(int code, double& u0, double& u1, double& v0, double& v1) {
@@ -317,20 +202,26 @@ __device__ int near_leaves(const double* X, int p, double xi0, double xi1, doubl
     for (int lev = 0; lev <= max_depth; ++lev) {
         if (tid == 0) S.nNext = 0;
         __syncthreads();
-        for (int q = tid; q < S.nCur; q += blockDim.x) {
-            const int code = S.cur[q];
-            double u0, u1, v0, v1;
+        // five lanes a square: its corners and its centre
+        const int lane = tid & 31, k = lane % 5, grp = lane - k;
+        for (int q0 = (tid >> 5) * 6; q0 < S.nCur; q0 += (blockDim.x >> 5) * 6) {
+            const int q = q0 + lane / 5;
+            const bool mine = lane < 30 && q < S.nCur;
+            const int code = mine ? S.cur[q] : 0;
+            double u0, u1, v0, v1, y[3] = {0.0, 0.0, 0.0};
             sq_box(code, u0, u1, v0, v1);
-            const double us[5] = {u0, u1, u1, u0, 0.5 * (u0 + u1)};
-            const double vs[5] = {v0, v0, v1, v1, 0.5 * (v0 + v1)};
-            double y[5][3];
-            for (int k = 0; k < 5; ++k) interp_pos(X, p, us[k], vs[k], y[k]);
-            double size = 0;
-            for (int k = 0; k < 4; ++k) {
-                const double dx = y[k][0] - y[4][0], dy = y[k][1] - y[4][1], dz = y[k][2] - y[4][2];
-                size = fmax(size, sqrt(dx * dx + dy * dy + dz * dz));
-            }
-            const double dx = xi0 - y[4][0], dy = xi1 - y[4][1], dz = xi2 - y[4][2];
+            if (mine)
+                interp_pos(X, p, k == 4 ? 0.5 * (u0 + u1) : (k == 0 || k == 3) ? u0 : u1,
+                           k == 4 ? 0.5 * (v0 + v1) : k < 2 ? v0 : v1, y);
+            double c[3];
+            for (int d = 0; d < 3; ++d) c[d] = __shfl_sync(0xffffffffu, y[d], min(grp + 4, 31));
+            const double ex = y[0] - c[0], ey = y[1] - c[1], ez = y[2] - c[2];
+            const double edge = sqrt(ex * ex + ey * ey + ez * ez);
+            double size = edge;
+            for (int o = 1; o < 4; ++o)
+                size = fmax(size, __shfl_sync(0xffffffffu, edge, min(grp + (k + o) % 5, 31)));
+            if (!mine || k != 0) continue;
+            const double dx = xi0 - c[0], dy = xi1 - c[1], dz = xi2 - c[2];
             const double dist = sqrt(dx * dx + dy * dy + dz * dz);
             const bool split = (lev < max_depth) && (dist < 2.0 * eta * size);
             if (split) {
@@ -370,107 +261,83 @@ __device__ int near_leaves(const double* X, int p, double xi0, double xi1, doubl
     return nleaves;
 }
 
-__global__ void __launch_bounds__(kQThreads)
-k_near_quad(int p, int nblk, const double* __restrict__ x, const double* __restrict__ J,
-            const double* __restrict__ n, const double* __restrict__ H,
-            const int* __restrict__ blk_row, const int* __restrict__ blk_patch,
-            const int* __restrict__ row_ptr, double eta, int max_depth, int max_leaves,
-            double* __restrict__ W_lb, double* __restrict__ W_g, double* __restrict__ W_k,
-            int* __restrict__ err) {
-    const int b = blockIdx.x;
-    const int i = blk_row[b];
-    if (b == row_ptr[i]) return;   // the self block is done by k_self_quad
-    const int P = blk_patch[b];
-    const int pp = p * p;
-    const int tid = threadIdx.x;
-    __shared__ double sD[3 * PM_MAX_P * PM_MAX_P];
-    __shared__ double sJ[PM_MAX_P * PM_MAX_P];
-    __shared__ double sLu[PM_GL16 * PM_MAX_P], sLv[PM_GL16 * PM_MAX_P];
-    __shared__ double sZ[4 * PM_MAX_P * PM_GL16];     // [4][a][r]
-    __shared__ double sF[5 * PM_GL16 * PM_GL16];      // [5][q*16 + r]
+// the leaves of a list of near blocks: start and count in codes for each (kept only while
+// they fit; *used is the number wanted)
+__global__ void __launch_bounds__(32)
+k_near_leaves(int p, const double* __restrict__ x, const int* __restrict__ blocks,
+              const int* __restrict__ blk_row, const int* __restrict__ blk_patch, double eta,
+              int max_depth, int max_leaves, int* __restrict__ start, int* __restrict__ count,
+              int* __restrict__ codes, int cap, int* __restrict__ used, int* __restrict__ err) {
     __shared__ NearBfs bfs;
-    const double* X = x + (size_t)3 * P * pp;
-    const double xi0 = x[3 * i], xi1 = x[3 * i + 1], xi2 = x[3 * i + 2];
-    for (int k = tid; k < pp; k += kQThreads) {
-        const size_t gk = (size_t)P * pp + k;
-        sD[k] = x[3 * gk] - xi0;
-        sD[pp + k] = x[3 * gk + 1] - xi1;
-        sD[2 * pp + k] = x[3 * gk + 2] - xi2;
-        sJ[k] = J[gk];
+    __shared__ int base;
+    const int b = blocks[blockIdx.x], i = blk_row[b];
+    const int nleaves = near_leaves(x + (size_t)3 * blk_patch[b] * p * p, p, x[3 * i], x[3 * i + 1],
+                                    x[3 * i + 2], eta, max_depth, max_leaves, bfs, err);
+    if (threadIdx.x == 0) {
+        base = atomicAdd(used, nleaves);
+        start[blockIdx.x] = base;
+        count[blockIdx.x] = nleaves;
     }
-    const int nleaves = near_leaves(X, p, xi0, xi1, xi2, eta, max_depth, max_leaves, bfs, err);
-    const int a_own = tid / p, b_own = tid - (tid / p) * p;
-    double acc[5] = {0, 0, 0, 0, 0};
-    const double n0 = n[3 * i], n1 = n[3 * i + 1], n2 = n[3 * i + 2];
-    const double Hi = H[i];
-    for (int L = 0; L < nleaves; ++L) {
-        double u0, u1, v0, v1;
-        sq_box(bfs.sorted[L], u0, u1, v0, v1);
-        const double hu = 0.5 * (u1 - u0), hv = 0.5 * (v1 - v0);
-        if (tid < PM_GL16) lagrange(u0 + hu * (cT.g16t[tid] + 1.0), p, sLu + tid * p);
-        else if (tid < 2 * PM_GL16)
-            lagrange(v0 + hv * (cT.g16t[tid - PM_GL16] + 1.0), p, sLv + (tid - PM_GL16) * p);
-        __syncthreads();
-        // Z[c][a][r] = sum_b D_c[a][b] l_b(v_r)  (c = 3: J)
-        for (int e = tid; e < 4 * p * PM_GL16; e += kQThreads) {
-            const int c = e / (p * PM_GL16), rem = e - c * p * PM_GL16;
-            const int a = rem / PM_GL16, r = rem - a * PM_GL16;
-            const double* src = (c < 3) ? (sD + c * pp) : sJ;
-            double z = 0;
-            for (int bb = 0; bb < p; ++bb) z += src[a * p + bb] * sLv[r * p + bb];
-            sZ[(c * p + a) * PM_GL16 + r] = z;
-        }
-        __syncthreads();
-        for (int e = tid; e < PM_GL16 * PM_GL16; e += kQThreads) {
-            const int qn = e / PM_GL16, r = e - qn * PM_GL16;
-            double d0 = 0, d1 = 0, d2 = 0, jj = 0;
-            for (int a = 0; a < p; ++a) {
-                const double l = sLu[qn * p + a];
-                d0 += l * sZ[(0 * p + a) * PM_GL16 + r];
-                d1 += l * sZ[(1 * p + a) * PM_GL16 + r];
-                d2 += l * sZ[(2 * p + a) * PM_GL16 + r];
-                jj += l * sZ[(3 * p + a) * PM_GL16 + r];
+    __syncthreads();
+    for (int k = threadIdx.x; k < nleaves; k += 32)
+        if (base + k < cap) codes[base + k] = bfs.sorted[k];
+}
+
+// ------------------------------------------------------------------ rule tables (pm_quadmm.cu)
+// One block a tile of 64 points.  SELF: tile t is the ray th0 + t of the polar plan (four
+// radial panels of 16 points); else a quarter of the 16 x 16 Gauss points of the cell codes[t / 4].
+constexpr int kTabThreads = 128;
+template <bool SELF>
+__global__ void __launch_bounds__(kTabThreads)
+k_quad_table(int p, int nloc, int th0, const int* __restrict__ th_off,
+             const double* __restrict__ th_ang, const double* __restrict__ th_w,
+             const double* __restrict__ th_L, const int* __restrict__ codes, QmTable T) {
+    __shared__ double sLu[kQmPts][PM_MAX_P_API], sLv[kQmPts][PM_MAX_P_API];
+    const int tile = blockIdx.x, q = threadIdx.x;
+    if (q < kQmPts) {
+        double u, v, wgt, lg = 0.0;
+        if (SELF) {
+            const int kth = th0 + tile;
+            int lo = 0, hi = nloc;                     // the node position whose rays hold kth
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) / 2;
+                if (th_off[mid] <= kth) lo = mid; else hi = mid;
             }
-            const double rx = -d0, ry = -d1, rz = -d2;
-            const double r2 = rx * rx + ry * ry + rz * rz;
-            const double inv = 1.0 / r2;
-            const double qq = (n0 * rx + n1 * ry + n2 * rz) * inv;
-            const double wgt = hu * cT.g16w[qn] * hv * cT.g16w[r] * jj;
-            sF[e] = wgt * (qq * qq - Hi * qq) * (1.0 / M_PI);
-            const double gfac = wgt * inv * (0.5 / M_PI);
-            sF[256 + e] = gfac * rx;
-            sF[512 + e] = gfac * ry;
-            sF[768 + e] = gfac * rz;
-            sF[1024 + e] = wgt * 0.25 / M_PI * log(r2);
+            const double lo_f[4] = {0.0, 0.125, 0.25, 0.5};
+            const double hi_f[4] = {0.125, 0.25, 0.5, 1.0};
+            const int panel = q / PM_GL16, node = q % PM_GL16;
+            const double L = th_L[kth], h = (hi_f[panel] - lo_f[panel]) * L;
+            const double r = lo_f[panel] * L + 0.5 * h * (cT.g16t[node] + 1.0);
+            double sn, cs;
+            sincos(th_ang[kth], &sn, &cs);
+            u = cT.t[lo / p] + r * cs;
+            v = cT.t[lo % p] + r * sn;
+            wgt = th_w[kth] * (0.5 * h * cT.g16w[node]) * r;
+            if (panel == 0) lg = cT.logE[node];
+        } else {
+            double u0, u1, v0, v1;
+            sq_box(codes[tile >> 2], u0, u1, v0, v1);
+            const int e = (tile & 3) * kQmPts + q, a = e / PM_GL16, b = e % PM_GL16;
+            const double hu = 0.5 * (u1 - u0), hv = 0.5 * (v1 - v0);
+            u = u0 + hu * (cT.g16t[a] + 1.0);
+            v = v0 + hv * (cT.g16t[b] + 1.0);
+            wgt = hu * cT.g16w[a] * hv * cT.g16w[b];
         }
-        __syncthreads();
-        // T[k][a][r] = sum_q F[k][q][r] l_a(u_q)  (reuse sZ region is too small; use a loop)
-        if (tid < pp) {
-            for (int r = 0; r < PM_GL16; ++r) {
-                double t5[5] = {0, 0, 0, 0, 0};
-                for (int qn = 0; qn < PM_GL16; ++qn) {
-                    const double l = sLu[qn * p + a_own];
-                    const int e = qn * PM_GL16 + r;
-                    t5[0] += sF[e] * l;
-                    t5[1] += sF[256 + e] * l;
-                    t5[2] += sF[512 + e] * l;
-                    t5[3] += sF[768 + e] * l;
-                    t5[4] += sF[1024 + e] * l;
-                }
-                const double lb = sLv[r * p + b_own];
-                for (int k = 0; k < 5; ++k) acc[k] += t5[k] * lb;
-            }
-        }
-        __syncthreads();
+        lagrange(u, p, sLu[q]);
+        lagrange(v, p, sLv[q]);
+        if (!T.top) T.pt[(size_t)tile * kQmPts + q] = make_double2(wgt * (0.5 / M_PI), 2.0 * lg);
     }
-    if (tid < pp) {
-        const size_t o = (size_t)b * pp + tid;
-        W_lb[o] = acc[0];
-        W_g[0 * (size_t)nblk * pp + o] = acc[1];
-        W_g[1 * (size_t)nblk * pp + o] = acc[2];
-        W_g[2 * (size_t)nblk * pp + o] = acc[3];
-        W_k[o] = acc[4];
+    __syncthreads();
+    const int half = T.npad / 2;
+    double top = 0.0;
+    for (int e = threadIdx.x; e < kQmPts * half; e += kTabThreads) {
+        const int pt = e / half, k = 2 * (e - pt * half);
+        const double a = k < T.n ? sLu[pt][k / p] * sLv[pt][k % p] : 0.0;
+        const double b = k + 1 < T.n ? sLu[pt][(k + 1) / p] * sLv[pt][(k + 1) % p] : 0.0;
+        if (T.top) top = fmax(top, fmax(fabs(a), fabs(b)));
+        else qm_put(T, tile, pt, k, a, b);
     }
+    if (T.top) atomicMax(T.top, __float_as_uint(__double2float_ru(top)));
 }
 
 // ------------------------------------------------------------------ coefficient combination
@@ -1209,20 +1076,32 @@ pm_status pm_near_build(pm_surface* s, const QuadTables& T) {
     k_node_normals<<<pm_ceil_div(N, 128), 128>>>(s->x, N, p, s->npatch_n);
     PM_CUDA_TRY(cudaGetLastError());
     PM_TRY(pm_near_structure(s));
-    const size_t smem = sizeof(double) * (4 * (size_t)pp + 2 * (size_t)kQThreads * p + 5 * kQThreads);
-    if (smem > 48 * 1024)
-        PM_CUDA_TRY(cudaFuncSetAttribute(k_self_quad, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem));
-    k_self_quad<<<N, kQThreads, smem>>>(N, p, s->x, s->J, s->npatch_n, s->H, s->th_off,
-                                        s->th_ang, s->th_w, s->th_L, s->row_ptr, s->nblk,
-                                        s->W_lb, s->W_g, s->W_k);
-    PM_CUDA_TRY(cudaGetLastError());
-    k_near_quad<<<s->nblk, kQThreads>>>(p, s->nblk, s->x, s->J, s->n, s->H, s->blk_row,
-                                        s->blk_patch, s->row_ptr, s->opts.near_eta,
-                                        std::min(s->opts.near_max_depth, 12),
-                                        s->opts.near_max_leaves, s->W_lb, s->W_g, s->W_k,
-                                        s->dev_err);
-    PM_CUDA_TRY(cudaGetLastError());
+    QmRules R;
+    R.n = pp;
+    R.tiles.resize(pp + 1);                     // a ray of the polar plan is a tile
+    PM_CUDA_TRY(cudaMemcpy(R.tiles.data(), s->th_off, sizeof(int) * (pp + 1), cudaMemcpyDeviceToHost));
+    R.self_table = [&](int loc0, int nloc, const QmTable& tab) -> pm_status {
+        const int th0 = R.tiles[loc0];
+        k_quad_table<true><<<R.tiles[loc0 + nloc] - th0, kTabThreads>>>(
+            p, pp, th0, s->th_off, s->th_ang, s->th_w, s->th_L, nullptr, tab);
+        PM_CUDA_TRY(cudaGetLastError());
+        return PM_OK;
+    };
+    R.near_table = [&](const int* codes, int ncodes, const QmTable& tab) -> pm_status {
+        k_quad_table<false><<<4 * ncodes, kTabThreads>>>(p, pp, 0, nullptr, nullptr, nullptr, nullptr,
+                                                         codes, tab);
+        PM_CUDA_TRY(cudaGetLastError());
+        return PM_OK;
+    };
+    R.leaves = [&](const int* blocks, int npairs, int* start, int* count, int* codes, int cap,
+                   int* used) -> pm_status {
+        k_near_leaves<<<npairs, 32>>>(p, s->x, blocks, s->blk_row, s->blk_patch, s->opts.near_eta,
+                                      std::min(s->opts.near_max_depth, 12), s->opts.near_max_leaves,
+                                      start, count, codes, cap, used, s->dev_err);
+        PM_CUDA_TRY(cudaGetLastError());
+        return PM_OK;
+    };
+    PM_TRY(pm_quad_weights(s, R));
     PM_CUDA_TRY(cudaDeviceSynchronize());
     int herr = 0;
     PM_CUDA_TRY(cudaMemcpy(&herr, s->dev_err, sizeof(int), cudaMemcpyDeviceToHost));

@@ -29,6 +29,7 @@
 // P_k^{(alpha, 0)} by their three-term recurrence; unnormalised (U absorbs the
 // scale), in the order m = 0..n, k = 0..n - m.
 #include "pm_internal.cuh"
+#include "pm_quadmm.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -104,8 +105,57 @@ struct TriConst {
     int p, n, nt;
     double U[PM_TRI_MAX_NT * PM_TRI_MAX_NT];
     double g16t[PM_GL16], g16w[PM_GL16], logE[PM_GL16];
+    // koornwinder's recurrences with their divisions done: A[m+1] = rA[m][0] a A[m] - rA[m][1] b^2 A[m-1],
+    // B_k = (rB[pos][0] t + rB[pos][1]) B_{k-1} - rB[pos][2] B_{k-2} at the position pos of (m, k)
+    double rA[PM_TRI_MAX_P][2], rB[PM_TRI_MAX_NT][3];
 };
 __constant__ TriConst cTri;
+
+void tri_recurrences(int n, TriConst* C) {
+    for (int m = 1; m < n; ++m) {
+        C->rA[m][0] = (2.0 * m + 1.0) / (m + 1.0);
+        C->rA[m][1] = m / (m + 1.0);
+    }
+    int pos = 0;
+    for (int m = 0; m <= n; ++m) {
+        const double al = 2.0 * m + 1.0;
+        for (int k = 0; k <= n - m; ++k, ++pos) {
+            double* r = C->rB[pos];
+            if (k == 1) {
+                r[0] = 0.5 * (al + 2.0);
+                r[1] = 0.5 * al;
+                r[2] = 0.0;
+            } else if (k > 1) {
+                const double j = k - 1.0, c2 = 2.0 * j + al, d = 2.0 * (j + 1.0) * (j + al + 1.0) * c2;
+                r[0] = (c2 + 1.0) * (c2 + 2.0) * c2 / d;
+                r[1] = (c2 + 1.0) * al * al / d;
+                r[2] = 2.0 * j * (j + al) * (c2 + 2.0) / d;
+            }
+        }
+    }
+}
+
+// koornwinder with the tabulated recurrences
+__device__ inline void tri_koornwinder(double u, double v, double* out) {
+    const int n = cTri.n;
+    const double a = 2.0 * u + v - 1.0, b2 = (1.0 - v) * (1.0 - v), t = 2.0 * v - 1.0;
+    double A0 = 0.0, A = 1.0;                       // A[m-1], A[m]
+    int pos = 0;
+    for (int m = 0; m <= n; ++m) {
+        double p0 = 0.0, p1 = A;                    // A[m] B_{k-2}, A[m] B_{k-1}
+        for (int k = 0; k <= n - m; ++k, ++pos) {
+            if (k > 0) {
+                const double p2 = fma(fma(cTri.rB[pos][0], t, cTri.rB[pos][1]), p1, -cTri.rB[pos][2] * p0);
+                p0 = p1;
+                p1 = p2;
+            }
+            out[pos] = p1;
+        }
+        const double An = m == 0 ? a : cTri.rA[m][0] * a * A - cTri.rA[m][1] * b2 * A0;
+        A0 = A;
+        A = An;
+    }
+}
 
 constexpr int kTT = 128;            // threads (quadrature points per chunk) of the kernels
 constexpr int kTriMaxLevel = 1024;  // sub-triangles per BFS level
@@ -114,7 +164,7 @@ constexpr int kTriMaxLeaves = 512;
 // l_k(u, v) for all nodes
 __device__ inline void tri_basis(double u, double v, double* l) {
     double K[PM_TRI_MAX_NT];
-    koornwinder<double>(cTri.n, u, v, K);
+    tri_koornwinder(u, v, K);
     const int nt = cTri.nt;
     for (int k = 0; k < nt; ++k) {
         double acc = 0.0;
@@ -180,145 +230,6 @@ __global__ void k_node_normals_tri(const double* __restrict__ x, int N, int nt,
     nn[3 * k + 2] = c2 * inv;
 }
 
-// One chunk of up to kTT quadrature points: each thread has put its point's basis
-// into sL[tid][.] and its five integrand values into sF[.][tid]; threads k < nt add
-// sum_q F[.][q] l_k(q) to their accumulators.
-__device__ inline void tri_accumulate(const double* sL, const double* sF, int lim, int nt,
-                                      double* acc) {
-    const int tid = threadIdx.x;
-    if (tid < nt) {
-        for (int q = 0; q < lim; ++q) {
-            const double l = sL[q * nt + tid];
-            for (int c = 0; c < 5; ++c) acc[c] += sF[c * kTT + q] * l;
-        }
-    }
-}
-
-// The five coefficient-free integrands (pm_nearfield.cu) at one point, r = x - y~.
-__device__ inline void tri_integrands(double rx, double ry, double rz, double n0, double n1,
-                                      double n2, double Hi, double wgt, double logc, double* f) {
-    const double r2 = rx * rx + ry * ry + rz * rz;
-    const double inv = 1.0 / r2;
-    const double qq = (n0 * rx + n1 * ry + n2 * rz) * inv;
-    f[0] = wgt * (qq * qq - Hi * qq) * (1.0 / M_PI);
-    const double gfac = wgt * inv * (0.5 / M_PI);
-    f[1] = gfac * rx;
-    f[2] = gfac * ry;
-    f[3] = gfac * rz;
-    f[4] = wgt * (0.5 * log(r2) + logc) * (0.5 / M_PI);
-}
-
-// Self patch.  The polar points depend only on the target's node position in its
-// patch, so one block takes kTriG targets at the same position in consecutive
-// patches: each point's basis values (the costly part: nt^2 products with U) are
-// computed once for all of them, then each target's offsets and element give its
-// integrands.  The (target, node) accumulators are spread over the block's threads;
-// every target's sum runs over the points in the same order as with one target a
-// block.  Dynamic shared memory (doubles): basis [kTT][nt], integrands
-// [kTriG][5][kTT], offsets [kTriG][3][nt], elements [kTriG][nt].
-constexpr int kTriG = 8;
-constexpr int kTriAccPerThread = (kTriG * PM_TRI_MAX_NT + kTT - 1) / kTT;
-
-__global__ void __launch_bounds__(kTT)
-k_self_quad_tri(int npatch, const double* __restrict__ x, const double* __restrict__ J,
-                const double* __restrict__ nn, const double* __restrict__ H,
-                const double* __restrict__ ref_u, const double* __restrict__ ref_v,
-                const int* __restrict__ th_off, const double* __restrict__ th_ang,
-                const double* __restrict__ th_w, const double* __restrict__ th_L,
-                const int* __restrict__ row_ptr, int nblk, double* __restrict__ W_lb,
-                double* __restrict__ W_g, double* __restrict__ W_k) {
-    extern __shared__ double sm[];
-    const int nt = cTri.nt;
-    const int loc = blockIdx.y, tid = threadIdx.x;   // x: patch groups (no 65,535 cap)
-    const int P0 = blockIdx.x * kTriG;
-    const int G = min(kTriG, npatch - P0);
-    double* sL = sm;                                   // [kTT][nt]
-    double* sF = sL + kTT * nt;                        // [kTriG][5][kTT]
-    double* sD = sF + kTriG * 5 * kTT;                 // [kTriG][3][nt]
-    double* sJ = sD + kTriG * 3 * nt;                  // [kTriG][nt]
-    for (int e = tid; e < G * nt; e += kTT) {
-        const int g = e / nt, k = e - (e / nt) * nt;
-        const size_t i = (size_t)(P0 + g) * nt + loc, gk = (size_t)(P0 + g) * nt + k;
-        sD[(g * 3 + 0) * nt + k] = x[3 * gk] - x[3 * i];
-        sD[(g * 3 + 1) * nt + k] = x[3 * gk + 1] - x[3 * i + 1];
-        sD[(g * 3 + 2) * nt + k] = x[3 * gk + 2] - x[3 * i + 2];
-        sJ[g * nt + k] = J[gk];
-    }
-    const double u0 = ref_u[loc], v0 = ref_v[loc];
-    const int t0 = th_off[loc], t1 = th_off[loc + 1];
-    const int npts = (t1 - t0) * (PM_RADIAL_PANELS * PM_GL16);
-    const double lo_f[4] = {0.0, 0.125, 0.25, 0.5};
-    const double hi_f[4] = {0.125, 0.25, 0.5, 1.0};
-    double acc[kTriAccPerThread][5];
-    for (int m = 0; m < kTriAccPerThread; ++m)
-        for (int c = 0; c < 5; ++c) acc[m][c] = 0.0;
-    __syncthreads();
-    for (int base = 0; base < npts; base += kTT) {
-        const int q = base + tid;
-        double* l = sL + tid * nt;
-        if (q < npts) {
-            const int kth = t0 + q / (PM_RADIAL_PANELS * PM_GL16);
-            const int rj = q % (PM_RADIAL_PANELS * PM_GL16);
-            const int panel = rj / PM_GL16, node = rj % PM_GL16;
-            const double L = th_L[kth];
-            const double h = (hi_f[panel] - lo_f[panel]) * L;
-            const double r = lo_f[panel] * L + 0.5 * h * (cTri.g16t[node] + 1.0);
-            const double wr = 0.5 * h * cTri.g16w[node];
-            double sn, cs;
-            sincos(th_ang[kth], &sn, &cs);
-            tri_basis(u0 + r * cs, v0 + r * sn, l);
-            const double wpt = th_w[kth] * wr * r;
-            const double logc = panel == 0 ? cTri.logE[node] : 0.0;
-            for (int g = 0; g < kTriG; ++g) {
-                double f[5] = {0, 0, 0, 0, 0};
-                if (g < G) {
-                    const double* D = sD + g * 3 * nt;
-                    const double* Jg = sJ + g * nt;
-                    double d0 = 0, d1 = 0, d2 = 0, jj = 0;
-                    for (int k = 0; k < nt; ++k) {
-                        d0 += l[k] * D[k];
-                        d1 += l[k] * D[nt + k];
-                        d2 += l[k] * D[2 * nt + k];
-                        jj += l[k] * Jg[k];
-                    }
-                    const size_t i = (size_t)(P0 + g) * nt + loc;
-                    tri_integrands(-d0, -d1, -d2, nn[3 * i], nn[3 * i + 1], nn[3 * i + 2], H[i],
-                                   wpt * jj, logc, f);
-                }
-                for (int c = 0; c < 5; ++c) sF[(g * 5 + c) * kTT + tid] = f[c];
-            }
-        } else {
-            for (int k = 0; k < nt; ++k) l[k] = 0.0;
-            for (int g = 0; g < kTriG; ++g)
-                for (int c = 0; c < 5; ++c) sF[(g * 5 + c) * kTT + tid] = 0.0;
-        }
-        __syncthreads();
-        const int lim = min(kTT, npts - base);
-        for (int m = 0; m < kTriAccPerThread; ++m) {
-            const int pr = tid + m * kTT;
-            if (pr >= G * nt) break;
-            const int g = pr / nt, k = pr - (pr / nt) * nt;
-            for (int e = 0; e < lim; ++e) {
-                const double lv = sL[e * nt + k];
-                for (int c = 0; c < 5; ++c) acc[m][c] += sF[(g * 5 + c) * kTT + e] * lv;
-            }
-        }
-        __syncthreads();
-    }
-    for (int m = 0; m < kTriAccPerThread; ++m) {
-        const int pr = tid + m * kTT;
-        if (pr >= G * nt) break;
-        const int g = pr / nt, k = pr - (pr / nt) * nt;
-        const size_t i = (size_t)(P0 + g) * nt + loc;
-        const size_t b0 = (size_t)row_ptr[i];          // own patch: the row's first block
-        W_lb[b0 * nt + k] = acc[m][0];
-        W_g[(0 * (size_t)nblk + b0) * nt + k] = acc[m][1];
-        W_g[(1 * (size_t)nblk + b0) * nt + k] = acc[m][2];
-        W_g[(2 * (size_t)nblk + b0) * nt + k] = acc[m][3];
-        W_k[b0 * nt + k] = acc[m][4];
-    }
-}
-
 // Sub-triangle codes: level (4 bits) << 24 | child path (2 bits a level, first
 // level in the high bits).  Children of (A, B, C): (A, AB, CA), (AB, B, BC),
 // (CA, BC, C), (BC, CA, AB).
@@ -338,54 +249,31 @@ __device__ inline void tri_box(int code, double* tu, double* tv) {
     tu[0] = au; tv[0] = av; tu[1] = bu; tv[1] = bv; tu[2] = cu; tv[2] = cv;
 }
 
-// Shared memory of k_near_quad_tri: the subdivision's work lists are dead once the
-// leaves are sorted, so they share storage with the points' basis values.
-struct TriNearShared {
-    double D[3 * PM_TRI_MAX_NT], J[PM_TRI_MAX_NT], X[3 * PM_TRI_MAX_NT];
-    double F[5 * kTT];
-    int sorted[kTriMaxLeaves];
-    int nCur, nNext, nLeaf, overflow;
-    union {
-        double L[kTT * PM_TRI_MAX_NT];
-        struct {
-            int cur[kTriMaxLevel], next[kTriMaxLevel], leaf[kTriMaxLeaves];
-        } bfs;
-    } u;
+// The leaves of a list of near blocks, a warp each (the subdivision of the file comment): start
+// and count in codes (kept only while they fit; *used is the number wanted).
+struct TriLeafShared {
+    double X[3 * PM_TRI_MAX_NT];
+    int cur[kTriMaxLevel], next[kTriMaxLevel], leaf[kTriMaxLeaves];
+    int nCur, nNext, nLeaf, overflow, base;
 };
-
-// Near, non-self patches: one block per (target, patch) block.
-__global__ void __launch_bounds__(kTT)
-k_near_quad_tri(int nblk, const double* __restrict__ x, const double* __restrict__ J,
-                const double* __restrict__ n, const double* __restrict__ H,
-                const int* __restrict__ blk_row, const int* __restrict__ blk_patch,
-                const int* __restrict__ row_ptr, double eta, int max_depth, int max_leaves,
-                double* __restrict__ W_lb, double* __restrict__ W_g, double* __restrict__ W_k,
-                int* __restrict__ err) {
-    const int b = blockIdx.x;
-    const int i = blk_row[b];
-    if (b == row_ptr[i]) return;   // the self block is done by k_self_quad_tri
-    const int nt = cTri.nt;
-    const int P = blk_patch[b];
-    const int tid = threadIdx.x;
-    __shared__ TriNearShared S;
-    double* sD = S.D;
-    double* sJ = S.J;
-    double* sX = S.X;
-    double* sF = S.F;
-    double* sL = S.u.L;
+__global__ void __launch_bounds__(32)
+k_tri_leaves(const double* __restrict__ x, const int* __restrict__ blocks,
+             const int* __restrict__ blk_row, const int* __restrict__ blk_patch, double eta,
+             int max_depth, int max_leaves, int* __restrict__ start, int* __restrict__ count,
+             int* __restrict__ codes, int cap, int* __restrict__ used, int* __restrict__ err) {
+    __shared__ TriLeafShared S;
+    const int b = blocks[blockIdx.x], i = blk_row[b], tid = threadIdx.x, nt = cTri.nt;
     const double xi0 = x[3 * i], xi1 = x[3 * i + 1], xi2 = x[3 * i + 2];
-    for (int k = tid; k < nt; k += kTT) {
-        const size_t gk = (size_t)P * nt + k;
-        sX[3 * k] = x[3 * gk];
-        sX[3 * k + 1] = x[3 * gk + 1];
-        sX[3 * k + 2] = x[3 * gk + 2];
-        sD[k] = x[3 * gk] - xi0;
-        sD[nt + k] = x[3 * gk + 1] - xi1;
-        sD[2 * nt + k] = x[3 * gk + 2] - xi2;
-        sJ[k] = J[gk];
+    // the patch in Koornwinder coefficients: a position costs 3 nt operations instead of nt^2
+    const double* X = x + (size_t)3 * blk_patch[b] * nt;
+    for (int e = tid; e < 3 * nt; e += 32) {
+        const int m = e / 3, c = e - 3 * m;
+        double v = 0.0;
+        for (int k = 0; k < nt; ++k) v += cTri.U[m * nt + k] * X[3 * k + c];
+        S.X[e] = v;
     }
     if (tid == 0) {
-        S.u.bfs.cur[0] = 0;            // level 0: T0 itself
+        S.cur[0] = 0;                  // level 0: T0 itself
         S.nCur = 1;
         S.nLeaf = 0;
         S.overflow = 0;
@@ -395,94 +283,126 @@ k_near_quad_tri(int nblk, const double* __restrict__ x, const double* __restrict
     for (int lev = 0; lev <= max_depth; ++lev) {
         if (tid == 0) S.nNext = 0;
         __syncthreads();
-        for (int q = tid; q < S.nCur; q += kTT) {
-            const int code = S.u.bfs.cur[q];
-            double tu[3], tv[3], y[4][3];
+        // four lanes a sub-triangle: its corners and its centroid
+        const int k = tid & 3, grp = tid & ~3;
+        for (int q0 = 0; q0 < S.nCur; q0 += 8) {
+            const int q = q0 + (tid >> 2);
+            const bool mine = q < S.nCur;
+            const int code = mine ? S.cur[q] : 0;
+            double tu[3], tv[3], y[3] = {0.0, 0.0, 0.0}, c[3];
             tri_box(code, tu, tv);
-            for (int k = 0; k < 3; ++k) tri_pos(sX, tu[k], tv[k], y[k]);
-            tri_pos(sX, (tu[0] + tu[1] + tu[2]) / 3.0, (tv[0] + tv[1] + tv[2]) / 3.0, y[3]);
-            double size = 0;
-            for (int k = 0; k < 3; ++k) {
-                const double dx = y[k][0] - y[3][0], dy = y[k][1] - y[3][1], dz = y[k][2] - y[3][2];
-                size = fmax(size, sqrt(dx * dx + dy * dy + dz * dz));
+            if (mine) {
+                double K[PM_TRI_MAX_NT];
+                tri_koornwinder(k == 0 ? tu[0] : k == 1 ? tu[1] : k == 2 ? tu[2] : (tu[0] + tu[1] + tu[2]) / 3.0,
+                                k == 0 ? tv[0] : k == 1 ? tv[1] : k == 2 ? tv[2] : (tv[0] + tv[1] + tv[2]) / 3.0, K);
+                for (int m = 0; m < nt; ++m)
+                    for (int d = 0; d < 3; ++d) y[d] += K[m] * S.X[3 * m + d];
             }
-            const double dx = xi0 - y[3][0], dy = xi1 - y[3][1], dz = xi2 - y[3][2];
+            for (int d = 0; d < 3; ++d) c[d] = __shfl_sync(0xffffffffu, y[d], grp + 3);
+            const double ex = y[0] - c[0], ey = y[1] - c[1], ez = y[2] - c[2];
+            double size = sqrt(ex * ex + ey * ey + ez * ez);
+            size = fmax(size, __shfl_xor_sync(0xffffffffu, size, 1));
+            size = fmax(size, __shfl_xor_sync(0xffffffffu, size, 2));
+            if (!mine || k != 0) continue;
+            const double dx = xi0 - c[0], dy = xi1 - c[1], dz = xi2 - c[2];
             const double dist = sqrt(dx * dx + dy * dy + dz * dz);
             if (lev < max_depth && dist < 2.0 * eta * size) {
                 const int slot = atomicAdd(&S.nNext, 4);
                 if (slot + 4 <= kTriMaxLevel) {
                     const int l1 = lev + 1, path = code & 0xffffff;
-                    for (int c = 0; c < 4; ++c) S.u.bfs.next[slot + c] = (l1 << 24) | (path << 2) | c;
+                    for (int ch = 0; ch < 4; ++ch) S.next[slot + ch] = (l1 << 24) | (path << 2) | ch;
                 } else {
                     S.overflow = 1;
                 }
             } else {
                 const int slot = atomicAdd(&S.nLeaf, 1);
-                if (slot < leaf_cap) S.u.bfs.leaf[slot] = code; else S.overflow = 1;
+                if (slot < leaf_cap) S.leaf[slot] = code; else S.overflow = 1;
             }
         }
         __syncthreads();
         const int nn_ = min(S.nNext, kTriMaxLevel);
-        for (int q = tid; q < nn_; q += kTT) S.u.bfs.cur[q] = S.u.bfs.next[q];
+        for (int q = tid; q < nn_; q += 32) S.cur[q] = S.next[q];
         __syncthreads();
         if (tid == 0) S.nCur = nn_;
         __syncthreads();
         if (S.nCur == 0) break;
     }
     const int nleaves = min(S.nLeaf, leaf_cap);
-    if (S.overflow && tid == 0) atomicExch(err, PM_DEV_LEAF_OVERFLOW);
-    for (int q = tid; q < nleaves; q += kTT) {
-        const int c = S.u.bfs.leaf[q];
-        int rank = 0;
-        for (int t = 0; t < nleaves; ++t) rank += (S.u.bfs.leaf[t] < c);
-        S.sorted[rank] = c;
+    if (tid == 0) {
+        if (S.overflow) atomicExch(err, PM_DEV_LEAF_OVERFLOW);
+        S.base = atomicAdd(used, nleaves);
+        start[blockIdx.x] = S.base;
+        count[blockIdx.x] = nleaves;
     }
-    __syncthreads();     // the work lists are dead from here: S.u holds basis values
-    const double n0 = n[3 * i], n1 = n[3 * i + 1], n2 = n[3 * i + 2];
-    const double Hi = H[i];
-    double acc[5] = {0, 0, 0, 0, 0};
-    const int npts = nleaves * PM_GL16 * PM_GL16;
-    for (int base = 0; base < npts; base += kTT) {
-        const int q = base + tid;
-        double* l = sL + tid * nt;
-        double f[5] = {0, 0, 0, 0, 0};
-        if (q < npts) {
-            const int leaf = q / (PM_GL16 * PM_GL16), e = q - leaf * PM_GL16 * PM_GL16;
-            const int is = e / PM_GL16, it = e - is * PM_GL16;
+    __syncthreads();
+    // in code order, so that a block's sum runs the same way every time
+    for (int q = tid; q < nleaves; q += 32) {
+        const int c = S.leaf[q];
+        int rank = 0;
+        for (int t = 0; t < nleaves; ++t) rank += (S.leaf[t] < c);
+        if (S.base + rank < cap) codes[S.base + rank] = c;
+    }
+}
+
+// Rule tables (pm_quadmm.cu), a block a tile of 64 points.  SELF: tile t is the ray th0 + t of
+// the polar plan; else a quarter of the 16 x 16 collapsed Gauss points of the cell codes[t / 4].
+template <bool SELF>
+__global__ void __launch_bounds__(kTT)
+k_tri_table(int th0, const double* __restrict__ ref_u, const double* __restrict__ ref_v,
+            const int* __restrict__ th_off, const double* __restrict__ th_ang,
+            const double* __restrict__ th_w, const double* __restrict__ th_L,
+            const int* __restrict__ codes, QmTable T) {
+    __shared__ double sK[kQmPts][PM_TRI_MAX_NT + 1];
+    const int tile = blockIdx.x, q = threadIdx.x, nt = cTri.nt;
+    if (q < kQmPts) {
+        double u, v, wgt, lg = 0.0;
+        if (SELF) {
+            const int kth = th0 + tile;
+            int lo = 0, hi = nt;                       // the node position whose rays hold kth
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) / 2;
+                if (th_off[mid] <= kth) lo = mid; else hi = mid;
+            }
+            const double lo_f[4] = {0.0, 0.125, 0.25, 0.5};
+            const double hi_f[4] = {0.125, 0.25, 0.5, 1.0};
+            const int panel = q / PM_GL16, node = q % PM_GL16;
+            const double L = th_L[kth], h = (hi_f[panel] - lo_f[panel]) * L;
+            const double r = lo_f[panel] * L + 0.5 * h * (cTri.g16t[node] + 1.0);
+            double sn, cs;
+            sincos(th_ang[kth], &sn, &cs);
+            u = ref_u[lo] + r * cs;
+            v = ref_v[lo] + r * sn;
+            wgt = th_w[kth] * (0.5 * h * cTri.g16w[node]) * r;
+            if (panel == 0) lg = cTri.logE[node];
+        } else {
             double tu[3], tv[3];
-            tri_box(S.sorted[leaf], tu, tv);
+            tri_box(codes[tile >> 2], tu, tv);
             // collapsed Gauss point of T0 (u' = s (1 - t), v' = t), mapped affinely
-            const double s = 0.5 * (cTri.g16t[is] + 1.0), t = 0.5 * (cTri.g16t[it] + 1.0);
-            const double up = s * (1.0 - t), vp = t;
-            const double wq = 0.25 * cTri.g16w[is] * cTri.g16w[it] * (1.0 - t);
+            const int e = (tile & 3) * kQmPts + q, is = e / PM_GL16, jt = e % PM_GL16;
+            const double s = 0.5 * (cTri.g16t[is] + 1.0), t = 0.5 * (cTri.g16t[jt] + 1.0);
             const double e1u = tu[1] - tu[0], e1v = tv[1] - tv[0];
             const double e2u = tu[2] - tu[0], e2v = tv[2] - tv[0];
-            const double det = fabs(e1u * e2v - e2u * e1v);
-            tri_basis(tu[0] + up * e1u + vp * e2u, tv[0] + up * e1v + vp * e2v, l);
-            double d0 = 0, d1 = 0, d2 = 0, jj = 0;
-            for (int k = 0; k < nt; ++k) {
-                d0 += l[k] * sD[k];
-                d1 += l[k] * sD[nt + k];
-                d2 += l[k] * sD[2 * nt + k];
-                jj += l[k] * sJ[k];
-            }
-            tri_integrands(-d0, -d1, -d2, n0, n1, n2, Hi, wq * det * jj, 0.0, f);
-        } else {
-            for (int k = 0; k < nt; ++k) l[k] = 0.0;
+            u = tu[0] + s * (1.0 - t) * e1u + t * e2u;
+            v = tv[0] + s * (1.0 - t) * e1v + t * e2v;
+            wgt = 0.25 * cTri.g16w[is] * cTri.g16w[jt] * (1.0 - t) * fabs(e1u * e2v - e2u * e1v);
         }
-        for (int c = 0; c < 5; ++c) sF[c * kTT + tid] = f[c];
-        __syncthreads();
-        tri_accumulate(sL, sF, min(kTT, npts - base), nt, acc);
-        __syncthreads();
+        tri_koornwinder(u, v, sK[q]);
+        if (!T.top) T.pt[(size_t)tile * kQmPts + q] = make_double2(wgt * (0.5 / M_PI), 2.0 * lg);
     }
-    if (tid < nt) {
-        const size_t o = (size_t)b * nt + tid;
-        W_lb[o] = acc[0];
-        W_g[0 * (size_t)nblk * nt + o] = acc[1];
-        W_g[1 * (size_t)nblk * nt + o] = acc[2];
-        W_g[2 * (size_t)nblk * nt + o] = acc[3];
-        W_k[o] = acc[4];
+    __syncthreads();
+    const int half = T.npad / 2;
+    double top = 0.0;
+    for (int e = threadIdx.x; e < kQmPts * half; e += kTT) {
+        const int pt = e % kQmPts, k = 2 * (e / kQmPts);
+        double a = 0.0, b = 0.0;
+        for (int m = 0; m < nt; ++m) {
+            if (k < nt) a += sK[pt][m] * cTri.U[m * nt + k];
+            if (k + 1 < nt) b += sK[pt][m] * cTri.U[m * nt + k + 1];
+        }
+        if (T.top) top = fmax(top, fmax(fabs(a), fabs(b)));
+        else qm_put(T, tile, pt, k, a, b);
     }
+    if (T.top) atomicMax(T.top, __float_as_uint(__double2float_ru(top)));
 }
 
 std::mutex g_tri_build_mu;   // cTri holds one surface's tables during its build
@@ -660,6 +580,7 @@ pm_status pm_near_build_tri(pm_surface* s, const QuadTables& Q) {
     C.n = T.p - 1;
     C.nt = nt;
     for (int k = 0; k < nt * nt; ++k) C.U[k] = T.U[k];
+    tri_recurrences(C.n, &C);
     for (int q = 0; q < PM_GL16; ++q) {
         C.g16t[q] = Q.g16t[q];
         C.g16w[q] = Q.g16w[q];
@@ -695,23 +616,38 @@ pm_status pm_near_build_tri(pm_surface* s, const QuadTables& Q) {
             break;
         }
         if ((st = pm_near_structure(s)) != PM_OK) break;
-        const size_t smem = sizeof(double) * ((size_t)kTT * nt + (size_t)kTriG * 5 * kTT +
-                                              (size_t)kTriG * 4 * nt);
-        ce = cudaFuncSetAttribute(k_self_quad_tri, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem);
+        QmRules R;
+        R.n = nt;
+        R.tiles.resize(nt + 1);                 // a ray of the polar plan is a tile
+        ce = cudaMemcpy(R.tiles.data(), s->th_off, sizeof(int) * (nt + 1), cudaMemcpyDeviceToHost);
         if (ce != cudaSuccess) {
             pm_set_error("triangle self rule: %s", cudaGetErrorString(ce));
             st = PM_ERR_CUDA;
             break;
         }
-        k_self_quad_tri<<<dim3(pm_ceil_div(npatch, kTriG), nt), kTT, smem>>>(
-            npatch, s->x, s->J, s->npatch_n, s->H, ru, rv, s->th_off, s->th_ang, s->th_w,
-            s->th_L, s->row_ptr, s->nblk, s->W_lb, s->W_g, s->W_k);
-        k_near_quad_tri<<<s->nblk, kTT>>>(s->nblk, s->x, s->J, s->n, s->H, s->blk_row,
-                                          s->blk_patch, s->row_ptr, s->opts.near_eta,
-                                          std::min(s->opts.near_max_depth, 12),
-                                          s->opts.near_max_leaves, s->W_lb, s->W_g, s->W_k,
-                                          s->dev_err);
+        R.self_table = [&](int loc0, int nloc, const QmTable& tab) -> pm_status {
+            const int th0 = R.tiles[loc0];
+            k_tri_table<true><<<R.tiles[loc0 + nloc] - th0, kTT>>>(th0, ru, rv, s->th_off, s->th_ang,
+                                                                   s->th_w, s->th_L, nullptr, tab);
+            PM_CUDA_TRY(cudaGetLastError());
+            return PM_OK;
+        };
+        R.near_table = [&](const int* codes, int ncodes, const QmTable& tab) -> pm_status {
+            k_tri_table<false><<<4 * ncodes, kTT>>>(0, ru, rv, nullptr, nullptr, nullptr, nullptr,
+                                                    codes, tab);
+            PM_CUDA_TRY(cudaGetLastError());
+            return PM_OK;
+        };
+        R.leaves = [&](const int* blocks, int npairs, int* start, int* count, int* codes, int cap,
+                       int* used) -> pm_status {
+            k_tri_leaves<<<npairs, 32>>>(s->x, blocks, s->blk_row, s->blk_patch, s->opts.near_eta,
+                                         std::min(s->opts.near_max_depth, 12),
+                                         s->opts.near_max_leaves, start, count, codes, cap, used,
+                                         s->dev_err);
+            PM_CUDA_TRY(cudaGetLastError());
+            return PM_OK;
+        };
+        if ((st = pm_quad_weights(s, R)) != PM_OK) break;
         ce = cudaGetLastError();
         if (ce == cudaSuccess) ce = cudaDeviceSynchronize();
         if (ce != cudaSuccess) {
