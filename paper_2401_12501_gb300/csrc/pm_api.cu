@@ -264,6 +264,7 @@ extern "C" void pm_ctx_destroy(pm_ctx* c) {
     cudaSetDevice(c->device);
     pm_dfree(c->fmm_opR);
     pm_dfree(c->fmm_opK);
+    pm_dfree(c->green_k1); pm_dfree(c->green_h1); pm_dfree(c->green_c2);
     pm_multi_free(c);
     delete c;
 }

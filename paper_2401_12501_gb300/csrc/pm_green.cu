@@ -173,3 +173,149 @@ extern "C" pm_status pm_smooth_c_f32(int N, const float* x, const float* n, cons
     PM_CUDA_TRY(cudaGetLastError());
     return PM_OK;
 }
+
+namespace {
+
+using pm_green::cplx_d;
+__constant__ double cG16[2 * PM_GL16];     // 16-point Gauss-Legendre nodes, weights
+
+// Taylor coefficients a_2.. about c from a_0, a_1 by c (n+2)(n+1) a_{n+2} =
+// s (c a_n + a_{n-1}) - (n+1)^2 a_{n+1}, s = 1 (K) or -1 (H)
+__device__ void taylor(cplx_d c, double s, int terms, cplx_d* a) {
+    const cplx_d ic = pm_green::cz_rcp(c);
+    for (int n = 0; n + 2 < terms; ++n) {
+        cplx_d v = pm_green::cz_mul(c, a[n]);
+        if (n > 0) v = pm_green::cz_add(v, a[n - 1]);
+        v = pm_green::cz_sub(pm_green::cz_scale(v, s), pm_green::cz_scale(a[n + 1], (n + 1.0) * (n + 1.0)));
+        a[n + 2] = pm_green::cz_scale(pm_green::cz_mul(v, ic), 1.0 / ((n + 2.0) * (n + 1.0)));
+    }
+}
+
+__global__ void k_green_rows(double2* __restrict__ k1, double2* __restrict__ h1) {
+    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= pm_green::kTabRows) return;
+    const int oct = row >> 3;
+    const double z = oct < pm_green::kTabOctaves
+                         ? ldexp(1.0 + ((row & 7) + 0.5) / 8.0, oct + pm_green::kTabLow)
+                         : row - pm_green::kTabOctaves * 8 + 16.5;
+    cplx_d a[15];
+    double K0, K1;
+    pm_green::bessel_k01(z, &K0, &K1);
+    a[0] = {K0, 0.0};
+    a[1] = {-K1, 0.0};
+    taylor({z, 0.0}, 1.0, 15, a);
+    k1[row * 8] = make_double2(z, a[0].re);
+    for (int n = 1; n < 8; ++n) k1[row * 8 + n] = make_double2(a[2 * n - 1].re, a[2 * n].re);
+    if (z < 8.0) {
+        a[0] = {j0(z), y0(z)};
+        a[1] = {-j1(z), -y1(z)};
+    } else if (z >= 32.0) {
+        // H_nu = sqrt(2 / (pi z)) e^{i (z - nu pi/2 - pi/4)} sum_k i^k a_k / z^k,
+        // a_k = a_{k-1} (4 nu^2 - (2k - 1)^2) / (8k) (A&S 9.2.7); its smallest term is below e^{-2z}
+        double sn, cs;
+        sincos(z, &sn, &cs);
+        const double m = sqrt(1.0 / (M_PI * z));              // times e^{i z} (1 - i) = e^{i (z - pi/4)} sqrt 2
+        const cplx_d e = {m * (cs + sn), m * (sn - cs)};
+        for (int nu = 0; nu < 2; ++nu) {
+            cplx_d sum = {1.0, 0.0};
+            double t = 1.0;
+            for (int k = 1; k < 40; ++k) {
+                t *= (4.0 * nu * nu - (2.0 * k - 1.0) * (2.0 * k - 1.0)) / (8.0 * k * z);
+                if (fabs(t) < 1e-18) break;
+                const double v = (k & 2) ? -t : t;            // i^k t
+                if (k & 1) sum.im += v;
+                else sum.re += v;
+            }
+            const cplx_d h = pm_green::cz_mul(e, sum);
+            // e^{-i pi/2} turns H1; a_1 = H0' = -H1
+            a[nu] = nu ? cplx_d{-h.im, h.re} : h;
+        }
+    } else {                            // H0 = (2 / (pi i)) K0(-i z), H1 = -(2 / pi) K1(-i z)
+        cplx_d C0, C1;
+        pm_green::bessel_k01_c({0.0, -z}, cG16, cG16 + PM_GL16, &C0, &C1);
+        a[0] = {2.0 / M_PI * C0.im, -2.0 / M_PI * C0.re};
+        a[1] = pm_green::cz_scale(C1, 2.0 / M_PI);
+    }
+    taylor({z, 0.0}, -1.0, 15, a);
+    h1[row * 16] = make_double2(z, 0.0);
+    for (int n = 0; n < 15; ++n) h1[row * 16 + 1 + n] = make_double2(a[n].re, a[n].im);
+}
+
+__global__ void k_green_cells(double2* __restrict__ c2) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= pm_green::kTabCells) return;
+    cplx_d c;
+    double s;
+    if (i < pm_green::kTabOctaves * 1024) {
+        s = ldexp(1.0, (i >> 10) + pm_green::kTabLow - 3);
+        c = {(((i >> 5) & 31) - 15.5) * s, ((i & 31) - 15.5) * s};
+    } else {
+        const int q = i - pm_green::kTabOctaves * 1024;
+        s = 1.0;
+        c = {(q >> 6) - 31.5, (q & 63) - 31.5};
+    }
+    cplx_d a[16];
+    for (int n = 0; n < 16; ++n) a[n] = {0.0, 0.0};
+    // arguments of w lie in (-3 pi/4, pi/4]; cells of the smaller octaves inside are not read
+    const double th = atan2(c.im, c.re);
+    if (th > -0.75 * M_PI - 0.4 && th < 0.25 * M_PI + 0.4 && fmax(fabs(c.re), fabs(c.im)) > 7.0 * s) {
+        cplx_d K0, K1;
+        pm_green::bessel_k01_c(c, cG16, cG16 + PM_GL16, &K0, &K1);
+        a[0] = K0;
+        a[1] = pm_green::cz_scale(K1, -1.0);
+        taylor(c, 1.0, 16, a);
+    }
+    for (int n = 0; n < 16; ++n) c2[(size_t)i * 16 + n] = make_double2(a[n].re, a[n].im);
+}
+
+}  // namespace
+
+pm_status pm_green_tables(pm_ctx* ctx, bool complex_q, pm_green::GreenTab* T) {
+    std::lock_guard<std::mutex> lock(ctx->green_mu);
+    if (!ctx->green_h1 || (complex_q && !ctx->green_c2)) {
+        QuadTables Q;
+        pm_build_tables(2, &Q);
+        double g16[2 * PM_GL16];
+        for (int k = 0; k < PM_GL16; ++k) {
+            g16[k] = Q.g16t[k];
+            g16[PM_GL16 + k] = Q.g16w[k];
+        }
+        PM_CUDA_TRY(cudaMemcpyToSymbol(cG16, g16, sizeof(g16)));
+        PM_CUDA_TRY(pm_green::upload_cheb_k01());
+    }
+    if (!ctx->green_h1) {
+        double2 *k1 = nullptr, *h1 = nullptr;
+        PM_TRY(pm_dmalloc(&k1, (size_t)pm_green::kTabRows * 8));
+        const pm_status st = pm_dmalloc(&h1, (size_t)pm_green::kTabRows * 16);
+        if (st != PM_OK) {
+            pm_dfree(k1);
+            return st;
+        }
+        k_green_rows<<<pm_ceil_div(pm_green::kTabRows, 32), 32>>>(k1, h1);
+        const cudaError_t e = cudaGetLastError() == cudaSuccess ? cudaDeviceSynchronize() : cudaErrorUnknown;
+        if (e != cudaSuccess) {
+            pm_dfree(k1);
+            pm_dfree(h1);
+            pm_set_error("Green's function tables: %s", cudaGetErrorString(e));
+            return PM_ERR_CUDA;
+        }
+        ctx->green_k1 = k1;
+        ctx->green_h1 = h1;
+    }
+    if (complex_q && !ctx->green_c2) {
+        double2* c2 = nullptr;
+        PM_TRY(pm_dmalloc(&c2, (size_t)pm_green::kTabCells * 16));
+        k_green_cells<<<pm_ceil_div(pm_green::kTabCells, 128), 128>>>(c2);
+        const cudaError_t e = cudaGetLastError() == cudaSuccess ? cudaDeviceSynchronize() : cudaErrorUnknown;
+        if (e != cudaSuccess) {
+            pm_dfree(c2);
+            pm_set_error("Green's function tables: %s", cudaGetErrorString(e));
+            return PM_ERR_CUDA;
+        }
+        ctx->green_c2 = c2;
+    }
+    T->k1 = ctx->green_k1;
+    T->h1 = ctx->green_h1;
+    T->c2 = ctx->green_c2;
+    return PM_OK;
+}

@@ -30,6 +30,8 @@
 
 #include <cmath>
 
+#include "pm_internal.cuh"
+
 namespace pm_green {
 
 constexpr double kPi = 3.14159265358979323846;
@@ -411,6 +413,173 @@ __host__ __device__ inline void pair_rk_cz(double rx, double ry, double rz, doub
     out[3] = g[1];
 }
 
+#ifdef __CUDACC__
+// ---------------------------------------------------------------------------
+// Device evaluation by tables.  The functions above cost 500 (J, Y), 170 (K) and some 10,000
+// (K at complex argument) float64 instructions a pair on a pipe of two a clock and SM.  Here
+// H0(z), K0(z) and K0(w) are Taylor sums about the centre of a cell, the derivatives -H1 and
+// -K1 coming out of the same Horner scheme: 15 terms on cells an eighth of an octave wide
+// (at most 1), 16 on square cells of the same size, so that a cell's reach is at most 1/17
+// (0.1 in the plane) of its distance to the singularity at 0 and 0.5 (0.71) of a period:
+// truncation below 1e-16.  The coefficients follow from the functions above at the centre (H0
+// from z = 8 on as K0 at -i z and from 32 on by its asymptotic series, for the math library's
+// J and Y are good to 5e-12 there) and the differential equation, z y'' + y' + z y = 0 (H) or
+// - z y (K).  52 and 26 multiply-adds
+// for real q, 120 for complex.  One set per context (pm_green_tables); arguments outside
+// [2^-12, 256) ([2^-12, 32) for complex ones) go to the functions.
+constexpr int kTabOctaves = 16, kTabLow = -12;
+constexpr int kTabRows = kTabOctaves * 8 + 240;             // z < 16 by eighths, then by ones to 256
+// (struct GreenTab, pm_internal.cuh: k1 [row][8] (centre, a_0), (a_1, a_2), ..., (a_13, a_14);
+// h1 [row][16] (centre, 0), a_0, ..., a_14 complex; c2 [cell][16] a_0, ..., a_15 complex)
+constexpr int kTabCells = kTabOctaves * 32 * 32 + 64 * 64;  // |w|_max < 16, then unit cells to 32
+// q = c~/a~ at a source, with what its pairs share
+struct GreenQ {
+    cplx_d q, kc;      // kc = -i k (complex q)
+    double k;          // sqrt |q| (real q)
+};
+__device__ __forceinline__ GreenQ green_q(cplx_d q) {
+    GreenQ G;
+    G.q = q;
+    G.k = sqrt(fabs(q.re));
+    G.kc = {0.0, 0.0};
+    if (q.im != 0.0) {             // the root and branch of green_scaled_cz
+        const double mod = sqrt(q.re * q.re + q.im * q.im);
+        double kr, ki;
+        if (q.re >= 0.0) {
+            kr = sqrt(0.5 * (mod + q.re));
+            ki = q.im / (2.0 * kr);
+        } else {
+            ki = copysign(sqrt(0.5 * (mod - q.re)), q.im);
+            kr = q.im / (2.0 * ki);
+        }
+        if (q.im < 0.0 && q.re <= 0.0) { kr = -kr; ki = -ki; }
+        G.kc = {ki, -kr};
+    }
+    return G;
+}
+
+__device__ __forceinline__ bool tab_holds(double z, int top) {
+    const int hi = __double2hiint(z);
+    return hi >= (1023 + kTabLow) << 20 && hi < (1023 + top) << 20;
+}
+__device__ __forceinline__ int tab_row(double z) {
+    return z < 16.0 ? (__double2hiint(z) >> 17) - ((1023 + kTabLow) << 3)
+                    : kTabOctaves * 8 - 16 + (int)z;
+}
+// the cell of w and its centre
+__device__ __forceinline__ int tab_cell(cplx_d w, cplx_d* c) {
+    const double m = fmax(fabs(w.re), fabs(w.im));
+    const int e = min((__double2hiint(m) >> 20) - 1023, 3);          // cells of 2^(e - 3)
+    const double inv = __hiloint2double((1023 + 3 - e) << 20, 0), s = __hiloint2double((1023 - 3 + e) << 20, 0);
+    const int ix = __double2int_rd(w.re * inv), iy = __double2int_rd(w.im * inv);
+    *c = {(ix + 0.5) * s, (iy + 0.5) * s};
+    return m < 16.0 ? ((e - kTabLow) * 32 + ix + 16) * 32 + iy + 16
+                    : kTabOctaves * 1024 + (ix + 32) * 64 + iy + 32;
+}
+
+// the functions above, for arguments off the tables (kept out of the callers' registers)
+static __device__ __noinline__ void green_off_tables(double r, cplx_d q, const double* g16t,
+                                                     const double* g16w, double* out) {
+    if (q.im == 0.0) green_scaled_any(r, q.re, out);
+    else green_scaled_cz(r, q, g16t, g16w, out);
+}
+
+// (g, g', g'') as green_scaled_cz gives them; inv_r = 1/r.  g'' = -q g - g'/r.
+__device__ __forceinline__ void green_by_tables(double r, double inv_r, const GreenQ& G,
+                                                const GreenTab& T, const double* g16t,
+                                                const double* g16w, double* out) {
+    const double inv2pi = 0.5 / kPi;
+    if (G.q.im == 0.0) {
+        const double z = G.k * r;
+        if (tab_holds(z, 8)) {
+            const int row = tab_row(z);
+            if (G.q.re > 0.0) {
+                const double2* R = T.h1 + row * 16;
+                const double t = z - R[0].x;
+                double2 p = R[15], d = make_double2(0.0, 0.0);
+#pragma unroll
+                for (int n = 14; n > 0; --n) {
+                    const double2 a = R[n];
+                    d.x = fma(d.x, t, p.x);
+                    d.y = fma(d.y, t, p.y);
+                    p.x = fma(p.x, t, a.x);
+                    p.y = fma(p.y, t, a.y);
+                }
+                out[0] = 0.25 * p.y;                         // -(i/4) H0
+                out[1] = -0.25 * p.x;
+                out[2] = 0.25 * G.k * d.y;                   // -(i k/4) H0'
+                out[3] = -0.25 * G.k * d.x;
+                out[4] = -G.q.re * out[0] - out[2] * inv_r;
+                out[5] = -G.q.re * out[1] - out[3] * inv_r;
+            } else {
+                const double2* R = T.k1 + row * 8;
+                const double2 r0 = R[0];
+                const double t = z - r0.x;
+                double2 a = R[7];
+                double d = a.y, p = fma(a.y, t, a.x);
+#pragma unroll
+                for (int n = 6; n > 0; --n) {
+                    a = R[n];
+                    d = fma(d, t, p);
+                    p = fma(p, t, a.y);
+                    d = fma(d, t, p);
+                    p = fma(p, t, a.x);
+                }
+                d = fma(d, t, p);
+                p = fma(p, t, r0.y);
+                out[0] = -p * inv2pi;
+                out[2] = -G.k * d * inv2pi;                  // kappa K1 / (2 pi)
+                out[4] = -G.q.re * out[0] - out[2] * inv_r;
+                out[1] = out[3] = out[5] = 0.0;
+            }
+            return;
+        }
+    } else if (T.c2) {
+        const cplx_d w = cz_scale(G.kc, r);
+        if (tab_holds(fmax(fabs(w.re), fabs(w.im)), 5)) {
+            cplx_d c;
+            const double2* R = T.c2 + (size_t)tab_cell(w, &c) * 16;
+            const cplx_d t = cz_sub(w, c);
+            cplx_d p = {R[15].x, R[15].y}, d = {0.0, 0.0};
+#pragma unroll
+            for (int n = 14; n >= 0; --n) {
+                const double2 a = R[n];
+                d = {fma(d.re, t.re, fma(-d.im, t.im, p.re)), fma(d.re, t.im, fma(d.im, t.re, p.im))};
+                p = {fma(p.re, t.re, fma(-p.im, t.im, a.x)), fma(p.re, t.im, fma(p.im, t.re, a.y))};
+            }
+            const cplx_d g = cz_scale(p, -inv2pi), g1 = cz_scale(cz_mul(G.kc, d), -inv2pi);
+            const cplx_d qg = cz_mul(G.q, g);
+            out[0] = g.re; out[1] = g.im;
+            out[2] = g1.re; out[3] = g1.im;
+            out[4] = -qg.re - g1.re * inv_r;
+            out[5] = -qg.im - g1.im * inv_r;
+            return;
+        }
+    }
+    green_off_tables(r, G.q, g16t, g16w, out);
+}
+
+// pair_rk_cz by the tables
+__device__ __forceinline__ void pair_rk_tab(double rx, double ry, double rz, double nx, double ny,
+                                            double nz, double H, double a, double gbx, double gby,
+                                            double gbz, cplx_d c, const GreenQ& G, const GreenTab& T,
+                                            const double* g16t, const double* g16w, double* out) {
+    const double r2 = rx * rx + ry * ry + rz * rz;
+    const double inv_r = rsqrt(r2), r = r2 * inv_r;
+    double g[6];
+    green_by_tables(r, inv_r, G, T, g16t, g16w, g);
+    const double nr = (nx * rx + ny * ry + nz * rz) * inv_r;
+    const double gr = (gbx * rx + gby * ry + gbz * rz) * inv_r;
+    const double t2 = a * nr * nr;
+    const double t1 = gr - 2.0 * a * H * nr;
+    const cplx_d t0 = {c.re - a * G.q.re, c.im - a * G.q.im};       // c(x) - a(x) q(y)
+    out[0] = t1 * g[2] - t2 * (g[4] - g[2] * inv_r) + (t0.re * g[0] - t0.im * g[1]);
+    out[1] = t1 * g[3] - t2 * (g[5] - g[3] * inv_r) + (t0.re * g[1] + t0.im * g[0]);
+    out[2] = g[0];
+    out[3] = g[1];
+}
+#endif  // __CUDACC__
+
 // ---------------------------------------------------------------------------
 // float32 versions for the per-pair smooth sums.  Same methods, tuned to
 // float32: the series for x < 2 with ten unrolled terms (t = x^2/4 <= 1, so
@@ -546,3 +715,9 @@ __host__ __device__ inline void pair_rk_c_f32(float rx, float ry, float rz, floa
 }
 
 }  // namespace pm_green
+
+#ifdef __CUDACC__
+struct pm_ctx;
+// the context's tables, built on first use (the complex ones only when asked for) (pm_green.cu)
+pm_status pm_green_tables(pm_ctx* ctx, bool complex_q, pm_green::GreenTab* T);
+#endif

@@ -50,9 +50,9 @@ k_direct_c64(const double* __restrict__ x, const double* __restrict__ n,
              const double* __restrict__ H, const double* __restrict__ a,
              const double* __restrict__ g, const double2* __restrict__ c,
              const double2* __restrict__ qn, const double2* __restrict__ sv, int N, int chunk,
-             double2* __restrict__ partial) {
-    __shared__ double4 sx[kHT];          // source x, y, z, Re q
-    __shared__ double sqi[kHT];          // source Im q
+             pm_green::GreenTab T, double2* __restrict__ partial) {
+    __shared__ double sx[kHT][3];        // source position
+    __shared__ pm_green::GreenQ sq[kHT]; // source q
     __shared__ double2 ss[kHT];          // source strength
     const int tid = threadIdx.x;
     const int i = blockIdx.x * kHT + tid;
@@ -75,8 +75,8 @@ k_direct_c64(const double* __restrict__ x, const double* __restrict__ n,
         __syncthreads();
         const int j = base + tid;
         if (j < s1) {
-            sx[tid] = make_double4(x[3 * j], x[3 * j + 1], x[3 * j + 2], qn[j].x);
-            sqi[tid] = qn[j].y;
+            for (int d = 0; d < 3; ++d) sx[tid][d] = x[3 * j + d];
+            sq[tid] = pm_green::green_q({qn[j].x, qn[j].y});
             ss[tid] = sv[j];
         }
         __syncthreads();
@@ -84,11 +84,11 @@ k_direct_c64(const double* __restrict__ x, const double* __restrict__ n,
         if (i < N) {
             for (int jj = 0; jj < len; ++jj) {
                 if (base + jj == i) continue;
-                const double4 y = sx[jj];
+                const double* y = sx[jj];
                 double out[4];
-                pm_green::pair_rk_cz(xi[0] - y.x, xi[1] - y.y, xi[2] - y.z, ni[0], ni[1], ni[2],
-                                     Hi, ai, gi[0], gi[1], gi[2], ci,
-                                     pm_green::cplx_d{y.w, sqi[jj]}, cHG16, cHG16 + PM_GL16, out);
+                pm_green::pair_rk_tab(xi[0] - y[0], xi[1] - y[1], xi[2] - y[2], ni[0], ni[1], ni[2],
+                                      Hi, ai, gi[0], gi[1], gi[2], ci, sq[jj], T, cHG16,
+                                      cHG16 + PM_GL16, out);
                 const double2 kv = WHICH ? make_double2(out[2], out[3])
                                          : make_double2(out[0], out[1]);
                 const double2 t = cmul(kv, ss[jj]);
@@ -111,7 +111,7 @@ k_fill_c64(const double* __restrict__ x, const double* __restrict__ n,
            const double* __restrict__ H, const double* __restrict__ a,
            const double* __restrict__ g, const double2* __restrict__ c,
            const double2* __restrict__ qn, const double* __restrict__ wa, int N,
-           double2* __restrict__ MR, double2* __restrict__ MK) {
+           pm_green::GreenTab T, double2* __restrict__ MR, double2* __restrict__ MK) {
     __shared__ double st[kFillRows][13];   // x, n, grad a, H, a, Re c, Im c
     const int i0 = blockIdx.y * kFillRows, rows = min(kFillRows, N - i0);
     for (int e = threadIdx.x; e < rows * 13; e += kHT) {
@@ -123,14 +123,14 @@ k_fill_c64(const double* __restrict__ x, const double* __restrict__ n,
     const int j = blockIdx.x * kHT + threadIdx.x;
     if (j >= N) return;
     const double xj0 = x[3 * j], xj1 = x[3 * j + 1], xj2 = x[3 * j + 2], wj = wa[j];
-    const pm_green::cplx_d qj = {qn[j].x, qn[j].y};
+    const pm_green::GreenQ qj = pm_green::green_q({qn[j].x, qn[j].y});
     for (int r = 0; r < rows; ++r) {
         const double* t = st[r];
         double out[4] = {0.0, 0.0, 0.0, 0.0};
         if (i0 + r != j)
-            pm_green::pair_rk_cz(t[0] - xj0, t[1] - xj1, t[2] - xj2, t[3], t[4], t[5], t[9], t[10],
-                                 t[6], t[7], t[8], pm_green::cplx_d{t[11], t[12]}, qj, cHG16,
-                                 cHG16 + PM_GL16, out);
+            pm_green::pair_rk_tab(t[0] - xj0, t[1] - xj1, t[2] - xj2, t[3], t[4], t[5], t[9], t[10],
+                                  t[6], t[7], t[8], pm_green::cplx_d{t[11], t[12]}, qj, T, cHG16,
+                                  cHG16 + PM_GL16, out);
         const size_t o = (size_t)(i0 + r) * N + j;
         MR[o] = make_double2(wj * out[0], wj * out[1]);
         MK[o] = make_double2(wj * out[2], wj * out[3]);
@@ -413,10 +413,10 @@ pm_status helm_apply(pm_surface* s, int which_K, const double2* sigma, double2* 
         PhaseTimer t(s, which_K ? PM_PHASE_DIRECT64_K : PM_PHASE_DIRECT64, st);
         if (which_K)
             k_direct_c64<1><<<grid, kHT, 0, st>>>(s->x, s->n, s->H, s->a, s->g, s->cc, s->qn,
-                                                  W->sv, N, chunk, part);
+                                                  W->sv, N, chunk, s->green, part);
         else
             k_direct_c64<0><<<grid, kHT, 0, st>>>(s->x, s->n, s->H, s->a, s->g, s->cc, s->qn,
-                                                  W->sv, N, chunk, part);
+                                                  W->sv, N, chunk, s->green, part);
     }
     PhaseTimer t(s, PM_PHASE_NEAR, st);
     k_near_apply_c64<<<pm_ceil_div((long long)N * 32, kRT), kRT, 0, st>>>(
@@ -451,7 +451,7 @@ struct HelmDense {
         PhaseTimer t(s, PM_PHASE_DIRECT64, st);
         dim3 grid(pm_ceil_div(s->N, kHT), pm_ceil_div(s->N, kFillRows));
         k_fill_c64<<<grid, kHT, 0, st>>>(s->x, s->n, s->H, s->a, s->g, s->cc, s->qn, s->wa, s->N,
-                                         MR, MK);
+                                         s->green, MR, MK);
         k_fill_near_c<<<pm_ceil_div((long long)s->nblk * s->pp, 256), 256, 0, st>>>(
             s->nblk, s->pp, s->blk_row, s->blk_patch, s->cRc, s->cKc, s->N, MR, MK);
         PM_CUDA_TRY(cudaGetLastError());
@@ -561,6 +561,9 @@ extern "C" pm_status pm_surface_set_coeff_c(pm_surface* s, const double* a, cons
         PM_CUDA_TRY(cudaMemcpyToSymbol(cHG16, g16, sizeof(g16)));
         PM_CUDA_TRY(pm_green::upload_cheb_k01());
     }
+    bool complex_q = false;
+    for (int k = 0; k < N; ++k) complex_q = complex_q || c[2 * k + 1] != 0.0;
+    PM_TRY(pm_green_tables(s->ctx, complex_q, &s->green));
     PM_TRY(pm_near_build_c(s));
     s->has_c = 1;
     s->graph_epoch = pm_new_epoch();

@@ -89,6 +89,13 @@ struct QuadTables {
     int p;
 };
 
+// Taylor tables of the c != 0 Green's functions (pm_green.cuh); c2 null: not built
+namespace pm_green {
+struct GreenTab {
+    const double2 *k1 = nullptr, *h1 = nullptr, *c2 = nullptr;
+};
+}  // namespace pm_green
+
 // ----------------------------------------------------------------------------- handles
 struct pm_ctx {
     int device = 0;
@@ -102,6 +109,9 @@ struct pm_ctx {
     // blocks a1 a0 a0 (pm_fmm.cu)
     __half* fmm_opR = nullptr;   // rows = 9 * 512
     __half* fmm_opK = nullptr;   // rows = 512
+    // Taylor tables of the c != 0 Green's functions (pm_green.cuh), built on first use
+    std::mutex green_mu;
+    double2 *green_k1 = nullptr, *green_h1 = nullptr, *green_c2 = nullptr;
     // multi-instance lockstep solve (pm_batch.cu): workspace of the last call's shape
     std::mutex multi_mu;
     struct PmMultiWork* multi = nullptr;
@@ -204,6 +214,7 @@ struct pm_surface {
     double2* cRc = nullptr;       // [nblk*pp]
     double2* cKc = nullptr;       // [nblk*pp]
     PmHelmWork* helm = nullptr;
+    pm_green::GreenTab green;     // the context's tables
 
     // stored float-float smooth-sum matrices (pm_ffmat.cu, pm_surface_store_ff): the
     // remainder and parametrix entries (6-byte format, row or symmetric tile layout)

@@ -409,7 +409,7 @@ k_self_quad_c(int N, int p, const double* __restrict__ x, const double* __restri
               const double2* __restrict__ c, const double2* __restrict__ qn,
               const int* __restrict__ th_off, const double* __restrict__ th_ang,
               const double* __restrict__ th_w, const double* __restrict__ th_L,
-              const int* __restrict__ row_ptr, double2* __restrict__ WR,
+              const int* __restrict__ row_ptr, pm_green::GreenTab T, double2* __restrict__ WR,
               double2* __restrict__ WK) {
     extern __shared__ double sm[];
     const int pp = p * p;
@@ -481,8 +481,8 @@ k_self_quad_c(int N, int p, const double* __restrict__ x, const double* __restri
                 qi += lu[aa] * zi;
             }
             double out[4];
-            pm_green::pair_rk_cz(-d0, -d1, -d2, n0, n1, n2, Hi, ai, g0, g1, g2, ci,
-                                 pm_green::cplx_d{qr, qi}, cT.g16t, cT.g16w, out);
+            pm_green::pair_rk_tab(-d0, -d1, -d2, n0, n1, n2, Hi, ai, g0, g1, g2, ci,
+                                  pm_green::green_q({qr, qi}), T, cT.g16t, cT.g16w, out);
             const double bw = th_w[kth] * wr * r * jj;
             for (int k = 0; k < 4; ++k) f[k] = bw * out[k];
         } else {
@@ -515,7 +515,7 @@ k_near_quad_c(int p, const double* __restrict__ x, const double* __restrict__ J,
               const double2* __restrict__ c, const double2* __restrict__ qn,
               const int* __restrict__ blk_row, const int* __restrict__ blk_patch,
               const int* __restrict__ row_ptr, double eta, int max_depth, int max_leaves,
-              double2* __restrict__ WR, double2* __restrict__ WK, int* __restrict__ err) {
+              pm_green::GreenTab T, double2* __restrict__ WR, double2* __restrict__ WK, int* __restrict__ err) {
     const int b = blockIdx.x;
     const int i = blk_row[b];
     if (b == row_ptr[i]) return;   // the self block is done by k_self_quad_c
@@ -575,8 +575,8 @@ k_near_quad_c(int p, const double* __restrict__ x, const double* __restrict__ J,
                 for (int cf = 0; cf < 6; ++cf) v5[cf] += l * sZ[(cf * p + aa) * PM_GL16 + r];
             }
             double out[4];
-            pm_green::pair_rk_cz(-v5[0], -v5[1], -v5[2], n0, n1, n2, Hi, ai, g0, g1, g2, ci,
-                                 pm_green::cplx_d{v5[4], v5[5]}, cT.g16t, cT.g16w, out);
+            pm_green::pair_rk_tab(-v5[0], -v5[1], -v5[2], n0, n1, n2, Hi, ai, g0, g1, g2, ci,
+                                  pm_green::green_q({v5[4], v5[5]}), T, cT.g16t, cT.g16w, out);
             const double wgt = hu * cT.g16w[qn_] * hv * cT.g16w[r] * v5[3];
             for (int k = 0; k < 4; ++k) sF[k * kQ2 + e] = wgt * out[k];
         }
@@ -609,8 +609,8 @@ __global__ void k_combine_c(int nblk, int pp, const int* __restrict__ blk_row,
                             const double* __restrict__ n, const double* __restrict__ H,
                             const double* __restrict__ w, const double* __restrict__ a,
                             const double* __restrict__ g, const double2* __restrict__ c,
-                            const double2* __restrict__ qn, double2* __restrict__ CR,
-                            double2* __restrict__ CK) {
+                            const double2* __restrict__ qn, pm_green::GreenTab T,
+                            double2* __restrict__ CR, double2* __restrict__ CK) {
     const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (size_t)nblk * pp) return;
     const int b = (int)(e / pp), k = (int)(e - (size_t)b * pp);
@@ -619,11 +619,11 @@ __global__ void k_combine_c(int nblk, int pp, const int* __restrict__ blk_row,
     const double inv_a = 1.0 / a[j];
     if (j != i) {
         double out[4];
-        pm_green::pair_rk_cz(x[3 * i] - x[3 * j], x[3 * i + 1] - x[3 * j + 1],
-                             x[3 * i + 2] - x[3 * j + 2], n[3 * i], n[3 * i + 1], n[3 * i + 2],
-                             H[i], a[i], g[3 * i], g[3 * i + 1], g[3 * i + 2],
-                             pm_green::cplx_d{c[i].x, c[i].y}, pm_green::cplx_d{qn[j].x, qn[j].y},
-                             cT.g16t, cT.g16w, out);
+        pm_green::pair_rk_tab(x[3 * i] - x[3 * j], x[3 * i + 1] - x[3 * j + 1],
+                              x[3 * i + 2] - x[3 * j + 2], n[3 * i], n[3 * i + 1], n[3 * i + 2],
+                              H[i], a[i], g[3 * i], g[3 * i + 1], g[3 * i + 2],
+                              pm_green::cplx_d{c[i].x, c[i].y},
+                              pm_green::green_q({qn[j].x, qn[j].y}), T, cT.g16t, cT.g16w, out);
         wr.x -= w[j] * out[0];
         wr.y -= w[j] * out[1];
         wk.x -= w[j] * out[2];
@@ -1265,17 +1265,17 @@ pm_status pm_near_build_c(pm_surface* s) {
                                          (int)smem));
     k_self_quad_c<<<N, kQThreads, smem>>>(N, p, s->x, s->J, s->npatch_n, s->H, s->a, s->g, s->cc,
                                           s->qn, s->th_off, s->th_ang, s->th_w, s->th_L,
-                                          s->row_ptr, s->cRc, s->cKc);
+                                          s->row_ptr, s->green, s->cRc, s->cKc);
     PM_CUDA_TRY(cudaGetLastError());
     k_near_quad_c<<<s->nblk, kQThreads>>>(p, s->x, s->J, s->n, s->H, s->a, s->g, s->cc, s->qn,
                                           s->blk_row, s->blk_patch, s->row_ptr, s->opts.near_eta,
                                           std::min(s->opts.near_max_depth, 12),
-                                          s->opts.near_max_leaves, s->cRc, s->cKc, s->dev_err);
+                                          s->opts.near_max_leaves, s->green, s->cRc, s->cKc, s->dev_err);
     PM_CUDA_TRY(cudaGetLastError());
     const size_t ne = (size_t)s->nblk * pp;
     k_combine_c<<<pm_ceil_div((long long)ne, 256), 256>>>(s->nblk, pp, s->blk_row, s->blk_patch,
                                                           s->x, s->n, s->H, s->w, s->a, s->g,
-                                                          s->cc, s->qn, s->cRc, s->cKc);
+                                                          s->cc, s->qn, s->green, s->cRc, s->cKc);
     PM_CUDA_TRY(cudaGetLastError());
     PM_CUDA_TRY(cudaDeviceSynchronize());
     int herr = 0;
