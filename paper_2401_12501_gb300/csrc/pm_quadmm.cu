@@ -33,6 +33,8 @@
 // an SM leaves it idle in the tensor phases.
 #include "pm_quadmm.cuh"
 
+#include "pm_fast64.cuh"
+
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -46,9 +48,6 @@ constexpr int kNT1 = kQmCols * 4 / 8;     // n-tiles of Y (4 fields a column)
 constexpr int kNT2 = kQmCols * 5 / 8;     // n-tiles of W (5 kinds a column)
 constexpr int kFStride = 72;              // words a k-step of an F n-tile (64 + 8: no bank conflicts)
 constexpr int kYStride = kQmPts + 4;      // doubles a row of Y
-
-// reciprocals 1 / (1 + (k + 1/2) / 128) and minus their logarithms (qm_log)
-__device__ double2 g_qm_log[128];
 
 template <int NK>
 struct QmShape {
@@ -93,34 +92,6 @@ __device__ __forceinline__ double fixed_double(long long v, int e) {
     // -(2^52 + 2^31 + 2^20) 2^(32 + e)
     const double off = __hiloint2double((int)0xc3300000 + ((32 + e) << 20), (int)0x80100000);
     return fma(lo, pow2d(e), fma(hi, pow2d(32 + e), off));
-}
-
-// 1 / x: the hardware's approximation (20 bits) and one cubic Newton step
-__device__ __forceinline__ double qm_rcp(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-
-// log x for x = 0 or normal x > 0 by a table (Tang, "Table-driven implementation of the logarithm
-// function in IEEE floating-point arithmetic", ACM TOMS 16, 1990): x = 2^e m, c the tabulated
-// reciprocal next to 1/m, log x = e log 2 - log c + log(1 + t), t = c m - 1, |t| <= 2^-8.
-__device__ __forceinline__ double qm_log(double x) {
-    const int hi = __double2hiint(x);
-    const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(x));
-    const double2 c = g_qm_log[(hi >> 13) & 127];
-    // e + 2^52 + 2^51 exactly, from its bits
-    const double ed = __hiloint2double(0x43380000, (hi >> 20) - 1023) -
-                      ((hi >> 20) < 1023 ? 6755403736023040.0 : 6755399441055744.0);
-    const double t = fma(m, c.x, -1.0);
-    double q = fma(t, 1.0 / 7.0, -1.0 / 6.0);
-    q = fma(t, q, 0.2);
-    q = fma(t, q, -0.25);
-    q = fma(t, q, 1.0 / 3.0);
-    q = fma(t, q, -0.5);
-    const double l = fma(ed, 0.69314718055994530942, c.y) + fma(t * t, q, t);
-    return hi < 0x00100000 ? __hiloint2double((int)0xfff00000, 0) : l;      // x = 0: -infinity
 }
 
 // columns: (target, patch, slot, 1 = own patch)
@@ -246,14 +217,14 @@ k_qm(const int4* __restrict__ items, const int4* __restrict__ cols, const __half
                 const double a = h ? d0.y : d0.x, b = h ? d1.y : d1.x, c = h ? d2.y : d2.x;
                 const double wj = (h ? pw1.x : pw0.x) * (h ? jj.y : jj.x);
                 const double r2 = fma(a, a, fma(b, b, c * c));
-                const double inv = qm_rcp(r2);
+                const double inv = pm_rcp64(r2);
                 const double q = fma(n0, a, fma(n1, b, n2 * c)) * inv;       // -n.r / r^2
                 f[0][h] = wj * (q * (q + Hi));
                 const double gf = wj * inv;
                 f[1][h] = gf * a;                                            // minus the integrand
                 f[2][h] = gf * b;
                 f[3][h] = gf * c;
-                f[4][h] = wj * (qm_log(r2) + (h ? pw1.y : pw0.y));
+                f[4][h] = wj * (pm_log64(r2) + (h ? pw1.y : pw0.y));
             }
         }
         __syncthreads();                              // every warp has read its Y
@@ -385,16 +356,6 @@ __global__ void k_qm_place(int npairs, const int* __restrict__ blocks, const int
     }
 }
 
-pm_status log_table() {
-    double2 t[128];
-    for (int k = 0; k < 128; ++k) {
-        t[k].x = 1.0 / (1.0 + (k + 0.5) / 128.0);
-        t[k].y = -std::log(t[k].x);
-    }
-    PM_CUDA_TRY(cudaMemcpyToSymbol(g_qm_log, t, sizeof(t)));
-    return PM_OK;
-}
-
 template <int NK>
 pm_status launch(const pm_surface* s, int nitems, const int4* items, const int4* cols,
                  const QmTable& T, double* partial) {
@@ -468,7 +429,6 @@ pm_status pm_quad_weights(pm_surface* s, const QmRules& R) {
     }
     float ftop = 0.f;
     std::memcpy(&ftop, &top, sizeof(ftop));
-    PM_TRY(log_table());
     int eB = (int)std::ceil(std::log2(std::min(1e30, std::max(1.0, 3.0 * (double)ftop))));
     for (;; eB += 3) {
         bool over = false;
