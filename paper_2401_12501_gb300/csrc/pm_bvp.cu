@@ -41,8 +41,10 @@
 //   each edge node (pm_nearfield.cu k_bvp_kp_quad: polar rule about the edge point on its
 //   own patch, the quadtree near rule on the others).
 // Everything runs in float64; a solve applies the system through its dense matrix where
-// that fits the device (else pair by pair); the solver is restarted GMRES with classical Gram-Schmidt
-// and one reorthogonalisation, the Hessenberg system on the host.
+// that fits the device (else pair by pair); the solver is restarted GMRES
+// (pm_arnoldi.cuh), the Hessenberg system on the host.
+#include "pm_arnoldi.cuh"
+#include "pm_fast64.cuh"
 #include "pm_internal.cuh"
 
 #include <algorithm>
@@ -71,14 +73,12 @@ struct pm_bvp {
     double *kp_C = nullptr;              // [nblk][pp] K'_Gamma (K_Gamma) corrections
     int kp_nblk = 0;
     double *mu_o = nullptr;              // [Fo]
-    double *part = nullptr;              // dot partials
     cudaStream_t st = nullptr;
 };
 
 namespace {
 
 constexpr int kT = 256;
-constexpr int kDotBlocks = 128;
 constexpr int kTile = 256;
 
 // mu_o[j] = sum_k I_c[j][k] mu[off_c + k] for the curve c of oversampled point j
@@ -131,8 +131,8 @@ __device__ __forceinline__ double edge_pair(const EdgeTarget& t, double y0, doub
                                             double u0, double u1, double u2) {
     const double r0 = t.x[0] - y0, r1 = t.x[1] - y1, r2 = t.x[2] - y2;
     const double rr = r0 * r0 + r1 * r1 + r2 * r2;
-    if (KIND == kEdgeK) return log(rr) * (0.25 / M_PI);
-    const double inv = 1.0 / rr;
+    if (KIND == kEdgeK) return pm_log64(rr) * (0.25 / M_PI);
+    const double inv = pm_rcp64(rr);
     if (KIND == kEdgeN) return -(u0 * r0 + u1 * r1 + u2 * r2) * inv * (0.5 / M_PI);
     const double nr = t.n[0] * r0 + t.n[1] * r1 + t.n[2] * r2;
     if (KIND == kEdgeR) {
@@ -199,7 +199,7 @@ k_bvp_fill_surface(int N, const double* __restrict__ x, const double* __restrict
     for (int r = 0; r < rows; ++r) {
         const double* t = st[r];
         const double r0 = t[0] - y0, r1 = t[1] - y1, r2 = t[2] - y2;
-        const double inv = 1.0 / (r0 * r0 + r1 * r1 + r2 * r2);
+        const double inv = pm_rcp64(r0 * r0 + r1 * r1 + r2 * r2);
         const double nr = t[3] * r0 + t[4] * r1 + t[5] * r2;
         const double mr = t[6] * r0 + t[7] * r1 + t[8] * r2;
         A[(size_t)(i0 + r) * ld + j] = i0 + r == j ? 1.0 : w * inv * (nr * nr * inv + mr);
@@ -274,8 +274,8 @@ __global__ void k_bvp_fill_edge_rows(int dirichlet, int N, int Me, const double*
                      r2 = xe[3 * e + 2] - x[3 * j + 2];
         const double rr = r0 * r0 + r1 * r1 + r2 * r2;
         v = wa[j] * (0.5 / M_PI) *
-            (dirichlet ? 0.5 * log(rr)
-                       : (nue[3 * e] * r0 + nue[3 * e + 1] * r1 + nue[3 * e + 2] * r2) / rr);
+            (dirichlet ? 0.5 * pm_log64(rr)
+                       : (nue[3 * e] * r0 + nue[3 * e + 1] * r1 + nue[3 * e + 2] * r2) * pm_rcp64(rr));
     } else {
         const int k = j - N;
         v = Kpg[(size_t)e * Me + k] + (dirichlet ? 0.0 : we[k]);
@@ -378,44 +378,10 @@ __global__ void k_bvp_axpy(int n, double alpha, const double* __restrict__ xv, d
     if (i < n) y[i] += alpha * xv[i];
 }
 
-// partial[j][b] = sum over block b's share of V[j] . w, j < nv
-__global__ void k_bvp_dots(int n, int nv, const double* __restrict__ V, const double* __restrict__ w,
-                           double* __restrict__ partial) {
-    __shared__ double red[kT / 32];
-    const int j = blockIdx.y;
-    const double* v = V + (size_t)j * n;
-    double acc = 0.0;
-    for (int i = blockIdx.x * kT + threadIdx.x; i < n; i += gridDim.x * kT) acc += v[i] * w[i];
-    const double t = block_sum(acc, red);
-    if (threadIdx.x == 0) partial[(size_t)j * gridDim.x + blockIdx.x] = t;
-}
-
-// w -= sum_j h_j V[j]
-__global__ void k_bvp_sub(int n, int nv, const double* __restrict__ V, const double* __restrict__ h,
-                          double* __restrict__ w) {
+// r = b - r
+__global__ void k_bvp_rsub(int n, const double* __restrict__ b, double* __restrict__ r) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double s = 0.0;
-    for (int j = 0; j < nv; ++j) s += h[j] * V[(size_t)j * n + i];
-    w[i] -= s;
-}
-
-__global__ void k_bvp_scale(int n, double a, const double* __restrict__ xv, double* __restrict__ y) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) y[i] = a * xv[i];
-}
-
-pm_status dots(pm_bvp* b, const double* V, int nv, const double* w, int n, std::vector<double>& out) {
-    dim3 grid(kDotBlocks, nv);
-    k_bvp_dots<<<grid, kT, 0, b->st>>>(n, nv, V, w, b->part);
-    PM_CUDA_TRY(cudaGetLastError());
-    std::vector<double> h((size_t)nv * kDotBlocks);
-    PM_CUDA_TRY(cudaMemcpyAsync(h.data(), b->part, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, b->st));
-    PM_CUDA_TRY(cudaStreamSynchronize(b->st));
-    out.assign(nv, 0.0);
-    for (int j = 0; j < nv; ++j)
-        for (int k = 0; k < kDotBlocks; ++k) out[j] += h[(size_t)j * kDotBlocks + k];
-    return PM_OK;
+    if (i < n) r[i] = b[i] - r[i];
 }
 
 // the system's operator on z = [sigma; mu] (device), out = [surface rows; edge rows]
@@ -505,7 +471,7 @@ void free_bvp(pm_bvp* b) {
     pm_dfree(b->xo); pm_dfree(b->wo); pm_dfree(b->ao); pm_dfree(b->nuo); pm_dfree(b->interp);
     pm_dfree(b->interp_off);
     pm_dfree(b->curve_of); pm_dfree(b->Kpg); pm_dfree(b->kp_ptr); pm_dfree(b->kp_patch);
-    pm_dfree(b->kp_C); pm_dfree(b->kp_edge); pm_dfree(b->mu_o); pm_dfree(b->part);
+    pm_dfree(b->kp_C); pm_dfree(b->kp_edge); pm_dfree(b->mu_o);
     delete b;
 }
 
@@ -620,7 +586,6 @@ pm_status create_impl(pm_bvp* b, const double* edge_x, const double* edge_d1,
     PM_TRY(upload(&b->kp_patch, kp_patch.data(), kp_patch.size()));
     PM_TRY(pm_dmalloc(&b->kp_C, (size_t)b->kp_nblk * pp));
     PM_TRY(pm_dmalloc(&b->mu_o, (size_t)std::max(Fo, 1)));
-    PM_TRY(pm_dmalloc(&b->part, (size_t)kDotBlocks * 128));
     pm_status stt = upload(&b->kp_edge, blk_edge.data(), blk_edge.size());
     if (stt == PM_OK) stt = upload(&d_own, blk_own.data(), blk_own.size());
     if (stt == PM_OK)
@@ -788,16 +753,18 @@ extern "C" pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_ga
     PM_CUDA_TRY(cudaSetDevice(b->s->ctx->device));
     const int n = b->N + b->Me;
     const int m = std::max(2, std::min(b->s->opts.gmres_restart, 120));
-    double *V = nullptr, *w = nullptr, *rhs = nullptr, *x = nullptr, *hd = nullptr, *ud = nullptr;
+    double *V = nullptr, *w = nullptr, *rhs = nullptr, *x = nullptr, *ud = nullptr;
+    pm_arnoldi::Steps<double> steps;
     double* A = nullptr;                 // the system's matrix, where the device has room for it
     pm_status st = pm_dmalloc(&V, (size_t)(m + 1) * n);
     if (st == PM_OK) st = pm_dmalloc(&w, (size_t)n);
     if (st == PM_OK) st = pm_dmalloc(&rhs, (size_t)n);
     if (st == PM_OK) st = pm_dmalloc(&x, (size_t)n);
-    if (st == PM_OK) st = pm_dmalloc(&hd, (size_t)m + 1);
+    if (st == PM_OK) st = steps.create(n, m);
     if (st == PM_OK) st = pm_dmalloc(&ud, (size_t)b->N);
     auto cleanup = [&]() {
-        pm_dfree(V); pm_dfree(w); pm_dfree(rhs); pm_dfree(x); pm_dfree(hd); pm_dfree(ud);
+        pm_dfree(V); pm_dfree(w); pm_dfree(rhs); pm_dfree(x); pm_dfree(ud);
+        steps.release();
         if (A) cudaFreeAsync(A, b->st);
     };
     if (st != PM_OK) { cleanup(); return st; }
@@ -814,10 +781,8 @@ extern "C" pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_ga
         }
     }
     const int grid = pm_ceil_div(n, kT);
-    std::vector<double> d;
-    st = dots(b, rhs, 1, rhs, n, d);
-    if (st != PM_OK) { cleanup(); return st; }
-    const double bnorm = std::sqrt(d[0]);
+    double bnorm = 0.0;
+    if ((st = steps.begin(rhs, V, b->st, &bnorm)) != PM_OK) { cleanup(); return st; }   // x = 0: r = rhs
     int iters = 0;
     double relres = bnorm > 0 ? 1.0 : 0.0;
     std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
@@ -831,37 +796,25 @@ extern "C" pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_ga
         cudaGetLastError();
         if (A && (st = fill_sys(b, A)) != PM_OK) { cleanup(); return st; }
     }
+    double beta = bnorm;
+    // A V_k and its orthogonalisation; through the matrix the next step is started before this
+    // one's coefficients are looked at (the last one in vain)
+    auto step = [&](int k) -> pm_status {
+        PM_TRY(apply_any(b, A, V + (size_t)k * n, w));
+        return steps.step(V, n, k, w, b->st);
+    };
     while (st == PM_OK && bnorm > 0 && relres > tol && iters < maxit) {
-        // r = b - A x
-        st = apply_any(b, A, x, w);
-        if (st != PM_OK) break;
-        k_bvp_scale<<<grid, kT, 0, b->st>>>(n, -1.0, w, w);
-        k_bvp_axpy<<<grid, kT, 0, b->st>>>(n, 1.0, rhs, w);
-        if ((st = dots(b, w, 1, w, n, d)) != PM_OK) break;
-        const double beta = std::sqrt(d[0]);
-        relres = beta / bnorm;
-        if (relres <= tol) break;
-        k_bvp_scale<<<grid, kT, 0, b->st>>>(n, 1.0 / beta, w, V);
         std::fill(g.begin(), g.end(), 0.0);
         g[0] = beta;
-        int k = 0;
+        int k = 0, started = 0;
         for (; k < m && iters < maxit; ++k, ++iters) {
-            double* vk1 = V + (size_t)(k + 1) * n;
-            if ((st = apply_any(b, A, V + (size_t)k * n, vk1)) != PM_OK) break;
-            // classical Gram-Schmidt with one reorthogonalisation
-            std::vector<double> h(k + 1, 0.0);
-            for (int pass = 0; pass < 2 && st == PM_OK; ++pass) {
-                if ((st = dots(b, V, k + 1, vk1, n, d)) != PM_OK) break;
-                for (int j = 0; j <= k; ++j) h[j] += d[j];
-                cudaMemcpyAsync(hd, d.data(), sizeof(double) * (k + 1), cudaMemcpyHostToDevice, b->st);
-                k_bvp_sub<<<grid, kT, 0, b->st>>>(n, k + 1, V, hd, vk1);
-            }
-            if (st != PM_OK) break;
-            if ((st = dots(b, vk1, 1, vk1, n, d)) != PM_OK) break;
-            const double hn = std::sqrt(d[0]);
-            for (int j = 0; j <= k; ++j) H[(size_t)j * m + k] = h[j];
+            if (started == k && (st = step(started++)) != PM_OK) break;
+            if (A && started < m && iters + 1 < maxit && (st = step(started++)) != PM_OK) break;
+            const double* c = nullptr;
+            double hn = 0.0;
+            if ((st = steps.wait(k, &c, &hn)) != PM_OK) break;
+            for (int j = 0; j <= k; ++j) H[(size_t)j * m + k] = c[j] + c[k + 1 + j];
             H[(size_t)(k + 1) * m + k] = hn;
-            if (hn > 0) k_bvp_scale<<<grid, kT, 0, b->st>>>(n, 1.0 / hn, vk1, vk1);
             // Givens rotations
             for (int j = 0; j < k; ++j) {
                 const double a0 = H[(size_t)j * m + k], a1 = H[(size_t)(j + 1) * m + k];
@@ -886,15 +839,12 @@ extern "C" pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_ga
             for (int j = i + 1; j < k; ++j) t -= H[(size_t)i * m + j] * y[j];
             y[i] = t / H[(size_t)i * m + i];
         }
-        for (int j = 0; j < k; ++j) k_bvp_axpy<<<grid, kT, 0, b->st>>>(n, y[j], V + (size_t)j * n, x);
-        if (relres <= tol) {
-            // the true residual confirms the estimate
-            if ((st = apply_any(b, A, x, w)) != PM_OK) break;
-            k_bvp_scale<<<grid, kT, 0, b->st>>>(n, -1.0, w, w);
-            k_bvp_axpy<<<grid, kT, 0, b->st>>>(n, 1.0, rhs, w);
-            if ((st = dots(b, w, 1, w, n, d)) != PM_OK) break;
-            relres = std::sqrt(d[0]) / bnorm;
-        }
+        if (k > 0 && (st = steps.combine(V, n, k, y.data(), x, b->st)) != PM_OK) break;
+        // the true residual r = b - A x
+        if ((st = apply_any(b, A, x, w)) != PM_OK) break;
+        k_bvp_rsub<<<grid, kT, 0, b->st>>>(n, rhs, w);
+        if ((st = steps.begin(w, V, b->st, &beta)) != PM_OK) break;
+        relres = beta / bnorm;
     }
     if (st == PM_OK) st = represent(b, x, ud);
     if (st == PM_OK) {

@@ -13,9 +13,10 @@
 //   - a solve evaluates the pairs once, into dense matrices of both operators (corrections
 //     included) that its Krylov steps stream, where 32 N^2 bytes fit; else the sums above;
 //   - near field: complex corrections from pm_nearfield.cu (pm_near_build_c);
-//   - GMRES(m) with classical Gram-Schmidt applied twice; the Krylov vectors and
-//     the orthogonalisation stay on the device, the (m+1) x m Hessenberg matrix and
-//     its Givens rotations on the host (a few hundred bytes per step).
+//   - GMRES(m) with classical Gram-Schmidt applied twice (pm_arnoldi.cuh); the Krylov
+//     vectors and the orthogonalisation stay on the device, the (m+1) x m Hessenberg
+//     matrix and its Givens rotations on the host (a few hundred bytes per step).
+#include "pm_arnoldi.cuh"
 #include "pm_green.cuh"
 #include "pm_internal.cuh"
 
@@ -225,73 +226,6 @@ __global__ void k_near_apply_c64(int N, int pp, const int* __restrict__ row_ptr,
     if (lane == 0) out[i] = make_double2(re, im);
 }
 
-// ------------------------------------------------------------------ Krylov kernels
-// partial[blk * ncols + j] = sum over the block's rows of conj(V_j[i]) w[i]
-__global__ void __launch_bounds__(kRT)
-k_cdots(const double2* __restrict__ V, long long ldv, int ncols, const double2* __restrict__ w,
-        int N, double2* __restrict__ partial) {
-    __shared__ double2 sh[kRT / 32];
-    const int stride = gridDim.x * blockDim.x;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int j = 0; j < ncols; ++j) {
-        const double2* v = V + j * ldv;
-        double re = 0.0, im = 0.0;
-        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
-            const double2 a = v[i], b = w[i];
-            re += a.x * b.x + a.y * b.y;
-            im += a.x * b.y - a.y * b.x;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            re += __shfl_down_sync(0xffffffffu, re, o);
-            im += __shfl_down_sync(0xffffffffu, im, o);
-        }
-        __syncthreads();
-        if (lane == 0) sh[wid] = make_double2(re, im);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double2 t = make_double2(0.0, 0.0);
-            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-                t.x += sh[k].x;
-                t.y += sh[k].y;
-            }
-            partial[blockIdx.x * ncols + j] = t;
-        }
-    }
-}
-
-// out[j] = sum_blk partial[blk * ncols + j] (fixed order)
-__global__ void k_creduce(const double2* __restrict__ partial, int nblk, int ncols,
-                          double2* __restrict__ out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= ncols) return;
-    double2 s = make_double2(0.0, 0.0);
-    for (int b = 0; b < nblk; ++b) {
-        s.x += partial[b * ncols + j].x;
-        s.y += partial[b * ncols + j].y;
-    }
-    out[j] = s;
-}
-
-// w -= sum_{j < ncols} V_j h_j
-__global__ void k_cupdate(const double2* __restrict__ V, long long ldv, int ncols,
-                          const double2* __restrict__ h, double2* __restrict__ w, int N) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    double2 acc = w[i];
-    for (int j = 0; j < ncols; ++j) {
-        const double2 t = cmul(V[j * ldv + i], h[j]);
-        acc.x -= t.x;
-        acc.y -= t.y;
-    }
-    w[i] = acc;
-}
-
-// out = s * v
-__global__ void k_cscale(const double2* __restrict__ v, double s, double2* __restrict__ out, int N) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) out[i] = make_double2(s * v[i].x, s * v[i].y);
-}
-
 // out = alpha * u + beta * v (real alpha, beta)
 __global__ void k_cadd(const double2* __restrict__ u, double alpha, const double2* __restrict__ v,
                        double beta, double2* __restrict__ out, int N) {
@@ -300,37 +234,29 @@ __global__ void k_cadd(const double2* __restrict__ u, double alpha, const double
         out[i] = make_double2(alpha * u[i].x + beta * v[i].x, alpha * u[i].y + beta * v[i].y);
 }
 
-// x += sum_{j < n} V_j y_j
-__global__ void k_ccombo(const double2* __restrict__ V, long long ldv, int n,
-                         const double2* __restrict__ y, double2* __restrict__ x, int N) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    double2 acc = x[i];
-    for (int j = 0; j < n; ++j) {
-        const double2 t = cmul(V[j * ldv + i], y[j]);
-        acc.x += t.x;
-        acc.y += t.y;
-    }
-    x[i] = acc;
-}
-
 }  // namespace
 
 struct PmHelmWork {
-    int N = 0, m = 0, nred = 0;
+    int N = 0, m = 0;
     double2 *V = nullptr, *w = nullptr, *tmp = nullptr, *x = nullptr, *f = nullptr;
     double2 *r = nullptr, *u = nullptr, *sv = nullptr, *io = nullptr;
-    double2 *part = nullptr, *h = nullptr, *y = nullptr;
-    double2* pinned = nullptr;          // host-pinned [2 (m + 2) + 1]
+    pm_arnoldi::Steps<double2> steps;
+
+    void release_krylov() {
+        pm_dfree(V); pm_dfree(w); pm_dfree(tmp); pm_dfree(x); pm_dfree(f); pm_dfree(r); pm_dfree(u);
+        steps.release();
+        m = 0;
+    }
+    void release() {
+        release_krylov();
+        pm_dfree(sv); pm_dfree(io);
+    }
 };
 
 void pm_helm_free(pm_surface* s) {
     pm_dfree(s->cc); pm_dfree(s->qn); pm_dfree(s->cRc); pm_dfree(s->cKc);
     if (!s->helm) return;
-    PmHelmWork& W = *s->helm;
-    pm_dfree(W.V); pm_dfree(W.w); pm_dfree(W.tmp); pm_dfree(W.x); pm_dfree(W.f); pm_dfree(W.r);
-    pm_dfree(W.u); pm_dfree(W.sv); pm_dfree(W.io); pm_dfree(W.part); pm_dfree(W.h); pm_dfree(W.y);
-    if (W.pinned) cudaFreeHost(W.pinned);
+    s->helm->release();
     delete s->helm;
     s->helm = nullptr;
 }
@@ -346,11 +272,7 @@ pm_status helm_work(pm_surface* s, int m, PmHelmWork** out) {
     const pm_status st = helm_work_alloc(s, m);
     if (st != PM_OK) {
         if (s->helm) {
-            PmHelmWork& W = *s->helm;
-            pm_dfree(W.V); pm_dfree(W.w); pm_dfree(W.tmp); pm_dfree(W.x); pm_dfree(W.f);
-            pm_dfree(W.r); pm_dfree(W.u); pm_dfree(W.sv); pm_dfree(W.io); pm_dfree(W.part);
-            pm_dfree(W.h); pm_dfree(W.y);
-            if (W.pinned) cudaFreeHost(W.pinned);
+            s->helm->release();
             delete s->helm;
             s->helm = nullptr;
         }
@@ -370,12 +292,8 @@ pm_status helm_work_alloc(pm_surface* s, int m) {
         PM_TRY(pm_dmalloc(&W.io, 2 * (size_t)N));
     }
     if (m > 0 && W.m != m) {
-        pm_dfree(W.V); pm_dfree(W.w); pm_dfree(W.tmp); pm_dfree(W.x); pm_dfree(W.f);
-        pm_dfree(W.r); pm_dfree(W.u); pm_dfree(W.part); pm_dfree(W.h); pm_dfree(W.y);
-        if (W.pinned) cudaFreeHost(W.pinned);
-        W.pinned = nullptr;
+        W.release_krylov();
         W.m = m;
-        W.nred = std::max(1, std::min(pm_ceil_div(N, 4 * kRT), 2 * s->ctx->num_sms));
         PM_TRY(pm_dmalloc(&W.V, (size_t)(m + 1) * N));
         PM_TRY(pm_dmalloc(&W.w, N));
         PM_TRY(pm_dmalloc(&W.tmp, N));
@@ -383,10 +301,7 @@ pm_status helm_work_alloc(pm_surface* s, int m) {
         PM_TRY(pm_dmalloc(&W.f, N));
         PM_TRY(pm_dmalloc(&W.r, N));
         PM_TRY(pm_dmalloc(&W.u, N));
-        PM_TRY(pm_dmalloc(&W.part, (size_t)W.nred * (m + 2)));
-        PM_TRY(pm_dmalloc(&W.h, 2 * (size_t)(m + 2) + 1));
-        PM_TRY(pm_dmalloc(&W.y, m + 1));
-        PM_CUDA_TRY(cudaMallocHost((void**)&W.pinned, sizeof(double2) * (2 * (size_t)(m + 2) + 1)));
+        PM_TRY(W.steps.create(N, m));
     }
     return PM_OK;
 }
@@ -473,22 +388,6 @@ struct HelmSolver {
         k_dense_c64<<<pm_ceil_div(W.N, kGemvRowsC), kHT, 0, st>>>(M, v, add, W.N, out);
         PM_CUDA_TRY(cudaGetLastError());
         s->launch_total++;
-        return PM_OK;
-    }
-
-    // dst[0..ncols) = V_j^H b on the device
-    pm_status dots(const double2* V, long long ldv, int ncols, const double2* b, double2* dst) {
-        k_cdots<<<W.nred, kRT, 0, st>>>(V, ldv, ncols, b, W.N, W.part);
-        k_creduce<<<pm_ceil_div(ncols, 64), 64, 0, st>>>(W.part, W.nred, ncols, dst);
-        PM_CUDA_TRY(cudaGetLastError());
-        return PM_OK;
-    }
-
-    pm_status norm(const double2* v, double* out) {
-        PM_TRY(dots(v, 0, 1, v, W.h));
-        PM_CUDA_TRY(cudaMemcpyAsync(W.pinned, W.h, sizeof(double2), cudaMemcpyDeviceToHost, st));
-        PM_CUDA_TRY(cudaStreamSynchronize(st));
-        *out = std::sqrt(std::max(0.0, W.pinned[0].x));
         return PM_OK;
     }
 
@@ -621,46 +520,39 @@ extern "C" pm_status pm_solve_c(pm_surface* s, const double* f, double* u, doubl
     PM_CUDA_TRY(cudaMemcpyAsync(W.f, f, bytes, cudaMemcpyHostToDevice, st));
     PM_CUDA_TRY(cudaMemsetAsync(W.x, 0, bytes, st));
     double fnorm = 0.0;
-    PM_TRY(S.norm(W.f, &fnorm));
+    PM_TRY(W.steps.begin(W.f, W.V, st, &fnorm));          // x = 0: the first residual is f
     int iters = 0, cycles = 0;
     double relres = 0.0;
     pm_status result = PM_OK;
     if (fnorm > 0.0) {
         PM_TRY(S.D.fill(s));
-        PM_CUDA_TRY(cudaMemcpyAsync(W.r, W.f, bytes, cudaMemcpyDeviceToDevice, st));
         std::vector<cplx> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
         const long long ldv = N;
+        // A V_k and its orthogonalisation.  Through the matrix the next step is started before
+        // this one's coefficients are looked at (the last one in vain); pair by pair it is not
+        auto step = [&](int k) -> pm_status {
+            PM_TRY(S.apply_A(W.V + (size_t)k * ldv, W.w));
+            return W.steps.step(W.V, ldv, k, W.w, st);
+        };
+        double beta = fnorm;
         for (;;) {
-            double beta = 0.0;
-            PM_TRY(S.norm(W.r, &beta));
             relres = beta / fnorm;
             if (relres <= tol || iters >= maxit) break;
-            // one cycle of GMRES(m) on A d = r, x += d
-            k_cscale<<<S.grid, kRT, 0, st>>>(W.r, 1.0 / beta, W.V, N);
+            // one cycle of GMRES(m) on A d = r, x += d; V_0 = r / |r|
             std::fill(g.begin(), g.end(), cplx(0.0));
             g[0] = beta;
-            int k = 0;
+            int k = 0, started = 0;
             for (; k < m && iters < maxit; ++k) {
-                double2* vk = W.V + (size_t)k * ldv;
-                PM_TRY(S.apply_A(vk, W.w));
-                // classical Gram-Schmidt, twice: h = V^H w, w -= V h; h2 = V^H w, w -= V h2
-                PM_TRY(S.dots(W.V, ldv, k + 1, W.w, W.h));
-                k_cupdate<<<S.grid, kRT, 0, st>>>(W.V, ldv, k + 1, W.h, W.w, N);
-                PM_TRY(S.dots(W.V, ldv, k + 1, W.w, W.h + (m + 2)));
-                k_cupdate<<<S.grid, kRT, 0, st>>>(W.V, ldv, k + 1, W.h + (m + 2), W.w, N);
-                PM_TRY(S.dots(W.w, 0, 1, W.w, W.h + 2 * (m + 2)));
-                PM_CUDA_TRY(cudaMemcpyAsync(W.pinned, W.h, sizeof(double2) * (2 * (size_t)(m + 2) + 1),
-                                            cudaMemcpyDeviceToHost, st));
-                PM_CUDA_TRY(cudaStreamSynchronize(st));
-                const double hn = std::sqrt(std::max(0.0, W.pinned[2 * (m + 2)].x));
+                if (started == k) PM_TRY(step(started++));
+                if (S.D.MR && started < m && iters + 1 < maxit) PM_TRY(step(started++));
+                const double2* c = nullptr;
+                double hn = 0.0;
+                PM_TRY(W.steps.wait(k, &c, &hn));
                 cplx* col = &H[(size_t)k * (m + 1)];
                 for (int j = 0; j <= k; ++j)
-                    col[j] = cplx(W.pinned[j].x + W.pinned[m + 2 + j].x,
-                                  W.pinned[j].y + W.pinned[m + 2 + j].y);
+                    col[j] = cplx(c[j].x + c[k + 1 + j].x, c[j].y + c[k + 1 + j].y);
                 col[k + 1] = hn;
                 ++iters;
-                if (hn > 0.0)
-                    k_cscale<<<S.grid, kRT, 0, st>>>(W.w, 1.0 / hn, W.V + (size_t)(k + 1) * ldv, N);
                 // the earlier rotations, then a new one that zeroes col[k + 1]:
                 // [c s; -conj(s) c] [a; b] = [rho; 0], c = |a|/t, s = (a/|a|) conj(b)/t
                 for (int j = 0; j < k; ++j) {
@@ -697,14 +589,13 @@ extern "C" pm_status pm_solve_c(pm_surface* s, const double* f, double* u, doubl
                 const cplx d = H[(size_t)i * (m + 1) + i];
                 y[i] = (std::abs(d) > 0.0) ? t / d : cplx(0.0);
             }
-            for (int i = 0; i < k; ++i) W.pinned[i] = make_double2(y[i].real(), y[i].imag());
-            PM_CUDA_TRY(cudaMemcpyAsync(W.y, W.pinned, sizeof(double2) * k, cudaMemcpyHostToDevice, st));
-            k_ccombo<<<S.grid, kRT, 0, st>>>(W.V, ldv, k, W.y, W.x, N);
-            PM_CUDA_TRY(cudaGetLastError());
+            std::vector<double2> yd(k);
+            for (int i = 0; i < k; ++i) yd[i] = make_double2(y[i].real(), y[i].imag());
+            if (k > 0) PM_TRY(W.steps.combine(W.V, ldv, k, yd.data(), W.x, st));
             ++cycles;
             PM_TRY(S.residual());            // the true residual of the new x
+            PM_TRY(W.steps.begin(W.r, W.V, st, &beta));
             if (k == 0) {
-                PM_TRY(S.norm(W.r, &beta));
                 relres = beta / fnorm;
                 break;
             }
