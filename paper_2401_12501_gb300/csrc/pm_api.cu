@@ -693,7 +693,9 @@ pm_status pm_apply_dev(pm_surface* s, int kernel_K, int smooth, int near, const 
                        double* out, pm_precision prec, cudaStream_t st, int prepped) {
     int nsplit = 0;
     prepped = prepped && (prec == PM_PREC_FP32 || prec == PM_PREC_FMM);
-    if ((smooth || near) && !prepped) {
+    // float32 sums on small surfaces form the strengths themselves
+    const bool fresh = !prepped && smooth && prec == PM_PREC_FP32 && pm_direct_fresh(s);
+    if ((smooth || near) && !prepped && !fresh) {
         PhaseTimer t(s, PM_PHASE_PREP, st);
         if (prec == PM_PREC_FF && pm_ffmat_has(s, kernel_K)) {
             PM_TRY(pm_ffmat_prep(s, sigma, st));
@@ -721,11 +723,11 @@ pm_status pm_apply_dev(pm_surface* s, int kernel_K, int smooth, int near, const 
             PM_TRY(pm_fmm_apply(s, kernel_K, st));
         } else {
             nsplit = pm_direct_splits(s, prec, kernel_K);
-            PM_TRY(pm_direct_sum(s, kernel_K, prec, nsplit, st));
+            PM_TRY(pm_direct_sum(s, kernel_K, prec, nsplit, st, fresh ? sigma : nullptr));
         }
     }
     PhaseTimer t(s, PM_PHASE_NEAR, st);
-    s->launch_total += ((smooth || near) && !prepped) + (smooth && prec != PM_PREC_FMM) + 1;
+    s->launch_total += ((smooth || near) && !prepped && !fresh) + (smooth && prec != PM_PREC_FMM) + 1;
     return pm_near_apply(s, kernel_K, sigma, out, near, nsplit,
                          prec == PM_PREC_FMM ? PM_PREC_FP32 : prec, st);
 }

@@ -66,6 +66,29 @@ __global__ void k_prep32(const double* __restrict__ sigma, const double* __restr
     sig32[(size_t)P * ppad + (j - P * pp)] = (float)sg;
 }
 
+// Strengths formed where the sums stage their sources, from the density itself (sigma null: src
+// holds them, k_prep32).  One launch less an apply: 2.5-3 us of host time and as much of the
+// device's, against a multiplication and a conversion on the float64 pipe for every source a
+// block stages, about 3 % of the sums.  Worth it up to kFreshNodes.  The first block column
+// leaves sig32 for the near field.
+constexpr int kFreshNodes = 16384;
+struct Fresh {
+    const double *sigma = nullptr, *wa = nullptr;
+    float* sig32 = nullptr;
+    int pp = 1, ppad = 1;
+};
+__device__ __forceinline__ float4 fresh_source(const Fresh& F, float4 v, int j) {
+    if (F.sigma) {
+        const double sg = F.sigma[j];
+        v.w = (float)(F.wa[j] * sg);
+        if (blockIdx.x == 0) {
+            const int P = j / F.pp;
+            F.sig32[(size_t)P * F.ppad + (j - P * F.pp)] = (float)sg;
+        }
+    }
+    return v;
+}
+
 __global__ void k_prep64(const double* __restrict__ sigma, const double* __restrict__ wa,
                          pm_d4* __restrict__ src, int N, const int* __restrict__ skip) {
     if (skip && *skip) return;
@@ -113,7 +136,7 @@ constexpr int kStage = 1024;
 template <int TPT>
 __global__ void __launch_bounds__(kThreads)
 k_direct_R32(const float4* __restrict__ src, const float4* __restrict__ tgt, int N, int chunk,
-             float eps2, float2* __restrict__ partial, const int* __restrict__ skip) {
+             float eps2, float2* __restrict__ partial, const int* __restrict__ skip, Fresh fresh) {
     if (skip && *skip) return;
     __shared__ float4 sh[kStage];
     const int tid = threadIdx.x;
@@ -139,7 +162,7 @@ k_direct_R32(const float4* __restrict__ src, const float4* __restrict__ tgt, int
     for (int base = s0; base < s1; base += kStage) {
         const int len = min(kStage, s1 - base);
         __syncthreads();
-        for (int j = tid; j < len; j += kThreads) sh[j] = src[base + j];
+        for (int j = tid; j < len; j += kThreads) sh[j] = fresh_source(fresh, src[base + j], base + j);
         __syncthreads();
         for (int j0 = 0; j0 < len; j0 += kTile) {
             const int j1 = min(j0 + kTile, len);
@@ -193,7 +216,7 @@ k_direct_R32(const float4* __restrict__ src, const float4* __restrict__ tgt, int
 template <int TPT, bool CENTRED>
 __global__ void __launch_bounds__(kThreads)
 k_direct_K32(const float4* __restrict__ src, const float4* __restrict__ tgt, int N, int chunk,
-             float2* __restrict__ partial, const int* __restrict__ skip) {
+             float2* __restrict__ partial, const int* __restrict__ skip, Fresh fresh) {
     if (skip && *skip) return;
     __shared__ float4 sh[kStage];
     __shared__ float sb2[CENTRED ? kStage : 1];
@@ -254,7 +277,7 @@ k_direct_K32(const float4* __restrict__ src, const float4* __restrict__ tgt, int
         const int len = min(kStage, s1 - base);
         __syncthreads();
         for (int j = tid; j < len; j += kThreads) {
-            const float4 v = src[base + j];
+            const float4 v = fresh_source(fresh, src[base + j], base + j);
             if (CENTRED) {
                 const float bx = v.x - cx, by = v.y - cy, bz = v.z - cz;
                 sh[j] = make_float4(-2.f * bx, -2.f * by, -2.f * bz, v.w);
@@ -405,9 +428,21 @@ pm_status pm_prep_sources(pm_surface* s, const double* sigma, pm_precision prec,
     return PM_OK;
 }
 
+// May this float32 sum form its strengths itself?
+bool pm_direct_fresh(const pm_surface* s) { return s->N <= kFreshNodes; }
+
+// sigma: float32 strengths are formed from it (pm_direct_fresh); null: they are in s->src32
 pm_status pm_direct_sum(pm_surface* s, int which_K, pm_precision prec, int nsplit,
-                        cudaStream_t st) {
+                        cudaStream_t st, const double* sigma) {
     const int N = s->N;
+    Fresh fresh;
+    if (sigma) {
+        fresh.sigma = sigma;
+        fresh.wa = s->wa;
+        fresh.sig32 = s->sig32;
+        fresh.pp = s->pp;
+        fresh.ppad = s->ppad;
+    }
     if (prec == PM_PREC_FP64) {
         const int chunk = pm_ceil_div(pm_ceil_div(s->Npad, nsplit), 8) * 8;
         dim3 grid(pm_ceil_div(N, kThreads), nsplit);
@@ -421,10 +456,10 @@ pm_status pm_direct_sum(pm_surface* s, int which_K, pm_precision prec, int nspli
 #define PM_LAUNCH(T)                                                                        \
         if (which_K)                                                                        \
             (s->k32_centred ? k_direct_K32<T, true> : k_direct_K32<T, false>)               \
-                <<<grid, kThreads, 0, st>>>(s->src32, s->tgt32, N, chunk, part, s->skip_flag); \
+                <<<grid, kThreads, 0, st>>>(s->src32, s->tgt32, N, chunk, part, s->skip_flag, fresh); \
         else                                                                                \
             k_direct_R32<T><<<grid, kThreads, 0, st>>>(s->src32, s->tgt32, N, chunk,        \
-                                                       s->eps2, part, s->skip_flag);
+                                                       s->eps2, part, s->skip_flag, fresh);
         if (tpt == 1) { PM_LAUNCH(1) } else if (tpt == 4) { PM_LAUNCH(4) } else { PM_LAUNCH(2) }
 #undef PM_LAUNCH
     }
@@ -551,7 +586,7 @@ extern "C" pm_status pm_smooth_remainder_f32_noalloc(int N, const float* x, cons
     // forms (1/r^2) * 0 before multiplying by the strength) while r^2 = 1e-30 keeps
     // 1/r^2 finite; 1e-30 is far below the squared distance of any two distinct nodes
     const float eps2 = 1e-30f;
-    k_direct_R32<2><<<grid, kThreads, 0, st>>>(src, tgt, N, chunk, eps2, part, nullptr);
+    k_direct_R32<2><<<grid, kThreads, 0, st>>>(src, tgt, N, chunk, eps2, part, nullptr, Fresh{});
     k_noalloc_reduce<<<pm_ceil_div(N, 256), 256, 0, st>>>(N, nsplit, part, out);
     PM_CUDA_TRY(cudaGetLastError());
     return PM_OK;

@@ -288,7 +288,8 @@ int pm_direct_splits(const pm_surface* s, pm_precision prec, int which_K);
 pm_status pm_prep_sources(pm_surface* s, const double* sigma, pm_precision prec,
                           cudaStream_t st);
 pm_status pm_direct_sum(pm_surface* s, int which_K, pm_precision prec, int nsplit,
-                        cudaStream_t st);
+                        cudaStream_t st, const double* sigma = nullptr);
+bool pm_direct_fresh(const pm_surface* s);
 pm_status pm_pack_targets(pm_surface* s, cudaStream_t st);
 
 // float-float sums (pm_ffsum.cu)
