@@ -30,7 +30,14 @@ def _f64(a, n):
 
 
 def _is_device(a) -> bool:
-    return hasattr(a, "is_cuda") and a.is_cuda
+    return getattr(a, "is_cuda", False)
+
+
+def _torch():
+    global _torch
+    import torch
+    _torch = lambda: torch           # noqa: E731  (the import's lookup once)
+    return torch
 
 
 class Context:
@@ -264,25 +271,33 @@ class Surface:
 
     def _apply(self, fn, args, sigma, prec, stream, out=None):
         prec = PRECISIONS[prec] if isinstance(prec, str) else int(prec)
-        dev = _is_device(sigma)
-        if dev:
-            import torch
-            if sigma.dtype != torch.float64 or not sigma.is_contiguous():
+        if _is_device(sigma):
+            # the smallest applies take less time on the device than a call through here, so
+            # this path makes no objects but the result: addresses go to ctypes as integers
+            torch = _torch()
+            if sigma.dtype is not torch.float64 or not sigma.is_contiguous():
                 raise ValueError("device sigma must be a contiguous float64 tensor")
-            nrhs = sigma.numel() // self.N
+            n = sigma.numel()
+            nrhs = n // self.N
+            if nrhs * self.N != n:
+                raise ValueError("sigma size is not a multiple of N")
             if out is None:
                 out = torch.empty_like(sigma)
-            st = C.c_void_p(stream if stream is not None else
-                            torch.cuda.current_stream(sigma.device).cuda_stream)
+                to = out.data_ptr()
+            else:
+                to = ptr(out)
+            if stream is None:
+                stream = torch.cuda.current_stream(sigma.device).cuda_stream
+            status = fn(self.handle, *args, sigma.data_ptr(), to, nrhs, prec, 1, stream)
         else:
             sigma = np.ascontiguousarray(sigma, dtype=np.float64)
             nrhs = sigma.size // self.N
             out = np.empty_like(sigma) if out is None else out
-            st = C.c_void_p(stream)
-        if nrhs * self.N != (sigma.numel() if dev else sigma.size):
-            raise ValueError("sigma size is not a multiple of N")
-        check(fn(self.handle, *args, ptr(sigma), ptr(out), nrhs, prec, 1 if dev else 0, st),
-              fn.__name__)
+            if nrhs * self.N != sigma.size:
+                raise ValueError("sigma size is not a multiple of N")
+            status = fn(self.handle, *args, ptr(sigma), ptr(out), nrhs, prec, 0, stream)
+        if status:
+            check(status, fn.__name__)
         return out
 
     def apply_R(self, sigma, prec="fp32", stream=None, out=None):
