@@ -431,6 +431,7 @@ struct PmBatchWork {
     int *pu_ptr = nullptr, *pu_list = nullptr, *blk_u = nullptr;
     int umax = 0;
     bool patch_tried = false;
+    PmFfmmWork fm;             // float-float sums on the tensor cores
 };
 
 void pm_batch_free(pm_surface* s) {
@@ -442,6 +443,7 @@ void pm_batch_free(pm_surface* s) {
     pm_dfree(s->batch->pu_ptr);
     pm_dfree(s->batch->pu_list);
     pm_dfree(s->batch->blk_u);
+    pm_ffmm_free(&s->batch->fm);
     delete s->batch;
     s->batch = nullptr;
 }
@@ -476,6 +478,27 @@ static int batch_splits(const pm_surface* s, int nrhs, int rb, int bps) {
     const int want = bps * s->ctx->num_sms;
     int ns = (want + tblocks / 2) / tblocks;
     return std::max(1, std::min(ns, std::min(8, std::max(1, s->N / 256))));
+}
+
+// Float-float sums of this many columns and more go to the tensor cores (pm_ffmm.cu): there a
+// pair costs about the same from 1 to 64 columns, in k_direct_multi_ff 12 instructions a column.
+constexpr int kFfmmMin = 8;
+
+// Source splits of the tensor-core sums, one block an SM: the split whose blocks of `targets`
+// rows fill whole rounds best.
+static int ffmm_splits(const pm_surface* s, int targets) {
+    const long long tb = pm_ceil_div(s->N, targets);
+    int best = 1;
+    long long cost = 0;
+    for (int ns = 1; ns <= 8; ++ns) {
+        const long long c = (long long)pm_ceil_div(tb * ns, s->ctx->num_sms) *
+                            (pm_ceil_div(pm_ceil_div(s->N, ns), 128) + 2);
+        if (ns == 1 || c < cost) {
+            best = ns;
+            cost = c;
+        }
+    }
+    return best;
 }
 
 // Near-patch unions of every patch (see k_near_multi32_patch); umax = 0 when the
@@ -537,12 +560,21 @@ pm_status pm_apply_batch(pm_surface* s, int kernel_K, const double* sigma, long 
         // 8 right-hand sides per block when the batch has no more: the per-RHS
         // float-float work runs over every slot of a block
         const int rbff = nrhs <= 8 ? 8 : kRBff;
-        const int ns = batch_splits(s, nrhs, rbff, 8);
-        {
+        int ns = ffmm_splits(s, 64);
+        bool summed = false;
+        if (nrhs >= kFfmmMin) {
+            PhaseTimer t(s, kernel_K ? PM_PHASE_DIRECT64_K : PM_PHASE_DIRECT64, st);
+            const pm_status r = pm_ffmm_sum(s, &B.fm, kernel_K ? PM_FFMM_K : PM_FFMM_R, 1, &s, &nrhs,
+                                            &sigma, ld_sigma, ns, B.part, st);
+            if (r != PM_OK && r != PM_ERR_OOM) return r;      // no room for its buffers: as below
+            summed = r == PM_OK;
+        }
+        if (!summed) ns = batch_splits(s, nrhs, rbff, 8);
+        if (!summed) {
             PhaseTimer t(s, PM_PHASE_PREP, st);
             k_prep_ff_multi<<<gp, 256, 0, st>>>(sigma, ld_sigma, s->wa, B.sff, N, skip);
         }
-        {
+        if (!summed) {
             PhaseTimer t(s, kernel_K ? PM_PHASE_DIRECT64_K : PM_PHASE_DIRECT64, st);
             dim3 g(pm_ceil_div(N, kThreads), ns, pm_ceil_div(nrhs, rbff));
             const int chunk = pm_ceil_div(N, ns);
@@ -2011,23 +2043,35 @@ pm_status multi_representation_ff(pm_surface* const* ops, int nops, const int* n
             PmBatchWork& B = *s0->batch;
             const int N = s0->N;
             const int rbff = cols <= 8 ? 8 : kRBff;
-            const int ns = batch_splits(s0, cols, rbff, 8);
-            int c = 0;
-            for (int q = k; q < k1; ++q) {
-                k_prep_ff_multi<<<dim3(pm_ceil_div(N, 256), nrhs[q]), 256, 0, st>>>(
-                    sig + (size_t)(c0 + c) * ld, ld, ops[q]->wa, B.sff + (size_t)c * N, N, nullptr);
-                c += nrhs[q];
+            int ns = ffmm_splits(s0, 64), c = 0;
+            bool summed = false;
+            if (cols >= kFfmmMin) {
+                std::vector<const double*> sg;
+                for (int q = k; q < k1; c += nrhs[q++]) sg.push_back(sig + (size_t)(c0 + c) * ld);
+                const pm_status r = pm_ffmm_sum(s0, &B.fm, PM_FFMM_K, k1 - k, ops + k, nrhs + k, sg.data(),
+                                                ld, ns, B.part, st);
+                if (r != PM_OK && r != PM_ERR_OOM) return r;
+                summed = r == PM_OK;
             }
-            const dim3 g(pm_ceil_div(N, kThreads), ns, pm_ceil_div(cols, rbff));
-            const int chunk = pm_ceil_div(N, ns);
-            if (rbff == 8)
-                k_direct_multi_ff<true, 8><<<g, kThreads, 0, st>>>(s0->src_kg, B.sff, cols, s0->tgt_ff,
-                                                                  s0->log_tab, N, chunk, B.part, ns,
-                                                                  nullptr);
-            else
-                k_direct_multi_ff<true, kRBff><<<g, kThreads, 0, st>>>(s0->src_kg, B.sff, cols,
-                                                                      s0->tgt_ff, s0->log_tab, N,
-                                                                      chunk, B.part, ns, nullptr);
+            if (!summed) {
+                ns = batch_splits(s0, cols, rbff, 8);
+                c = 0;
+                for (int q = k; q < k1; ++q) {
+                    k_prep_ff_multi<<<dim3(pm_ceil_div(N, 256), nrhs[q]), 256, 0, st>>>(
+                        sig + (size_t)(c0 + c) * ld, ld, ops[q]->wa, B.sff + (size_t)c * N, N, nullptr);
+                    c += nrhs[q];
+                }
+                const dim3 g(pm_ceil_div(N, kThreads), ns, pm_ceil_div(cols, rbff));
+                const int chunk = pm_ceil_div(N, ns);
+                if (rbff == 8)
+                    k_direct_multi_ff<true, 8><<<g, kThreads, 0, st>>>(s0->src_kg, B.sff, cols, s0->tgt_ff,
+                                                                      s0->log_tab, N, chunk, B.part, ns,
+                                                                      nullptr);
+                else
+                    k_direct_multi_ff<true, kRBff><<<g, kThreads, 0, st>>>(s0->src_kg, B.sff, cols,
+                                                                          s0->tgt_ff, s0->log_tab, N,
+                                                                          chunk, B.part, ns, nullptr);
+            }
             c = 0;
             for (int q = k; q < k1; ++q) {
                 const dim3 gn(pm_ceil_div((long long)N * 32, 256), nrhs[q]);
@@ -2042,6 +2086,53 @@ pm_status multi_representation_ff(pm_surface* const* ops, int nops, const int* n
             PM_CUDA_TRY(cudaGetLastError());
         }
         c0 += cols;
+        k = k1;
+    }
+    return PM_OK;
+}
+
+// R~ sigma (float-float) of the instances marked in `which`.  Consecutive ones on one geometry
+// share the tensor-core sum of the four coefficient-free matrices (pm_ffmm.cu RG) from kRGMin
+// operators on; fewer take one matrix each (24,576 nodes: 24.4 ms against 5.2 ms an operator of 8
+// columns).
+constexpr int kRGMin = 5;
+pm_status multi_remainder_ff(pm_surface* const* ops, int nops, const int* nrhs,
+                             const std::vector<int>& which, const double* sig, double* out,
+                             long long ld, cudaStream_t st) {
+    std::vector<int> col(nops + 1, 0);
+    for (int k = 0; k < nops; ++k) col[k + 1] = col[k] + nrhs[k];
+    for (int k = 0; k < nops;) {
+        if (!which[k]) {
+            ++k;
+            continue;
+        }
+        int k1 = k + 1;
+        while (k1 < nops && which[k1] && ops[k1]->x == ops[k]->x) ++k1;
+        pm_surface* s0 = ops[k];
+        bool summed = false;
+        if (k1 - k >= kRGMin) {
+            PM_TRY(batch_ensure(s0, col[k1] - col[k]));
+            PmBatchWork& B = *s0->batch;
+            const int ns = ffmm_splits(s0, 16);
+            std::vector<const double*> sg;
+            for (int q = k; q < k1; ++q) sg.push_back(sig + (size_t)col[q] * ld);
+            const pm_status r = pm_ffmm_sum(s0, &B.fm, PM_FFMM_RG, k1 - k, ops + k, nrhs + k, sg.data(), ld,
+                                            ns, B.part, st);
+            if (r != PM_OK && r != PM_ERR_OOM) return r;
+            summed = r == PM_OK;
+            for (int q = k; summed && q < k1; ++q) {
+                const dim3 gn(pm_ceil_div((long long)s0->N * 32, 256), nrhs[q]);
+                k_near_multi64<<<gn, 256, 0, st>>>(
+                    s0->N, ops[q]->pp, ops[q]->row_ptr, ops[q]->blk_patch, ops[q]->cR64,
+                    sig + (size_t)col[q] * ld, ld, B.part + (size_t)(col[q] - col[k]) * ns * s0->N, ns,
+                    out + (size_t)col[q] * ld, ld, nullptr);
+                s0->launch_total++;
+            }
+            PM_CUDA_TRY(cudaGetLastError());
+        }
+        for (int q = k; !summed && q < k1; ++q)
+            PM_TRY(pm_apply_batch(ops[q], 0, sig + (size_t)col[q] * ld, ld, out + (size_t)col[q] * ld, ld,
+                                  nrhs[q], PM_PREC_FF, st));
         k = k1;
     }
     return PM_OK;
@@ -2175,13 +2266,7 @@ extern "C" pm_status pm_solve_multi(pm_surface* const* ops, int nops, const int*
             k_bsubv<<<dim3(S.grid_n, nc), 256, 0, st>>>(W.res, W.w, N);
             S.launches += 1;
             if (any_exact) {
-                c0 = 0;
-                for (int k = 0; k < nops; ++k) {
-                    if (exact[k])
-                        PM_TRY(pm_apply_batch(ops[k], 0, W.sig + (size_t)c0 * N, N,
-                                              W.tmp + (size_t)c0 * N, N, nrhs[k], PM_PREC_FF, st));
-                    c0 += nrhs[k];
-                }
+                PM_TRY(multi_remainder_ff(ops, nops, nrhs, exact, W.sig, W.tmp, N, st));
                 S.dots(M.wcol, 0, N, 1, W.sig, N, W.dots + 0, 8, nullptr);
                 c0 = 0;
                 for (int k = 0; k < nops; ++k) {

@@ -307,6 +307,21 @@ pm_status pm_ffmat_refresh(pm_surface* s, cudaStream_t st);
 pm_status pm_ffmat_prep(pm_surface* s, const double* sigma, cudaStream_t st);
 pm_status pm_ffmat_apply(pm_surface* s, int which_K, int* nsplit, cudaStream_t st);
 
+// float-float sums of many right-hand sides on the tensor cores (pm_ffmm.cu)
+constexpr int PM_FFMM_OPS = 16;
+enum { PM_FFMM_K = 0, PM_FFMM_R = 1, PM_FFMM_RG = 2 };
+struct PmFfmmWork {
+    unsigned int* S = nullptr;      // the strengths' digits
+    int* top = nullptr;             // per column: exponent of the largest strength
+    unsigned int* bound = nullptr;  // the geometry's largest kernel values by target
+};
+void pm_ffmm_free(PmFfmmWork* W);
+// partial[(column nsplit + split) N + i] for the columns of ops[0..nops) (all on s's geometry;
+// PM_FFMM_R: one operator), sigma[q] + r ld operator q's column r
+pm_status pm_ffmm_sum(pm_surface* s, PmFfmmWork* W, int kind, int nops, pm_surface* const* ops,
+                      const int* ncols, const double* const* sigma, long long ld, int nsplit,
+                      float2* partial, cudaStream_t st);
+
 // free device memory now (cudaMemGetInfo), or the value of the environment variable
 // PM_FAKE_HBM_BYTES when set (a host-side stand-in for a full device) (pm_api.cu)
 size_t pm_free_hbm_bytes();
