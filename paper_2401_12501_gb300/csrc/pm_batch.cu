@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 namespace {
@@ -1327,17 +1328,23 @@ struct MGroup {                // instances on one geometry (a surface and its c
 // persistent float32 remainder sums sharing each pair's geometry across the
 // coefficient fields of a geometry: block b takes items b, b + gridDim.x, ...;
 // item = (group, target tile, source chunk, block of FB fields x RB right-hand sides).
-// Per pair: r, 1/r^2, n.r and (n.r)^2 / r^2 once; per field A, B, g; per right-hand
-// side one FMA.
+// With q = n.r / r^2, field k's remainder is a_k/pi times q (q - H) + g_k' . r / r^2,
+// g_k' = grad a_k / (2 a_k): q (q - H) and r / r^2 once a pair (15 operations), three FMAs a field,
+// one a right-hand side; a_k/pi multiplies the finished sums.  Bound by the FMA pipe: 59
+// operations for 4 fields x 8 right-hand sides, where A, B and g in the pair cost 78 in
+// two halves of 2 fields (24,576 nodes, 8 x 8 columns: a batch solve's sums 75.2 -> 51.8 ms).
+// The compensated sums lie in shared memory (they are touched every
+// 288 sources), which leaves the registers to four blocks an SM at FB = 4.
+constexpr int kGeoSt = 96;               // sources a stage
 template <int FB, int RB>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 k_mgeo32(const MGroup* __restrict__ G, const MInst* __restrict__ I,
          const int4* __restrict__ items, int nitems, const int* __restrict__ skip) {
     if (skip && *skip) return;
     static_assert(RB % 4 == 0 && RB >= 4, "RB right-hand sides in float4 groups");
-    constexpr int kSt = (FB * RB <= 16) ? kStage : kStage / 2;
-    __shared__ float4 sP[kSt];
-    __shared__ float4 sS[kSt][FB * RB / 4];
+    __shared__ float4 sP[kGeoSt];
+    __shared__ float4 sS[kGeoSt][FB * RB / 4];
+    __shared__ float2 sAcc[FB * RB][kThreads];           // (hi, lo)
     const int tid = threadIdx.x;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int4 w = items[it];          // (group, tile, split, field block * 4096 + rhs block)
@@ -1347,7 +1354,7 @@ k_mgeo32(const MGroup* __restrict__ G, const MInst* __restrict__ I,
         const int f0 = (w.w >> 12) * FB, r0 = (w.w & 4095) * RB;
         const int nf = min(FB, gr.ninst - f0);
         int nrr[FB];
-        float A[FB], B[FB], gx[FB], gy[FB], gz[FB];
+        float A[FB], gx[FB], gy[FB], gz[FB], H = 0.f;
         float tx = 0, ty = 0, tz = 0, nx = 0, ny = 0, nz = 0;
         if (i < N) {
             const float4 a = gr.tgt[i], b = gr.nrm[i];
@@ -1357,73 +1364,89 @@ k_mgeo32(const MGroup* __restrict__ G, const MInst* __restrict__ I,
 #pragma unroll
         for (int f = 0; f < FB; ++f) {
             nrr[f] = 0;
-            A[f] = B[f] = gx[f] = gy[f] = gz[f] = 0.f;
+            A[f] = gx[f] = gy[f] = gz[f] = 0.f;
             if (f < nf) {
                 const int k = gr.inst[f0 + f];
                 nrr[f] = max(0, min(RB, I[k].nrhs - r0));
                 if (i < N) {
-                    const float4 q = I[k].fac[i];                 // (g, A) of field k
-                    gx[f] = q.x; gy[f] = q.y; gz[f] = q.z; A[f] = q.w;
-                    B[f] = I[k].facB[i];
+                    const float4 q = I[k].fac[i];                 // (grad a / (2 pi), a / pi) of field k
+                    const float ia = 1.f / q.w;
+                    gx[f] = q.x * ia; gy[f] = q.y * ia; gz[f] = q.z * ia; A[f] = q.w;
+                    if (f == 0) H = -I[k].facB[i] * ia;           // facB = -a H / pi
                 }
             }
         }
-        float hi[FB * RB], lo[FB * RB];
 #pragma unroll
-        for (int q = 0; q < FB * RB; ++q) hi[q] = lo[q] = 0.f;
+        for (int q = 0; q < FB * RB; ++q) sAcc[q][tid] = make_float2(0.f, 0.f);
         const int s0 = w.z * gr.chunk;
         const int s1 = min(s0 + gr.chunk, N);
-        for (int base = s0; base < s1; base += kSt) {
-            const int len = min(kSt, s1 - base);
-            __syncthreads();
-            for (int j = tid; j < len; j += kThreads) {
-                sP[j] = gr.pos[base + j];
+        float part[FB * RB];
+#pragma unroll
+        for (int q = 0; q < FB * RB; ++q) part[q] = 0.f;
+        int fill = 0;                        // sources in part
+        auto flush = [&]() {
+#pragma unroll
+            for (int q = 0; q < FB * RB; ++q) {
+                float2 v = sAcc[q][tid];
+                two_sum_acc(v.x, v.y, part[q]);
+                sAcc[q][tid] = v;
+                part[q] = 0.f;
+            }
+            fill = 0;
+        };
+        // a stage's pairs; FULL: all FB fields are there
+        auto pairs = [&](int len, auto full) {
+#pragma unroll 2
+            for (int j = 0; j < len; ++j) {
+                const float4 p = sP[j];
+                const float dx = tx - p.x, dy = ty - p.y, dz = tz - p.z;
+                const float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, gr.eps2)));
+                const float inv = rcp_approx(r2);
+                const float q = fmaf(nx, dx, fmaf(ny, dy, nz * dz)) * inv;
+                const float base = q * (q - H);
+                const float zx = dx * inv, zy = dy * inv, zz = dz * inv;
 #pragma unroll
                 for (int f = 0; f < FB; ++f) {
-                    float v[RB];
-                    const float* sf = (f < nf) ? I[gr.inst[f0 + f]].s32 : nullptr;
+                    if (!decltype(full)::value && f >= nf) break;
+                    const float gfac = fmaf(gx[f], zx, fmaf(gy[f], zy, fmaf(gz[f], zz, base)));
 #pragma unroll
-                    for (int q = 0; q < RB; ++q)
-                        v[q] = (q < nrr[f]) ? sf[(size_t)(r0 + q) * N + base + j] : 0.f;
-#pragma unroll
-                    for (int q = 0; q < RB / 4; ++q)
-                        sS[j][f * (RB / 4) + q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                }
-            }
-            __syncthreads();
-            for (int j0 = 0; j0 < len; j0 += kTile) {
-                const int j1 = min(j0 + kTile, len);
-                float part[FB * RB];
-#pragma unroll
-                for (int q = 0; q < FB * RB; ++q) part[q] = 0.f;
-#pragma unroll 2
-                for (int j = j0; j < j1; ++j) {
-                    const float4 p = sP[j];
-                    const float dx = tx - p.x, dy = ty - p.y, dz = tz - p.z;
-                    const float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, gr.eps2)));
-                    const float inv = rcp_approx(r2);
-                    const float nr = fmaf(nx, dx, fmaf(ny, dy, nz * dz));
-                    const float t1 = nr * nr * inv;
-#pragma unroll
-                    for (int f = 0; f < FB; ++f) {
-                        if (f >= nf) break;
-                        const float gr_ = fmaf(gx[f], dx, fmaf(gy[f], dy, gz[f] * dz));
-                        const float gfac = inv * fmaf(A[f], t1, fmaf(B[f], nr, gr_));
-#pragma unroll
-                        for (int q = 0; q < RB / 4; ++q) {
-                            const float4 sv = sS[j][f * (RB / 4) + q];
-                            float* pq = part + f * RB + 4 * q;
-                            pq[0] = fmaf(sv.x, gfac, pq[0]);
-                            pq[1] = fmaf(sv.y, gfac, pq[1]);
-                            pq[2] = fmaf(sv.z, gfac, pq[2]);
-                            pq[3] = fmaf(sv.w, gfac, pq[3]);
-                        }
+                    for (int k = 0; k < RB / 4; ++k) {
+                        const float4 sv = sS[j][f * (RB / 4) + k];
+                        float* pq = part + f * RB + 4 * k;
+                        pq[0] = fmaf(sv.x, gfac, pq[0]);
+                        pq[1] = fmaf(sv.y, gfac, pq[1]);
+                        pq[2] = fmaf(sv.z, gfac, pq[2]);
+                        pq[3] = fmaf(sv.w, gfac, pq[3]);
                     }
                 }
-#pragma unroll
-                for (int q = 0; q < FB * RB; ++q) two_sum_acc(hi[q], lo[q], part[q]);
             }
+        };
+        for (int base = s0; base < s1; base += kGeoSt) {
+            const int len = min(kGeoSt, s1 - base);
+            __syncthreads();
+            for (int e = tid; e < len * (FB + 1); e += kThreads) {
+                const int f = e / len - 1, j = e - (f + 1) * len;
+                if (f < 0) {
+                    sP[j] = gr.pos[base + j];
+                    continue;
+                }
+                float v[RB];
+                const float* sf = (f < nf) ? I[gr.inst[f0 + f]].s32 : nullptr;
+                const int nr = (f < nf) ? min(RB, I[gr.inst[f0 + f]].nrhs - r0) : 0;
+#pragma unroll
+                for (int q = 0; q < RB; ++q)
+                    v[q] = (q < nr) ? sf[(size_t)(r0 + q) * N + base + j] : 0.f;
+#pragma unroll
+                for (int q = 0; q < RB / 4; ++q)
+                    sS[j][f * (RB / 4) + q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            }
+            __syncthreads();
+            if (nf == FB) pairs(len, std::true_type{});
+            else pairs(len, std::false_type{});
+            fill += len;
+            if (fill > 256) flush();
         }
+        flush();
         if (i < N) {
 #pragma unroll
             for (int f = 0; f < FB; ++f) {
@@ -1431,9 +1454,12 @@ k_mgeo32(const MGroup* __restrict__ G, const MInst* __restrict__ I,
                 const MInst& in = I[gr.inst[f0 + f]];
 #pragma unroll
                 for (int q = 0; q < RB; ++q)
-                    if (q < nrr[f])
+                    if (q < nrr[f]) {
+                        const float2 v = sAcc[f * RB + q][tid];
+                        const float h = v.x * A[f];
                         in.part[((size_t)(r0 + q) * in.nsplit + w.z) * N + i] =
-                            make_float2(hi[f * RB + q], lo[f * RB + q]);
+                            make_float2(h, fmaf(v.y, A[f], fmaf(v.x, A[f], -h)));
+                    }
             }
         }
         __syncthreads();                 // the next item restages the shared arrays
@@ -1767,7 +1793,7 @@ pm_status multi_setup(pm_ctx* ctx, pm_surface* const* ops, int nops, const int* 
     int gmax = 1;
     for (const MGroup& g : hG) gmax = std::max(gmax, g.ninst);
     const int knob = ops[0]->batch_rb;
-    M->fb = knob == 32 ? 4 : (knob == 16 ? 2 : (knob == 8 ? 1 : (gmax >= 2 ? 2 : 1)));
+    M->fb = knob == 32 ? 4 : (knob == 16 ? 2 : (knob == 8 ? 1 : (gmax >= 3 ? 4 : gmax == 2 ? 2 : 1)));
     for (int gi = 0; gi < (int)hG.size(); ++gi) {
         const MGroup& g = hG[gi];
         int rmax = 0;
