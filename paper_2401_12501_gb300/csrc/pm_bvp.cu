@@ -66,7 +66,10 @@ struct pm_bvp {
     double *xe = nullptr, *nue = nullptr, *we = nullptr, *ae = nullptr, *uv = nullptr;
     double *xo = nullptr, *wo = nullptr, *ao = nullptr, *nuo = nullptr;
     double *interp = nullptr;            // per curve [F M][M], curve blocks concatenated
-    int *interp_off = nullptr;           // [ncurves + 1] offsets into interp
+    int *interp_off = nullptr;           // five rows of [ncurves + 1]: offset into interp, first
+                                         // oversampled point, first edge node, M, offset into fourier
+    double *fourier = nullptr;           // per curve [F M / 4 + 1][M] and [M][M] (k_bvp_fill_edge_fourier)
+    bool foldable = false;               // every curve has them
     int *curve_of = nullptr;             // [Fo] curve of an oversampled point
     double *Kpg = nullptr;               // [Me][Me] K'_gamma (Neumann) or N_gamma (Dirichlet), weighted
     int *kp_ptr = nullptr, *kp_patch = nullptr, *kp_edge = nullptr;
@@ -141,11 +144,11 @@ __device__ __forceinline__ double edge_pair(const EdgeTarget& t, double y0, doub
                (t.g[0] * r0 + t.g[1] * r1 + t.g[2] * r2) * inv * (0.5 / M_PI);
     }
     // -(1/pi) [2 (n.r)(n.nu')/r^4 - 4 (n.r)^2 (r.nu')/r^6 - H (n.nu')/r^2
-    //          + 2 H (n.r)(r.nu')/r^4]
+    //          + 2 H (n.r)(r.nu')/r^4], with q = (n.r)/r^2 a product of two factors
     const double nnu = t.n[0] * u0 + t.n[1] * u1 + t.n[2] * u2;
     const double rnu = r0 * u0 + r1 * u1 + r2 * u2;
-    return -(1.0 / M_PI) * inv * (2.0 * nr * nnu * inv - 4.0 * nr * nr * rnu * inv * inv -
-                                  t.H * nnu + 2.0 * t.H * nr * rnu * inv);
+    const double q = nr * inv;
+    return (-(1.0 / M_PI) * inv) * ((2.0 * q - t.H) * (nnu - 2.0 * q * rnu));
 }
 
 // A warp a target, its lanes over the oversampled points: float64-pipe work, for which a
@@ -175,7 +178,7 @@ k_bvp_edge_to_surface(int N, const double* __restrict__ x, const double* __restr
 // A solve forms the system's matrix once, A [n][n] over z = [sigma; mu] (n = N + Me), and
 // its Krylov steps stream it: 8 n^2 bytes a step instead of the float64 pair sums of
 // apply_sys.  Dirichlet, 2,048 nodes and 128 edge nodes (a matrix of 38 MB, so it stays in
-// L2): a solve of 15 steps 176 -> 4.7 ms.
+// L2): a solve of 15 steps 176 -> 3.2 ms.
 
 // surface rows, sigma columns: delta_ij + w_j R(x_i, x_j) / a_j (kDI targets x kDJ sources a block)
 constexpr int kDI = 32, kDJ = 128;
@@ -219,6 +222,7 @@ __global__ void k_bvp_fill_near(int nblk, int pp, const int* __restrict__ row_of
 // surface rows, mu columns: sum over curve c's oversampled points of the pair kernel times the
 // interpolation row.  Block: kEI targets x 128 edge nodes of one curve; the points pass in
 // tiles of 128, a thread evaluating its point for every target, then its edge node's sums.
+// For the curves that k_bvp_fill_edge_fourier does not take.
 constexpr int kEI = 4;
 template <int KIND>
 __global__ void __launch_bounds__(128)
@@ -258,6 +262,136 @@ k_bvp_fill_edge_columns(int N, const double* __restrict__ x, const double* __res
     }
     if (e < M)
         for (int r = 0; r < kEI && i0 + r < N; ++r) A[(size_t)(i0 + r) * ld + N + off + e] = acc[r];
+}
+
+// The same columns by the trigonometric interpolant's own basis, for curves of n = F M points,
+// n a multiple of 4 and M <= kEM.  Interpolating at t_j = 2 pi j / n from the M nodes is the
+// sum over M functions cos(q t), sin(q t), so the weights of the nodes are those functions'
+// sums over the points, C_q = sum_j f_j cos(q t_j) and S_q, times an M x M matrix; and the four
+// points t, -t, pi - t, pi + t of a quarter share every function up to its sign, so a quarter
+// of the products remains once their values are added with the four patterns of signs (even
+// and odd q of the cosines, then of the sines).  Bound by the float64 pipe (two multiply-adds a
+// clock an SM): at 2,048 targets, two curves of 64 nodes and 2,048 points, 0.5 ms of pair
+// kernels stay and the products are 0.25 ms instead of 0.95 (by operation counts; the whole
+// Dirichlet solve of 2,048 + 128 unknowns 3.70 -> 3.16 ms).
+// fourier[off]: [n / 4 + 1][M] functions at t_j, then [M][M] functions at the nodes, scaled;
+// order: even q cosines, odd q cosines, even q sines, odd q sines.
+constexpr int kEM = 512;              // [M][kEI] beside sk in 48 KB of shared memory
+__host__ __device__ __forceinline__ int cosines(int M, int odd) {    // q = 0 .. ceil(M / 2) - 1
+    return ((M + 1) / 2 + 1 - odd) / 2;
+}
+__host__ __device__ __forceinline__ int sines(int M, int odd) {      // q = 1 .. floor(M / 2)
+    return (M / 2 + odd) / 2;
+}
+template <int KIND>
+__global__ void __launch_bounds__(128)
+k_bvp_fill_edge_fourier(int N, const double* __restrict__ x, const double* __restrict__ n,
+                        const double* __restrict__ H, const double* __restrict__ a,
+                        const double* __restrict__ g, int ncurves, const double* __restrict__ xo,
+                        const double* __restrict__ wo, const double* __restrict__ ao,
+                        const double* __restrict__ nuo, const double* __restrict__ fourier,
+                        const int* __restrict__ ioff, int ld, double* __restrict__ A) {
+    __shared__ EdgeTarget t[kEI];
+    __shared__ double sk[4][128][kEI];
+    extern __shared__ double coef[];     // [M][kEI]
+    const int c = blockIdx.y, nc1 = ncurves + 1, tid = threadIdx.x;
+    const int o0 = ioff[nc1 + c], np = ioff[nc1 + c + 1] - o0, off = ioff[2 * nc1 + c], M = ioff[3 * nc1 + c];
+    const double* F = fourier + ioff[4 * nc1 + c];
+    const int i0 = blockIdx.x * kEI, quarter = np / 4;
+    const int k1 = cosines(M, 0), k2 = k1 + cosines(M, 1), k3 = k2 + sines(M, 0);
+    if (tid < kEI) t[tid] = edge_target<KIND>(min(i0 + tid, N - 1), x, n, H, a, g);
+    for (int e = tid; e < M * kEI; e += 128) coef[e] = 0.0;
+    __syncthreads();
+    for (int base = 0; base <= quarter; base += 128) {
+        const int j = base + tid;
+        if (j <= quarter) {
+            // t_j, -t_j, pi - t_j, pi + t_j; at j = 0 and n / 4 two of them are one point
+            const int pt[4] = {j, np - j, np / 2 - j, np / 2 + j};
+            const bool end = j == 0 || j == quarter;
+            double v[4][kEI];
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const int y = o0 + pt[s];
+                if (end && !(s == 0 || s == (j == 0 ? 2 : 1))) {
+#pragma unroll
+                    for (int r = 0; r < kEI; ++r) v[s][r] = 0.0;
+                    continue;
+                }
+                const double w = KIND == kEdgeT ? wo[y] : wo[y] / ao[y];
+#pragma unroll
+                for (int r = 0; r < kEI; ++r)
+                    v[s][r] = w * edge_pair<KIND>(t[r], xo[3 * y], xo[3 * y + 1], xo[3 * y + 2],
+                                                  nuo[3 * y], nuo[3 * y + 1], nuo[3 * y + 2]);
+            }
+#pragma unroll
+            for (int r = 0; r < kEI; ++r) {
+                const double sum0 = v[0][r] + v[1][r], dif0 = v[0][r] - v[1][r];
+                const double sum1 = v[2][r] + v[3][r], dif1 = v[2][r] - v[3][r];
+                sk[0][tid][r] = sum0 + sum1;
+                sk[1][tid][r] = sum0 - sum1;
+                sk[2][tid][r] = dif0 - dif1;
+                sk[3][tid][r] = dif0 + dif1;
+            }
+        }
+        __syncthreads();
+        const int cnt = min(128, quarter + 1 - base);
+        for (int e = tid; e < M; e += 128) {
+            const double(*f)[kEI] = sk[(e >= k1) + (e >= k2) + (e >= k3)];
+            const double* col = F + (size_t)base * M + e;
+            double acc[kEI];
+#pragma unroll
+            for (int r = 0; r < kEI; ++r) acc[r] = coef[e * kEI + r];
+#pragma unroll 4
+            for (int q = 0; q < cnt; ++q) {
+                const double b = col[(size_t)q * M];
+#pragma unroll
+                for (int r = 0; r < kEI; ++r) acc[r] = fma(b, f[q][r], acc[r]);
+            }
+#pragma unroll
+            for (int r = 0; r < kEI; ++r) coef[e * kEI + r] = acc[r];
+        }
+        __syncthreads();
+    }
+    const double* D = F + (size_t)(quarter + 1) * M;
+    for (int e = tid; e < M; e += 128) {
+        double acc[kEI] = {};
+#pragma unroll 4
+        for (int q = 0; q < M; ++q) {
+            const double b = D[(size_t)q * M + e];
+#pragma unroll
+            for (int r = 0; r < kEI; ++r) acc[r] = fma(b, coef[q * kEI + r], acc[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < kEI; ++r)
+            if (i0 + r < N) A[(size_t)(i0 + r) * ld + N + off + e] = acc[r];
+    }
+}
+
+// fourier of one curve of m nodes and f m points
+void fourier_tables(int m, int f, std::vector<double>* out) {
+    const int n = f * m;
+    auto function = [m](int e, int* q, bool* sine) {
+        const int k1 = cosines(m, 0), k2 = k1 + cosines(m, 1), k3 = k2 + sines(m, 0);
+        *sine = e >= k2;
+        *q = e < k1 ? 2 * e : e < k2 ? 2 * (e - k1) + 1 : e < k3 ? 2 * (e - k2) + 2 : 2 * (e - k3) + 1;
+    };
+    // function e at the angle 2 pi num / den
+    auto value = [&](int e, long long num, int den) {
+        int q;
+        bool sine;
+        function(e, &q, &sine);
+        const double t = 2.0 * M_PI * (double)(num * q % den) / den;
+        return sine ? std::sin(t) : std::cos(t);
+    };
+    for (int j = 0; j <= n / 4; ++j)
+        for (int e = 0; e < m; ++e) out->push_back(value(e, j, n));
+    for (int e = 0; e < m; ++e) {
+        int q;
+        bool sine;
+        function(e, &q, &sine);
+        const double scale = (q == 0 || 2 * q == m ? 1.0 : 2.0) / m;
+        for (int k = 0; k < m; ++k) out->push_back(scale * value(e, 2 * k + 1, 2 * m));
+    }
 }
 
 // edge rows (as k_bvp_edge_row, without the corrections)
@@ -421,10 +555,16 @@ pm_status fill_sys(pm_bvp* b, double* A) {
         s->nblk, s->pp, s->blk_row, 0, s->blk_patch, s->cR64, ld, A);
     if (Me > 0) {
         const int mmax = *std::max_element(b->M.begin(), b->M.end());
-        dim3 grid(pm_ceil_div(N, kEI), b->ncurves, pm_ceil_div(mmax, 128));
-        (b->kind ? k_bvp_fill_edge_columns<kEdgeT> : k_bvp_fill_edge_columns<kEdgeR>)
-            <<<grid, 128, 0, st>>>(N, s->x, s->n, s->H, s->a, s->g, b->ncurves, b->xo, b->wo, b->ao,
-                                   b->nuo, b->interp, b->interp_off, ld, A);
+        dim3 grid(pm_ceil_div(N, kEI), b->ncurves, b->foldable ? 1 : pm_ceil_div(mmax, 128));
+        if (b->foldable)
+            (b->kind ? k_bvp_fill_edge_fourier<kEdgeT> : k_bvp_fill_edge_fourier<kEdgeR>)
+                <<<grid, 128, (size_t)mmax * kEI * sizeof(double), st>>>(
+                    N, s->x, s->n, s->H, s->a, s->g, b->ncurves, b->xo, b->wo, b->ao, b->nuo,
+                    b->fourier, b->interp_off, ld, A);
+        else
+            (b->kind ? k_bvp_fill_edge_columns<kEdgeT> : k_bvp_fill_edge_columns<kEdgeR>)
+                <<<grid, 128, 0, st>>>(N, s->x, s->n, s->H, s->a, s->g, b->ncurves, b->xo, b->wo,
+                                       b->ao, b->nuo, b->interp, b->interp_off, ld, A);
         k_bvp_fill_edge_rows<<<dim3(pm_ceil_div(ld, kT), Me), kT, 0, st>>>(
             b->kind, N, Me, s->x, s->wa, b->xe, b->nue, b->ae, b->we, b->Kpg, ld, A);
         k_bvp_fill_near<<<pm_ceil_div((long long)b->kp_nblk * s->pp, kT), kT, 0, st>>>(
@@ -469,7 +609,7 @@ void free_bvp(pm_bvp* b) {
     if (b->s) cudaSetDevice(b->s->ctx->device);
     pm_dfree(b->xe); pm_dfree(b->nue); pm_dfree(b->we); pm_dfree(b->ae); pm_dfree(b->uv);
     pm_dfree(b->xo); pm_dfree(b->wo); pm_dfree(b->ao); pm_dfree(b->nuo); pm_dfree(b->interp);
-    pm_dfree(b->interp_off);
+    pm_dfree(b->interp_off); pm_dfree(b->fourier);
     pm_dfree(b->curve_of); pm_dfree(b->Kpg); pm_dfree(b->kp_ptr); pm_dfree(b->kp_patch);
     pm_dfree(b->kp_C); pm_dfree(b->kp_edge); pm_dfree(b->mu_o);
     delete b;
@@ -490,8 +630,8 @@ pm_status create_impl(pm_bvp* b, const double* edge_x, const double* edge_d1,
     const int Me = b->Me, Fo = b->Fo, pp = s->pp;
     // trapezoid weights, K'_gamma (host, dense), interpolation matrices
     b->h_we.resize(Me);
-    std::vector<double> wo(Fo), Kpg((size_t)Me * Me), I;
-    std::vector<int> ioff(4 * (b->ncurves + 1), 0), curve_of(Fo);
+    std::vector<double> wo(Fo), Kpg((size_t)Me * Me), I, fourier;
+    std::vector<int> ioff(5 * (b->ncurves + 1), 0), curve_of(Fo);
     for (int c = 0; c < b->ncurves; ++c) {
         const int m = b->M[c], f = b->F[c];
         for (int k = 0; k < m; ++k) {
@@ -518,6 +658,13 @@ pm_status create_impl(pm_bvp* b, const double* edge_x, const double* edge_d1,
     }
     const int nc1 = b->ncurves + 1;
     ioff[b->ncurves] = (int)I.size();
+    b->foldable = b->ncurves > 0;
+    for (int c = 0; c < b->ncurves; ++c)
+        b->foldable = b->foldable && b->M[c] <= kEM && b->M[c] * b->F[c] % 4 == 0;
+    for (int c = 0; c < b->ncurves && b->foldable; ++c) {
+        ioff[4 * nc1 + c] = (int)fourier.size();
+        fourier_tables(b->M[c], b->F[c], &fourier);
+    }
     for (int c = 0; c < nc1; ++c) {
         ioff[nc1 + c] = c < b->ncurves ? b->offo[c] : Fo;
         ioff[2 * nc1 + c] = c < b->ncurves ? b->off[c] : Me;
@@ -579,6 +726,7 @@ pm_status create_impl(pm_bvp* b, const double* edge_x, const double* edge_d1,
     PM_TRY(upload(&b->ao, over_a, (size_t)Fo));
     PM_TRY(upload(&b->nuo, over_nu, 3 * (size_t)Fo));
     PM_TRY(upload(&b->interp, I.data(), I.size()));
+    PM_TRY(upload(&b->fourier, fourier.data(), fourier.size()));
     PM_TRY(upload(&b->interp_off, ioff.data(), ioff.size()));
     PM_TRY(upload(&b->curve_of, curve_of.data(), curve_of.size()));
     PM_TRY(upload(&b->Kpg, Kpg.data(), Kpg.size()));

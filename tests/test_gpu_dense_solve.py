@@ -57,8 +57,19 @@ def test_wave_solve(ctx, monkeypatch, m, p, kind):
 @pytest.mark.parametrize("kind,n,p,M", [("neumann", 4, 5, 12), ("dirichlet", 4, 6, 36),
                                         ("dirichlet", 3, 7, 135), ("neumann", 3, 6, 129)])
 def test_edge_solve(ctx, monkeypatch, kind, n, p, M):
+    edge_solve(ctx, monkeypatch, kind, n, p, M, 4)
+
+
+# F M a multiple of 4 with M even (a Nyquist function) and odd, one tile of points and a
+# remainder; F M not a multiple of 4, below and above a block's 128 nodes
+@pytest.mark.parametrize("kind,M,F", [("neumann", 6, 6), ("dirichlet", 9, 8), ("neumann", 129, 8),
+                                      ("dirichlet", 66, 8), ("dirichlet", 9, 6), ("neumann", 135, 6)])
+def test_edge_columns(ctx, monkeypatch, kind, M, F):
+    edge_solve(ctx, monkeypatch, kind, 3, 6, M, F)
+
+
+def edge_solve(ctx, monkeypatch, kind, n, p, M, F):
     import paper_2401_12501_gb300 as pm
-    F = 4
     band = bands.torus_band(2, n, p, M, F)
     co = (bands.band_coefficient(band) if kind == "neumann" else bands.constant_band_coefficient(band))
     S = pm.Surface.from_fixture(ctx, band.surface)
