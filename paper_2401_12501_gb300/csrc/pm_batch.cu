@@ -1121,6 +1121,8 @@ size_t pm_batch_need_bytes(const pm_surface* s, int nrhs) {
     if (!(s->batch && s->batch->cap >= nrhs))
         need += R * N * (sizeof(float) + sizeof(float2) + 8 * sizeof(float2)) +
                 R * (size_t)s->npatch * s->ppad * sizeof(float);
+    if (nrhs >= kFfmmMin && !(s->batch && s->batch->cap >= nrhs && s->batch->fm.S))
+        need += pm_ffmm_bytes(s->N);
     return need;
 }
 

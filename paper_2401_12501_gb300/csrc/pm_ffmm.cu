@@ -402,27 +402,39 @@ pm_status launch(pm_surface* s, const PmFfmmWork& W, const Cols& C, int nsplit, 
 
 }  // namespace
 
+static size_t digit_words(int N) {
+    return (size_t)pm_ceil_div(N, kFmK) * kFmK / 16 * 8 * kQmDigits * 64;
+}
+static size_t bound_words(int N) { return 2 * (size_t)N + 1; }
+
+size_t pm_ffmm_bytes(int N) { return (digit_words(N) + bound_words(N) + kFmCols) * sizeof(int); }
+
 void pm_ffmm_free(PmFfmmWork* W) {
     pm_dfree(W->S);
     pm_dfree(W->top);
     pm_dfree(W->bound);
 }
 
-// Buffers and the geometry's bounds; PM_ERR_OOM leaves W empty
+// Buffers and the geometry's bounds; PM_ERR_OOM leaves W empty and no error behind, and the
+// caller takes the sums without buffers -- as it does on a stream under capture, where nothing
+// can be allocated
 static pm_status ffmm_ready(pm_surface* s, PmFfmmWork* W, cudaStream_t st) {
     if (W->S) return PM_OK;
-    const int Npad = pm_ceil_div(s->N, kFmK) * kFmK;
-    pm_status r = pm_dmalloc(&W->S, (size_t)Npad / 16 * 8 * kQmDigits * 64);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    PM_CUDA_TRY(cudaStreamIsCapturing(st, &capture));
+    if (capture != cudaStreamCaptureStatusNone) return PM_ERR_OOM;
+    pm_status r = pm_dmalloc(&W->S, digit_words(s->N));
     if (r == PM_OK) r = pm_dmalloc(&W->top, kFmCols);
-    if (r == PM_OK) r = pm_dmalloc(&W->bound, 2 * (size_t)s->N + 1);
+    if (r == PM_OK) r = pm_dmalloc(&W->bound, bound_words(s->N));
     if (r == PM_OK) {
-        cudaMemsetAsync(W->bound, 0, (2 * (size_t)s->N + 1) * sizeof(int), st);
+        cudaMemsetAsync(W->bound, 0, bound_words(s->N) * sizeof(int), st);
         const int blocks = pm_ceil_div(s->N, 128);
         k_fm_top<<<dim3(blocks, std::max(1, std::min(blocks, 4 * s->ctx->num_sms / blocks))), 128, 0, st>>>(
             s->x, s->n, s->H, s->N, W->bound);
         if (cudaGetLastError() != cudaSuccess) r = PM_ERR_CUDA;
     }
     if (r != PM_OK) pm_ffmm_free(W);
+    if (r == PM_ERR_OOM) cudaGetLastError();
     return r;
 }
 

@@ -316,6 +316,7 @@ struct PmFfmmWork {
     unsigned int* bound = nullptr;  // the geometry's largest kernel values by target
 };
 void pm_ffmm_free(PmFfmmWork* W);
+size_t pm_ffmm_bytes(int N);        // device bytes of its buffers
 // partial[(column nsplit + split) N + i] for the columns of ops[0..nops) (all on s's geometry;
 // PM_FFMM_R: one operator), sigma[q] + r ld operator q's column r
 pm_status pm_ffmm_sum(pm_surface* s, PmFfmmWork* W, int kind, int nops, pm_surface* const* ops,

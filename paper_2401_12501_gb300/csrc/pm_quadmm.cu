@@ -590,9 +590,13 @@ pm_status weights(pm_surface* s, const QmRules& R, int eB, bool* over) {
             cell_cols.emplace_back(c0, hcnt[h]);
             c0 += hcnt[h];
         }
-        if (c0 != nleaf) {
-            pm_set_error("near-field weights: more than %d different cells in a batch", kQmHash);
-            return PM_ERR_INTERNAL;
+        if (c0 != nleaf) {                                 // more different cells than kQmHash
+            if (np == 1) {
+                pm_set_error("near-field weights: more than %d different cells in a block", kQmHash);
+                return PM_ERR_INTERNAL;
+            }
+            take = np / 2;
+            continue;
         }
         PM_CUDA_TRY(cudaMemcpy(cnt, hpos.data(), sizeof(int) * kQmHash, cudaMemcpyHostToDevice));
         k_qm_place<<<pm_ceil_div(np, 128), 128>>>(np, blocks, start, count, where, cnt, s->blk_row,
