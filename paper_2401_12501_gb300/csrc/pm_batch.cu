@@ -454,14 +454,14 @@ static pm_status batch_ensure(pm_surface* s, int nrhs) {
     if (s->batch && s->batch->cap >= nrhs) return PM_OK;
     pm_batch_free(s);
     s->batch = new PmBatchWork();
-    PmBatchWork& B = *s->batch;
-    B.cap = nrhs;
+    PmBatchWork& B = *s->batch;          // cap stays 0 until every buffer is there
     B.nsplit_max = nsplit_max;
     PM_TRY(pm_dmalloc(&B.s32, (size_t)nrhs * s->N));
     PM_TRY(pm_dmalloc(&B.sig32, (size_t)nrhs * s->npatch * s->ppad));
     PM_CUDA_TRY(cudaMemset(B.sig32, 0, sizeof(float) * (size_t)nrhs * s->npatch * s->ppad));
     PM_TRY(pm_dmalloc(&B.sff, (size_t)nrhs * s->N));
     PM_TRY(pm_dmalloc(&B.part, (size_t)nrhs * nsplit_max * s->N));
+    B.cap = nrhs;
     return PM_OK;
 }
 
@@ -951,7 +951,11 @@ static pm_status bsolve_work(pm_surface* s, int nrhs, PmBatchSolveWork** out) {
     }
     pm_batch_solve_free(s);
     s->bsolve = new PmBatchSolveWork();
-    PM_TRY(bsolve_alloc(*s->bsolve, nrhs, m, s->N));
+    const pm_status r = bsolve_alloc(*s->bsolve, nrhs, m, s->N);
+    if (r != PM_OK) {
+        pm_batch_solve_free(s);          // its shape would pass for a whole workspace
+        return r;
+    }
     *out = s->bsolve;
     return PM_OK;
 }
