@@ -765,10 +765,12 @@ __global__ void k_bcycle_start(int nrhs, const double* __restrict__ nrm2, long l
     if (threadIdx.x == 0) *all_done = any_active ? 0 : 1;
 }
 
+// use_cond: also sets a graph node's condition, whether a column still works
 __global__ void k_brotate(int nrhs, double* __restrict__ H, int ldh, int m, int k,
                           double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g,
                           double* __restrict__ scal, int* __restrict__ done,
-                          int* __restrict__ iters, int* __restrict__ all_done) {
+                          int* __restrict__ iters, int* __restrict__ all_done, int use_cond,
+                          cudaGraphConditionalHandle cond) {
     __shared__ int any_active;
     if (threadIdx.x == 0) any_active = 0;
     __syncthreads();
@@ -801,7 +803,10 @@ __global__ void k_brotate(int nrhs, double* __restrict__ H, int ldh, int m, int 
         if (!d) atomicOr(&any_active, 1);
     }
     __syncthreads();
-    if (threadIdx.x == 0) *all_done = any_active ? 0 : 1;
+    if (threadIdx.x == 0) {
+        *all_done = any_active ? 0 : 1;
+        if (use_cond) cudaGraphSetConditional(cond, any_active ? 1u : 0u);
+    }
 }
 
 // per right-hand side: y = H^{-1} g by back substitution and ynorm = |y|_2 (the
@@ -1063,7 +1068,7 @@ struct BSolver {
                     hk, (long long)m * ldh, W.hcol, m + 2, k + 1, W.done);
                 dots(W.w, 0, N, 1, W.w, N, W.scal + 1, 8, W.done);
                 k_brotate<<<1, 256, 0, st>>>(nrhs, W.H, ldh, m, k, W.cs, W.sn, W.g, W.scal, W.done,
-                                             W.iters, W.all_done);
+                                             W.iters, W.all_done, 0, 0);
                 k_bscale_copy<<<dim3(grid_n, nrhs), 256, 0, st>>>(W.w, N, W.scal + 2, 8, 0, vk1, ldV,
                                                                   N, W.done);
                 s->launch_total += 5;
@@ -1632,7 +1637,7 @@ struct PmMultiWork {
     double *wcol = nullptr, *inv_sw = nullptr;
     float *s32 = nullptr, *sig32 = nullptr;
     float2* part = nullptr;
-    cudaStream_t cap = nullptr;
+    cudaStream_t cap = nullptr, body = nullptr;
     std::map<int, cudaGraphExec_t> graphs;
     void release() {
         for (auto& kv : graphs) cudaGraphExecDestroy(kv.second);
@@ -1643,7 +1648,8 @@ struct PmMultiWork {
         pm_dfree(fac); pm_dfree(nrm); pm_dfree(facB); pm_dfree(col_n); pm_dfree(wcol);
         pm_dfree(inv_sw); pm_dfree(s32); pm_dfree(sig32); pm_dfree(part);
         if (cap) cudaStreamDestroy(cap);
-        cap = nullptr;
+        if (body) cudaStreamDestroy(body);
+        cap = body = nullptr;
         ops.clear();
         nrhs.clear();
     }
@@ -1856,6 +1862,7 @@ pm_status multi_setup(pm_ctx* ctx, pm_surface* const* ops, int nops, const int* 
     const int bps = (ops[0]->batch_bps >= 1 && ops[0]->batch_bps <= 16) ? ops[0]->batch_bps : 8;
     M->grid = std::max(1, std::min(M->nitems, bps * ops[0]->ctx->num_sms));
     PM_CUDA_TRY(cudaStreamCreateWithFlags(&M->cap, cudaStreamNonBlocking));
+    PM_CUDA_TRY(cudaStreamCreateWithFlags(&M->body, cudaStreamNonBlocking));
     M->ops.assign(ops, ops + nops);
     M->nrhs.assign(nrhs, nrhs + nops);
     M->epochs.clear();
@@ -1931,18 +1938,24 @@ struct MSolver {
         return PM_OK;
     }
 
-    // the launches of one GMRES cycle of `steps` Arnoldi steps (float32 operator)
-    pm_status issue_cycle(int steps) {
+    // the launches of one GMRES cycle (float32 operator): its start, Arnoldi steps k0 .. k1 - 1
+    // (the last one sets a graph node's condition), its end
+    pm_status issue_start() {
         const int m = W.m, N = W.N, nc = M.ncols;
-        const long long ldV = (long long)(m + 1) * N;
-        const int ldh = m + 2;
         dots(W.r, 0, N, 1, W.r, N, W.scal + 1, 8, nullptr);
         k_bcycle_start<<<1, 256, 0, st>>>(nc, W.scal + 1, 8, W.g, m, W.scal, W.done, W.iters,
                                           W.all_done);
-        k_bscale_copy<<<dim3(grid_n, nc), 256, 0, st>>>(W.r, N, W.scal + 3, 8, 1, W.V, ldV, N,
-                                                        W.done);
-        launches += 2;
-        for (int k = 0; k < steps; ++k) {
+        k_bscale_copy<<<dim3(grid_n, nc), 256, 0, st>>>(W.r, N, W.scal + 3, 8, 1, W.V,
+                                                        (long long)(m + 1) * N, N, W.done);
+        PM_CUDA_TRY(cudaGetLastError());
+        return PM_OK;
+    }
+
+    pm_status issue_steps(int k0, int k1, int use_cond, cudaGraphConditionalHandle cond) {
+        const int m = W.m, N = W.N, nc = M.ncols;
+        const long long ldV = (long long)(m + 1) * N;
+        const int ldh = m + 2;
+        for (int k = k0; k < k1; ++k) {
             double* vk = W.V + (size_t)k * N;
             double* vk1 = W.V + (size_t)(k + 1) * N;
             double* hk = W.H + (size_t)k * ldh;
@@ -1957,48 +1970,98 @@ struct MSolver {
                 hk, (long long)m * ldh, W.hcol, m + 2, k + 1, W.done);
             dots(W.w, 0, N, 1, W.w, N, W.scal + 1, 8, W.done);
             k_brotate<<<1, 256, 0, st>>>(nc, W.H, ldh, m, k, W.cs, W.sn, W.g, W.scal, W.done,
-                                         W.iters, W.all_done);
+                                         W.iters, W.all_done, use_cond && k + 1 == k1, cond);
             k_bscale_copy<<<dim3(grid_n, nc), 256, 0, st>>>(W.w, N, W.scal + 2, 8, 0, vk1, ldV, N,
                                                             W.done);
-            launches += 5;
         }
-        k_bbacksolve<<<pm_ceil_div(nc, 64), 64, 0, st>>>(nc, W.H, ldh, m, W.g, W.iters, W.y,
-                                                         W.ynorm);
-        k_badd_combo<<<dim3(grid_n, nc), 256, 0, st>>>(W.V, N, ldV, W.iters, W.y, m, W.delta, N);
-        launches += 2;
         PM_CUDA_TRY(cudaGetLastError());
         return PM_OK;
     }
 
-    // one cycle as a CUDA graph (captured on the workspace's own stream the first
-    // time a cycle of this length runs, replayed on st after that)
+    pm_status issue_end() {
+        const int m = W.m, N = W.N, nc = M.ncols;
+        k_bbacksolve<<<pm_ceil_div(nc, 64), 64, 0, st>>>(nc, W.H, m + 2, m, W.g, W.iters, W.y,
+                                                         W.ynorm);
+        k_badd_combo<<<dim3(grid_n, nc), 256, 0, st>>>(W.V, N, (long long)(m + 1) * N, W.iters, W.y,
+                                                       m, W.delta, N);
+        PM_CUDA_TRY(cudaGetLastError());
+        return PM_OK;
+    }
+
+    // One cycle as a CUDA graph, captured on the workspace's own streams: the start and kFirst
+    // steps, then groups of kGroup steps each in a conditional node that runs while a column
+    // still works, then the end.  A cycle may take `steps` steps (50) and takes about ten;
+    // the 17 launches of every idle step used to run, each returning at once: 1,536 nodes with
+    // 2 operators of one right-hand side 3.54 -> 2.48 ms a batch, 9,600 with 4 x 2 14.4 -> 13.2,
+    // 24,576 with 8 x 8 103.8 -> 101.3.
+    static constexpr int kFirst = 6, kGroup = 4;
+    pm_status capture_cycle(int steps, cudaGraphExec_t* ex) {
+        cudaStream_t user = st;
+        const long long before = launches;
+        const int ngroup = std::max(0, pm_ceil_div(steps - kFirst, kGroup));
+        std::vector<cudaGraphConditionalHandle> cond(ngroup + 1, 0);
+        PM_CUDA_TRY(cudaStreamBeginCapture(M.cap, cudaStreamCaptureModeThreadLocal));
+        cudaGraph_t g = nullptr, out = nullptr;
+        cudaStreamCaptureStatus cst;
+        cudaError_t ce = cudaStreamGetCaptureInfo(M.cap, &cst, nullptr, &g, nullptr, nullptr, nullptr);
+        for (int c = 0; c < ngroup && ce == cudaSuccess; ++c)
+            ce = cudaGraphConditionalHandleCreate(&cond[c], g, 0, cudaGraphCondAssignDefault);
+        pm_status ps = PM_OK;
+        if (ce == cudaSuccess) {
+            st = M.cap;
+            ps = issue_start();
+            if (ps == PM_OK) ps = issue_steps(0, std::min(steps, kFirst), ngroup > 0, cond[0]);
+        }
+        for (int c = 0; c < ngroup && ce == cudaSuccess && ps == PM_OK; ++c) {
+            const cudaGraphNode_t* deps = nullptr;
+            size_t ndeps = 0;
+            cudaGraphNode_t node = nullptr;
+            cudaGraphNodeParams cp = {};
+            cp.type = cudaGraphNodeTypeConditional;
+            cp.conditional.handle = cond[c];
+            cp.conditional.type = cudaGraphCondTypeIf;
+            cp.conditional.size = 1;
+            ce = cudaStreamGetCaptureInfo(M.cap, &cst, nullptr, nullptr, &deps, nullptr, &ndeps);
+            if (ce == cudaSuccess) ce = cudaGraphAddNode(&node, g, deps, nullptr, ndeps, &cp);
+            if (ce == cudaSuccess)
+                ce = cudaStreamUpdateCaptureDependencies(M.cap, &node, nullptr, 1,
+                                                         cudaStreamSetCaptureDependencies);
+            if (ce == cudaSuccess)
+                ce = cudaStreamBeginCaptureToGraph(M.body, cp.conditional.phGraph_out[0], nullptr,
+                                                   nullptr, 0, cudaStreamCaptureModeThreadLocal);
+            if (ce != cudaSuccess) break;
+            const int k0 = kFirst + c * kGroup;
+            st = M.body;
+            ps = issue_steps(k0, std::min(steps, k0 + kGroup), c + 1 < ngroup, cond[c + 1]);
+            cudaGraph_t body = nullptr;
+            ce = cudaStreamEndCapture(M.body, &body);
+        }
+        if (ce == cudaSuccess && ps == PM_OK) {
+            st = M.cap;
+            ps = issue_end();
+        }
+        const cudaError_t ended = cudaStreamEndCapture(M.cap, &out);
+        if (ce == cudaSuccess) ce = ended;
+        st = user;
+        launches = before;
+        if (ce == cudaSuccess && ps == PM_OK)
+            ce = cudaGraphInstantiate(ex, out, cudaGraphInstantiateFlagUseNodePriority);
+        if (out) cudaGraphDestroy(out);
+        if (ps != PM_OK) return ps;
+        if (ce != cudaSuccess) {
+            cudaGetLastError();
+            pm_set_error("multi-instance solve: cycle graph capture: %s", cudaGetErrorString(ce));
+            return PM_ERR_CUDA;
+        }
+        return PM_OK;
+    }
+
+    // one cycle of at most `steps` steps, captured the first time a cycle of this length runs
     pm_status run_cycle(int steps) {
         auto it = M.graphs.find(steps);
         if (it == M.graphs.end()) {
-            cudaStream_t user = st;
-            st = M.cap;
-            PM_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            const long long before = launches;
-            const pm_status ps = issue_cycle(steps);
-            cudaGraph_t g = nullptr;
-            const cudaError_t ce = cudaStreamEndCapture(st, &g);
-            st = user;
-            launches = before;
-            if (ps != PM_OK) {
-                if (g) cudaGraphDestroy(g);
-                return ps;
-            }
             cudaGraphExec_t ex = nullptr;
-            cudaError_t ce2 =
-                ce == cudaSuccess
-                    ? cudaGraphInstantiate(&ex, g, cudaGraphInstantiateFlagUseNodePriority)
-                    : ce;
-            if (g) cudaGraphDestroy(g);
-            if (ce2 != cudaSuccess) {
-                cudaGetLastError();
-                pm_set_error("multi-instance solve: cycle graph capture: %s", cudaGetErrorString(ce2));
-                return PM_ERR_CUDA;
-            }
+            PM_TRY(capture_cycle(steps, &ex));
             it = M.graphs.emplace(steps, ex).first;
         }
         PM_CUDA_TRY(cudaGraphLaunch(it->second, st));

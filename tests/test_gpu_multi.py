@@ -132,3 +132,25 @@ def test_workspace_follows_recreated_operators(ctx):
             assert np.abs(u - ref).max() <= 1e-8 * np.abs(ref).max()
         for op in ops:
             op.close()
+
+
+# a cycle's graph: all in its first steps, one short group, whole groups, a last group of one step
+@pytest.mark.parametrize("restart", [2, 6, 7, 10, 11, 50])
+def test_cycle_lengths(ctx, restart):
+    import paper_2401_12501_gb300 as pm
+    o = pm.default_opts()
+    o.gmres_restart = restart
+    wls = [make_workload(n) for n in ("star_small", "sphere_1536")]
+    surfs = [_surface(ctx, wl, opts=o) for wl in wls]
+    solo = [_surface(ctx, wl) for wl in wls]         # a single solve needs longer cycles than 2
+    F = [rhs_set(wl, 2, 11 + i) for i, wl in enumerate(wls)]
+    try:
+        U, infos = pm.solve_multi(surfs, F, tol=1e-10)
+        for wl, s, f, u, inf in zip(wls, solo, F, U, infos):
+            for r in range(f.shape[0]):
+                alone, _ = s.solve(f[r], tol=1e-10, prec="fp32")
+                assert inf[r].residual <= 1e-10
+                assert rel(u[r], alone, wl.surface.weights) < 1e-9
+    finally:
+        for s in surfs + solo:
+            s.close()
