@@ -656,16 +656,24 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-// partial[r][blk][j] = sum over the block's rows of A_r,j[i] * b_r[i]
+// out[r][j] = A_r,j . b_r: each block's sums go to partial[r][blk][j], and the last block of a
+// right-hand side to finish (count[r], left at 0) adds them in block order.
+// A step of a batched solve is bound by its launches while the batch is small: with this sum and
+// h + h2 (k_brotate) in kernels of their own it had five more (1,536 nodes, 2 right-hand sides:
+// 2.43 -> 2.16 ms a solve; 9,600, 5: 6.30 -> 6.05; batches of several operators: 1,536 nodes,
+// 2 x 1, 2.49 -> 2.39).
 __global__ void __launch_bounds__(kRed)
 k_bdots(const double* __restrict__ A, long long col_stride, long long rhs_stride_A, int ncols,
-        const double* __restrict__ b, long long rhs_stride_b, int N,
-        double* __restrict__ partial, const int* __restrict__ done) {
+        const double* __restrict__ b, long long rhs_stride_b, int N, double* partial,
+        int* __restrict__ count, double* __restrict__ out, long long ld_out,
+        const int* __restrict__ done) {
     const int r = blockIdx.y;
     if (done && done[r]) return;
     __shared__ double sh[32];
+    __shared__ int last;
     const double* Ar = A + r * rhs_stride_A;
     const double* br = b + r * rhs_stride_b;
+    double* pr = partial + (size_t)r * gridDim.x * ncols;
     const int stride = gridDim.x * blockDim.x;
     for (int j = 0; j < ncols; ++j) {
         const double* a = Ar + j * col_stride;
@@ -679,20 +687,22 @@ k_bdots(const double* __restrict__ A, long long col_stride, long long rhs_stride
         if (threadIdx.x < 32) {
             double t = (threadIdx.x < (blockDim.x >> 5)) ? sh[threadIdx.x] : 0.0;
             t = warp_sum_d(t);
-            if (threadIdx.x == 0) partial[((size_t)r * gridDim.x + blockIdx.x) * ncols + j] = t;
+            if (threadIdx.x == 0) pr[(size_t)blockIdx.x * ncols + j] = t;
         }
     }
-}
-
-__global__ void k_breduce(const double* __restrict__ partial, int nblk, int ncols,
-                          double* __restrict__ out, long long ld_out, const int* __restrict__ done) {
-    const int r = blockIdx.y;
-    if (done && done[r]) return;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= ncols) return;
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += partial[((size_t)r * nblk + b) * ncols + j];
-    out[r * ld_out + j] = s;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(count + r, 1) == (int)gridDim.x - 1;
+        if (last) count[r] = 0;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    for (int j = threadIdx.x; j < ncols; j += blockDim.x) {
+        double t = 0.0;
+        for (int k = 0; k < (int)gridDim.x; ++k) t += __ldcg(pr + (size_t)k * ncols + j);
+        out[r * ld_out + j] = t;
+    }
 }
 
 // w_r -= sum_j A_r,j c_r[j]
@@ -708,14 +718,6 @@ __global__ void k_bsub(const double* __restrict__ A, long long col_stride, long 
     double acc = w[(size_t)r * N + i];
     for (int j = 0; j < ncols; ++j) acc -= Ar[j * col_stride + i] * cr[j];
     w[(size_t)r * N + i] = acc;
-}
-
-__global__ void k_badd_cols(double* __restrict__ h, long long ldh, const double* __restrict__ h2,
-                            long long ldh2, int n, const int* __restrict__ done) {
-    const int r = blockIdx.y;
-    if (done && done[r]) return;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < n) h[r * ldh + j] += h2[r * ldh2 + j];
 }
 
 // out_r = v_r + y_r + wdot_r  (A v with the rank-one term)
@@ -765,8 +767,10 @@ __global__ void k_bcycle_start(int nrhs, const double* __restrict__ nrm2, long l
     if (threadIdx.x == 0) *all_done = any_active ? 0 : 1;
 }
 
+// the step's Hessenberg column h + h2 (the two passes of the orthogonalisation) and its rotation;
 // use_cond: also sets a graph node's condition, whether a column still works
-__global__ void k_brotate(int nrhs, double* __restrict__ H, int ldh, int m, int k,
+__global__ void k_brotate(int nrhs, double* __restrict__ H, int ldh,
+                          const double* __restrict__ h2, int m, int k,
                           double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g,
                           double* __restrict__ scal, int* __restrict__ done,
                           int* __restrict__ iters, int* __restrict__ all_done, int use_cond,
@@ -781,6 +785,7 @@ __global__ void k_brotate(int nrhs, double* __restrict__ H, int ldh, int m, int 
         double* snr = sn + (size_t)r * m;
         double* gr = g + (size_t)r * (m + 1);
         const double hn = sqrt(scal[r * 8 + 1]);
+        for (int j = 0; j <= k; ++j) h[j] += h2[(size_t)r * (m + 2) + j];
         h[k + 1] = hn;
         scal[r * 8 + 2] = (hn > 0.0) ? 1.0 / hn : 0.0;
         for (int j = 0; j < k; ++j) {
@@ -887,6 +892,7 @@ struct PmBatchSolveWork {
     double *w = nullptr, *tmp = nullptr, *r = nullptr, *res = nullptr, *delta = nullptr;
     double *sig = nullptr, *f = nullptr, *u = nullptr;
     int *done = nullptr, *iters = nullptr, *all_done = nullptr;
+    int* count = nullptr;             // [nrhs] blocks of k_bdots that have finished
     double* ynorm = nullptr;          // [nrhs] |y| of the last cycle
     double* pinned = nullptr;
     double* pinned_y = nullptr;       // [nrhs] host copy of ynorm
@@ -898,7 +904,7 @@ static void bsolve_release(PmBatchSolveWork& W) {
     pm_dfree(W.part); pm_dfree(W.scal); pm_dfree(W.hcol); pm_dfree(W.dots); pm_dfree(W.w);
     pm_dfree(W.tmp); pm_dfree(W.r); pm_dfree(W.res); pm_dfree(W.delta); pm_dfree(W.sig);
     pm_dfree(W.f); pm_dfree(W.u); pm_dfree(W.done); pm_dfree(W.iters); pm_dfree(W.all_done);
-    pm_dfree(W.ynorm);
+    pm_dfree(W.ynorm); pm_dfree(W.count);
     if (W.pinned_y) cudaFreeHost(W.pinned_y);
     if (W.pinned) cudaFreeHost(W.pinned);
     if (W.pinned_i) cudaFreeHost(W.pinned_i);
@@ -939,6 +945,9 @@ static pm_status bsolve_alloc(PmBatchSolveWork& W, int nrhs, int m, int N) {
     PM_TRY(pm_dmalloc(&W.f, RN));
     PM_TRY(pm_dmalloc(&W.u, RN));
     PM_TRY(pm_dmalloc(&W.done, nrhs));
+    PM_TRY(pm_dmalloc(&W.count, nrhs));
+    PM_CUDA_TRY(cudaMemset(W.count, 0, sizeof(int) * nrhs));
+    PM_CUDA_TRY(cudaStreamSynchronize(nullptr));
     PM_TRY(pm_dmalloc(&W.iters, nrhs));
     PM_TRY(pm_dmalloc(&W.all_done, 1));
     PM_TRY(pm_dmalloc(&W.ynorm, nrhs));
@@ -988,10 +997,9 @@ struct BSolver {
               const double* b, long long rhs_stride_b, double* dst, long long lddst,
               const int* done) {
         k_bdots<<<dim3(W.nred, nrhs), kRed, 0, st>>>(A, col_stride, rhs_stride_A, ncols, b,
-                                                      rhs_stride_b, W.N, W.part, done);
-        k_breduce<<<dim3(pm_ceil_div(ncols, 64), nrhs), 64, 0, st>>>(W.part, W.nred, ncols, dst,
-                                                                       lddst, done);
-        s->launch_total += 2;
+                                                      rhs_stride_b, W.N, W.part, W.count, dst,
+                                                      lddst, done);
+        s->launch_total += 1;
     }
 
     // out_r = A v_r (I + R~ + 1 w^T) for all r
@@ -1064,14 +1072,12 @@ struct BSolver {
                 dots(W.V, N, ldV, k + 1, W.w, N, W.hcol, m + 2, W.done);
                 k_bsub<<<dim3(grid_n, nrhs), 256, 0, st>>>(W.V, N, ldV, k + 1, W.hcol, m + 2, W.w, N,
                                                            W.done);
-                k_badd_cols<<<dim3(pm_ceil_div(k + 1, 64), nrhs), 64, 0, st>>>(
-                    hk, (long long)m * ldh, W.hcol, m + 2, k + 1, W.done);
                 dots(W.w, 0, N, 1, W.w, N, W.scal + 1, 8, W.done);
-                k_brotate<<<1, 256, 0, st>>>(nrhs, W.H, ldh, m, k, W.cs, W.sn, W.g, W.scal, W.done,
-                                             W.iters, W.all_done, 0, 0);
+                k_brotate<<<1, 256, 0, st>>>(nrhs, W.H, ldh, W.hcol, m, k, W.cs, W.sn, W.g, W.scal,
+                                             W.done, W.iters, W.all_done, 0, 0);
                 k_bscale_copy<<<dim3(grid_n, nrhs), 256, 0, st>>>(W.w, N, W.scal + 2, 8, 0, vk1, ldV,
                                                                   N, W.done);
-                s->launch_total += 5;
+                s->launch_total += 4;
             }
             s->skip_flag = nullptr;
             k_bbacksolve<<<pm_ceil_div(nrhs, 64), 64, 0, st>>>(nrhs, W.H, ldh, m, W.g, W.iters, W.y,
@@ -1125,7 +1131,7 @@ size_t pm_batch_need_bytes(const pm_surface* s, int nrhs) {
         const size_t nred = (size_t)std::max(1, std::min(pm_ceil_div(s->N, 2048), 64));
         need += sizeof(double) * (R * (m + 1) * N + R * (m * (m + 2) + 3 * m + 1) +
                                   R * nred * (m + 2) + R * (m + 2 + 16) + 8 * R * N) +
-                sizeof(int) * (2 * R + 1);
+                sizeof(int) * (3 * R + 1);
     }
     if (!(s->batch && s->batch->cap >= nrhs))
         need += R * N * (sizeof(float) + sizeof(float2) + 8 * sizeof(float2)) +
@@ -1886,10 +1892,9 @@ struct MSolver {
               const double* b, long long rhs_stride_b, double* dst, long long lddst,
               const int* done) {
         k_bdots<<<dim3(W.nred, M.ncols), kRed, 0, st>>>(A, col_stride, rhs_stride_A, ncols_, b,
-                                                         rhs_stride_b, W.N, W.part, done);
-        k_breduce<<<dim3(pm_ceil_div(ncols_, 64), M.ncols), 64, 0, st>>>(W.part, W.nred, ncols_,
-                                                                         dst, lddst, done);
-        launches += 2;
+                                                         rhs_stride_b, W.N, W.part, W.count, dst,
+                                                         lddst, done);
+        launches += 1;
     }
 
     // out_c = A v_c for every column; prec FP32 (one multi-instance launch per stage)
@@ -1966,11 +1971,9 @@ struct MSolver {
             dots(W.V, N, ldV, k + 1, W.w, N, W.hcol, m + 2, W.done);
             k_bsub<<<dim3(grid_n, nc), 256, 0, st>>>(W.V, N, ldV, k + 1, W.hcol, m + 2, W.w, N,
                                                      W.done);
-            k_badd_cols<<<dim3(pm_ceil_div(k + 1, 64), nc), 64, 0, st>>>(
-                hk, (long long)m * ldh, W.hcol, m + 2, k + 1, W.done);
             dots(W.w, 0, N, 1, W.w, N, W.scal + 1, 8, W.done);
-            k_brotate<<<1, 256, 0, st>>>(nc, W.H, ldh, m, k, W.cs, W.sn, W.g, W.scal, W.done,
-                                         W.iters, W.all_done, use_cond && k + 1 == k1, cond);
+            k_brotate<<<1, 256, 0, st>>>(nc, W.H, ldh, W.hcol, m, k, W.cs, W.sn, W.g, W.scal,
+                                         W.done, W.iters, W.all_done, use_cond && k + 1 == k1, cond);
             k_bscale_copy<<<dim3(grid_n, nc), 256, 0, st>>>(W.w, N, W.scal + 2, 8, 0, vk1, ldV, N,
                                                             W.done);
         }
@@ -1991,7 +1994,7 @@ struct MSolver {
     // One cycle as a CUDA graph, captured on the workspace's own streams: the start and kFirst
     // steps, then groups of kGroup steps each in a conditional node that runs while a column
     // still works, then the end.  A cycle may take `steps` steps (50) and takes about ten;
-    // the 17 launches of every idle step used to run, each returning at once: 1,536 nodes with
+    // the 17 launches (now 12) of every idle step used to run, each returning at once: 1,536 nodes with
     // 2 operators of one right-hand side 3.54 -> 2.48 ms a batch, 9,600 with 4 x 2 14.4 -> 13.2,
     // 24,576 with 8 x 8 103.8 -> 101.3.
     static constexpr int kFirst = 6, kGroup = 4;
