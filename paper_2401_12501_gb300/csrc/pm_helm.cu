@@ -351,7 +351,8 @@ struct HelmDense {
     }
     // 32 N^2 bytes.  One evaluation of the pairs serves every step, residual and the
     // representation; the pair sums evaluate all of them each time.  A solve to 1e-12 on the
-    // GB300: 3,456 nodes with c/a > 0 206 -> 14.7 ms, 864 nodes with complex c 878 -> 28.7 ms.
+    // GB300: 3,456 nodes with c/a > 0 206 -> 14.7 ms, 864 nodes with complex c 878 -> 28.7 ms
+    // (7.1 and 2.0 ms with the kernels from tables and the steps of pm_arnoldi.cuh).
     pm_status fill(pm_surface* s) {
         const size_t N = s->N, need = 2 * sizeof(double2) * N * N;
         size_t fr = 0, total = 0;

@@ -394,7 +394,7 @@ __global__ void k_combine(int nblk, int pp, int ppad, const int* __restrict__ bl
 // The kernels depend on the source through k(y)^2 = q(y) = c(y)/a(y), which is
 // interpolated on the patch from its nodes with the tensor Lagrange basis, so
 // these weights hold the coefficients and are built per coefficient field.
-// Self patch: the polar rule of k_self_quad, with dyadic radial panels
+// Self patch: the polar rule of the real weights, with dyadic radial panels
 // [0, L 2^-12], [L 2^-12, L 2^-11], ..., [L/2, L] in place of the product-log
 // panel: here g = log(r) A(r) + B(r) with A = J0(kr) or I0(kr) not constant, and
 // R has r log r terms (Thm. remainder); each graded panel sees an analytic
@@ -506,7 +506,7 @@ k_self_quad_c(int N, int p, const double* __restrict__ x, const double* __restri
     }
 }
 
-// Near, non-self patches: the subdivision of k_near_quad, 16 x 16 Gauss points
+// Near, non-self patches: the subdivision of the real weights, 16 x 16 Gauss points
 // per leaf, the target's given normal.
 __global__ void __launch_bounds__(kQThreads)
 k_near_quad_c(int p, const double* __restrict__ x, const double* __restrict__ J,
@@ -862,7 +862,7 @@ __global__ void k_tile_radius(const double* __restrict__ x, int N, int tile,
 // 16-point Gauss in theta and on each radial panel: [0, L/4], [L/4, L] for the
 // gradient kernel (after the polar Jacobian its integrand is smooth), dyadic panels
 // [2^-(k+1), 2^-k] L, k < 18, and [0, 2^-18 L] for the log kernel (rho log rho).
-// own == 0: the quadtree near rule about x = x_e as in k_near_quad.
+// own == 0: the quadtree near rule of the surface weights about x = x_e.
 constexpr int kBvpPts = 128;          // quadrature points per pass of the polar rule
 constexpr int kBvpLogLevels = 18;     // dyadic radial panels of the log-kernel polar rule
 
