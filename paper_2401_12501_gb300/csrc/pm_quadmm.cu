@@ -398,14 +398,15 @@ struct Buffers {
 };
 
 // Room for a batch's table and slots.  Larger batches leave fewer half-empty last waves; these
-// keep what a build takes beside its results below 0.4 GB.
+// keep what a build takes beside its results below 0.4 GB.  On a device without that much left
+// the batches are halved, up to five times; the weights do not depend on it.
 constexpr size_t kTableBytes = 192u << 20, kSlotBytes = 128u << 20;
 
 }  // namespace
 
 namespace {
 
-pm_status weights(pm_surface* s, const QmRules& R, int eB, bool* over);
+pm_status weights(pm_surface* s, const QmRules& R, int eB, int halved, bool* over);
 
 }  // namespace
 
@@ -430,10 +431,18 @@ pm_status pm_quad_weights(pm_surface* s, const QmRules& R) {
     float ftop = 0.f;
     std::memcpy(&ftop, &top, sizeof(ftop));
     int eB = (int)std::ceil(std::log2(std::min(1e30, std::max(1.0, 3.0 * (double)ftop))));
-    for (;; eB += 3) {
+    int halved = 0;
+    for (;;) {
         bool over = false;
-        PM_TRY(weights(s, R, eB, &over));
+        const pm_status st = weights(s, R, eB, halved, &over);
+        if (st == PM_ERR_OOM && halved < 5) {
+            cudaGetLastError();
+            ++halved;
+            continue;
+        }
+        PM_TRY(st);
         if (!over) return PM_OK;
+        eB += 3;
         if (eB > 200) {
             pm_set_error("near-field weights: basis values above 2^%d", eB);
             return PM_ERR_INTERNAL;
@@ -443,7 +452,7 @@ pm_status pm_quad_weights(pm_surface* s, const QmRules& R) {
 
 namespace {
 
-pm_status weights(pm_surface* s, const QmRules& R, int eB, bool* over) {
+pm_status weights(pm_surface* s, const QmRules& R, int eB, int halved, bool* over) {
     const int n = R.n, npatch = s->npatch;
     QmTable T;
     T.n = n;
@@ -452,8 +461,8 @@ pm_status weights(pm_surface* s, const QmRules& R, int eB, bool* over) {
     const size_t tile_bytes = (size_t)kQmDigits * kQmPts * T.npad * 2 + kQmPts * sizeof(double2);
     int max_loc = 0;
     for (int l = 0; l < n; ++l) max_loc = std::max(max_loc, R.tiles[l + 1] - R.tiles[l]);
-    const int cap_tiles = std::max<int>(std::max(max_loc, R.near_tiles), (int)(kTableBytes / tile_bytes));
-    const int cap_slots = (int)std::max<size_t>(4096, kSlotBytes / (5 * (size_t)n * sizeof(double)));
+    const int cap_tiles = std::max<int>(std::max(max_loc, R.near_tiles), (int)((kTableBytes >> halved) / tile_bytes));
+    const int cap_slots = (int)std::max<size_t>(4096, (kSlotBytes >> halved) / (5 * (size_t)n * sizeof(double)));
     Buffers B;
     double* partial = nullptr;
     PM_TRY(B.get(&T.dig, (size_t)cap_tiles * kQmDigits * kQmPts * T.npad));
@@ -492,7 +501,8 @@ pm_status weights(pm_surface* s, const QmRules& R, int eB, bool* over) {
         int l1 = l0 + 1;
         while (l1 < n && R.tiles[l1 + 1] - R.tiles[l0] <= cap_tiles) ++l1;
         PM_TRY(R.self_table(l0, l1 - l0, T));
-        const int pieces = std::max(1, std::min(max_loc / 4, pm_ceil_div(want, (long long)ngroup * (l1 - l0))));
+        const int pieces = std::max(1, std::min({max_loc / 4, pm_ceil_div(want, (long long)ngroup * (l1 - l0)),
+                                                 cap_slots / ((l1 - l0) * kQmCols)}));
         // patches at a time that the slots hold (all but on very large surfaces)
         const int gstep = std::max(1, (int)std::min<long long>(ngroup, cap_slots / ((long long)(l1 - l0) * pieces * kQmCols)));
         for (int g0 = 0; g0 < ngroup; g0 += gstep) {
