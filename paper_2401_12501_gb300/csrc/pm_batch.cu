@@ -565,10 +565,8 @@ pm_status pm_apply_batch(pm_surface* s, int kernel_K, const double* sigma, long 
         bool summed = false;
         if (nrhs >= kFfmmMin) {
             PhaseTimer t(s, kernel_K ? PM_PHASE_DIRECT64_K : PM_PHASE_DIRECT64, st);
-            const pm_status r = pm_ffmm_sum(s, &B.fm, kernel_K ? PM_FFMM_K : PM_FFMM_R, 1, &s, &nrhs,
-                                            &sigma, ld_sigma, ns, B.part, st);
-            if (r != PM_OK && r != PM_ERR_OOM) return r;      // no room for its buffers: as below
-            summed = r == PM_OK;
+            PM_TRY(pm_ffmm_sum(s, &B.fm, kernel_K ? PM_FFMM_K : PM_FFMM_R, 1, &s, &nrhs, &sigma, ld_sigma,
+                               ns, B.part, &summed, st));
         }
         if (!summed) ns = batch_splits(s, nrhs, rbff, 8);
         if (!summed) {
@@ -2146,10 +2144,8 @@ pm_status multi_representation_ff(pm_surface* const* ops, int nops, const int* n
             if (cols >= kFfmmMin) {
                 std::vector<const double*> sg;
                 for (int q = k; q < k1; c += nrhs[q++]) sg.push_back(sig + (size_t)(c0 + c) * ld);
-                const pm_status r = pm_ffmm_sum(s0, &B.fm, PM_FFMM_K, k1 - k, ops + k, nrhs + k, sg.data(),
-                                                ld, ns, B.part, st);
-                if (r != PM_OK && r != PM_ERR_OOM) return r;
-                summed = r == PM_OK;
+                PM_TRY(pm_ffmm_sum(s0, &B.fm, PM_FFMM_K, k1 - k, ops + k, nrhs + k, sg.data(), ld, ns, B.part,
+                                   &summed, st));
             }
             if (!summed) {
                 ns = batch_splits(s0, cols, rbff, 8);
@@ -2214,10 +2210,8 @@ pm_status multi_remainder_ff(pm_surface* const* ops, int nops, const int* nrhs,
             const int ns = ffmm_splits(s0, 16);
             std::vector<const double*> sg;
             for (int q = k; q < k1; ++q) sg.push_back(sig + (size_t)col[q] * ld);
-            const pm_status r = pm_ffmm_sum(s0, &B.fm, PM_FFMM_RG, k1 - k, ops + k, nrhs + k, sg.data(), ld,
-                                            ns, B.part, st);
-            if (r != PM_OK && r != PM_ERR_OOM) return r;
-            summed = r == PM_OK;
+            PM_TRY(pm_ffmm_sum(s0, &B.fm, PM_FFMM_RG, k1 - k, ops + k, nrhs + k, sg.data(), ld, ns, B.part,
+                               &summed, st));
             for (int q = k; summed && q < k1; ++q) {
                 const dim3 gn(pm_ceil_div((long long)s0->N * 32, 256), nrhs[q]);
                 k_near_multi64<<<gn, 256, 0, st>>>(

@@ -5,7 +5,12 @@
 // instructions a pair and column in k_direct_multi_ff (pm_batch.cu), are integer arithmetic on
 // the tensor cores, as in pm_quadmm.cu: entries and strengths in 54-bit fixed point (a power of
 // two per target row, bounded over its pairs once per surface, and per column), six base-512
-// digits in float16, float32 sums of 128 sources at a time, exact integers, added up in 64 bits.
+// digits in float16, float32 sums of 128 sources at a time, added up in 64 bits.  Those sums are
+// integers, exact below 2^24: the two of largest weight always (128 256^2 and twice that), the
+// others, of three products a source and more, unless nearly all digits of both operands sit at
+// their extremes, which would cost 2^-24 of a sum that weighs 512^-2 or less.
+// Surfaces whose nodes lie so unevenly that a row's largest entry dwarfs the rest of it, or with
+// fewer nodes than a stage, keep k_direct_multi_ff (kFmSpread; pm_batch.cu kFfmmNodes).
 // Of the digit products the remainder's matrices keep the 26 above 2^-58 of the scale, for a row's
 // nearest neighbours set the scale and stand far above the rest of it; log r^2 varies little and
 // keeps 21 (2^-54).
@@ -41,6 +46,15 @@ constexpr int kKS = kFmK / 16;
 constexpr int kFmCols = 64;
 constexpr size_t kBufWords = (size_t)4 * kKS * kQmDigits * 4 * 32;
 constexpr int kRecord = 20;                // floats of a target in shared memory
+// The remainder's fixed point serves while no row's largest |q^2 - H q| or 1/r stands more than
+// this factor above the row's mean over the surface: every entry of a row is rounded to some 2^-54
+// of its largest, a typical one to S 2^-54 of itself at a factor S, and float-float arithmetic
+// rounds each to about 2^-44.  Surfaces of even patches have 2^5 to 2^10.5 (1,500 to 400,000
+// nodes); patches halved towards a point pass 2^11 at a size of 2^-8.  Errors against float64
+// over those of k_direct_multi_ff, 8 columns: 0.1 to 0.2 at 2^8 (24,576 nodes of a torus), 0.4 to
+// 0.7 at 2^10.7 (flat ellipsoid, 21,600), 0.7 to 1.3 at 2^15.5 and 49 to 53 at 2^21.5 (patches
+// halved 12 and 18 times).  log r^2 has no such rows and is taken whenever it is defined.
+constexpr float kFmSpread = 2048.f;
 
 // Columns of one launch: operators in order, first[q] <= column < first[q + 1]
 struct Cols {
@@ -54,42 +68,90 @@ __device__ __forceinline__ int op_of(const Cols& C, int col) {
     return q;
 }
 
-// Each target's largest |q^2 - H q| (top[i]) and 1/r (top[N + i]) over its pairs, and the largest
-// |log r^2| of all (top[2 N]), in float32.
+// What the fixed point of a row is laid out for, by target i: its pairs' largest |q^2 - H q| and
+// 1/r, their means over the surface and the largest |log r^2|, of the sources of one split;
+// part[(split 5 + k) N + i] in the order max, max, sum, sum, max, and the sources' weights in
+// area[split N + i].  The differences and n.r are those of the sums (float-float): n.r is of the
+// order r^2, and of coordinates rounded to float32 its error grows past it where nodes are close.
 __global__ void __launch_bounds__(128)
-k_fm_top(const double* __restrict__ x, const double* __restrict__ n, const double* __restrict__ H,
-         int N, unsigned int* __restrict__ top) {
-    __shared__ float sx[128][3];
+k_fm_rows(const float4* __restrict__ src, const double* __restrict__ nrm, const double* __restrict__ H,
+          const double* __restrict__ w, int N, int chunk, float* __restrict__ part,
+          float* __restrict__ area) {
+    __shared__ float4 sa[128], sb[128];
     const int i = blockIdx.x * 128 + threadIdx.x, ii = min(i, N - 1);
-    float X[3], M[3];
-    for (int d = 0; d < 3; ++d) {
-        X[d] = (float)x[3 * ii + d];
-        M[d] = (float)n[3 * ii + d];
-    }
+    const float4 ta = src[2 * (size_t)ii], tb = src[2 * (size_t)ii + 1];
+    ff n[3];
+    for (int d = 0; d < 3; ++d) n[d] = ff_from_double(nrm[3 * (size_t)ii + d]);
     const float h = (float)H[ii];
-    float t0 = 0.f, t1 = 0.f, t2 = 0.f;
-    for (int base = blockIdx.y * 128; base < N; base += gridDim.y * 128) {
+    float top0 = 0.f, top1 = 0.f, toplog = 0.f, sum0 = 0.f, sum1 = 0.f, sw = 0.f;
+    const int s0 = blockIdx.y * chunk, s1 = min(s0 + chunk, N);
+    for (int base = s0; base < s1; base += 128) {
         __syncthreads();
         const int j = min(base + (int)threadIdx.x, N - 1);
-        for (int d = 0; d < 3; ++d) sx[threadIdx.x][d] = (float)x[3 * j + d];
+        sa[threadIdx.x] = src[2 * (size_t)j];
+        sb[threadIdx.x] = src[2 * (size_t)j + 1];
+        sb[threadIdx.x].w = (float)w[j];
         __syncthreads();
-        const int len = min(128, N - base);
+        const int len = min(128, s1 - base);
         for (int k = 0; k < len; ++k) {
-            const float a = X[0] - sx[k][0], b = X[1] - sx[k][1], c = X[2] - sx[k][2];
-            const float r2 = a * a + b * b + c * c;
-            if (base + k == ii || !(r2 > 0.f)) continue;
-            const float inv = 1.f / r2, q = (M[0] * a + M[1] * b + M[2] * c) * inv;
-            t0 = fmaxf(t0, fabsf(q * (q - h)));
-            t1 = fmaxf(t1, inv);
-            t2 = fmaxf(t2, fabsf(__logf(r2)));
+            if (base + k == ii) continue;
+            const float4 a = sa[k], b = sb[k];
+            const ff dx = ff_sub(ff{ta.x, tb.x}, ff{a.x, b.x}), dy = ff_sub(ff{ta.y, tb.y}, ff{a.y, b.y}),
+                     dz = ff_sub(ff{ta.z, tb.z}, ff{a.z, b.z});
+            const float r2 = fmaf(dx.h, dx.h, fmaf(dy.h, dy.h, dz.h * dz.h)), inv = 1.f / r2;
+            const ff nr = ff_norm(ff_add_lazy(ff_add_lazy(ff_mul_lazy(n[0], dx), ff_mul_lazy(n[1], dy)),
+                                              ff_mul_lazy(n[2], dz)));
+            const float q = nr.h * inv, e0 = fabsf(q * (q - h)), e1 = sqrtf(inv);
+            sum0 = fmaf(b.w, e0, sum0);          // an undefined pair leaves the sums undefined
+            sum1 = fmaf(b.w, e1, sum1);
+            sw += b.w;
+            top0 = fmaxf(top0, e0);
+            top1 = fmaxf(top1, e1);
+            toplog = fmaxf(toplog, fabsf(__logf(r2)));
         }
     }
-    if (i < N) {
-        atomicMax(top + i, __float_as_uint(t0));
-        atomicMax(top + N + i, __float_as_uint(sqrtf(t1)));
+    if (i >= N) return;
+    float* p = part + (size_t)blockIdx.y * 5 * N + i;
+    p[0] = top0;
+    p[N] = top1;
+    p[2 * (size_t)N] = sum0;
+    p[3 * (size_t)N] = sum1;
+    p[4 * (size_t)N] = toplog;
+    area[(size_t)blockIdx.y * N + i] = sw;
+}
+
+// bound[i], bound[N + i], bound[2 N]: the largest |q^2 - H q| and 1/r of target i and the largest
+// |log r^2| of all; bound[2 N + 1]: how far a row's largest entry stands above the row's mean, at
+// worst (infinity where a pair is undefined)
+__global__ void k_fm_bounds(int N, int nsplit, const float* __restrict__ part,
+                            const float* __restrict__ area, unsigned int* __restrict__ bound) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    float top0 = 0.f, top1 = 0.f, toplog = 0.f, sum0 = 0.f, sum1 = 0.f, sw = 0.f;
+    for (int s = 0; s < nsplit && i < N; ++s) {
+        const float* p = part + (size_t)s * 5 * N + i;
+        top0 = fmaxf(top0, p[0]);
+        top1 = fmaxf(top1, p[N]);
+        sum0 += p[2 * (size_t)N];
+        sum1 += p[3 * (size_t)N];
+        toplog = fmaxf(toplog, p[4 * (size_t)N]);
+        sw += area[(size_t)s * N + i];
     }
-    for (int o = 16; o > 0; o >>= 1) t2 = fmaxf(t2, __shfl_xor_sync(0xffffffffu, t2, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(top + 2 * (size_t)N, __float_as_uint(t2));
+    float over = 0.f;
+    if (i < N) {
+        bound[i] = __float_as_uint(top0);
+        bound[N + i] = __float_as_uint(top1);
+        const bool defined = sum0 < 3e38f && sum1 < 3e38f && sw > 0.f;
+        over = !defined && N > 1 ? __int_as_float(0x7f800000)
+                                 : fmaxf(top0 > 0.f ? top0 * sw / sum0 : 0.f, top1 > 0.f ? top1 * sw / sum1 : 0.f);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        over = fmaxf(over, __shfl_xor_sync(0xffffffffu, over, o));
+        toplog = fmaxf(toplog, __shfl_xor_sync(0xffffffffu, toplog, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(bound + 2 * (size_t)N, __float_as_uint(toplog));
+        atomicMax(bound + 2 * (size_t)N + 1, __float_as_uint(over));
+    }
 }
 
 // E with a bit to spare: bound < 2^(E - 1)
@@ -141,8 +203,9 @@ k_fm_strengths(Cols C, int N, int Npad, const int* __restrict__ top, unsigned in
             qm_digit2(v[0], v[1], d);
 }
 
-// The base-512 digits of (h + l) 2^(8 - E), the first in [-256, 256], as floats: three from h, then
-// three from what is left of it and l, so that they hold the value to 2^-51 of the scale.
+// The base-512 digits of (h + l) 2^(8 - E) as floats: three from h, then three from what is left of
+// it and l, so that they hold the value to 2^-51 of the scale.  All lie in [-256, 256] but the
+// fourth, which takes in l and may reach 512 (float16 holds integers to 2,048).
 struct FloatDigits {
     float r, l;
     __device__ __forceinline__ FloatDigits(ff v, int E) {
@@ -405,7 +468,7 @@ pm_status launch(pm_surface* s, const PmFfmmWork& W, const Cols& C, int nsplit, 
 static size_t digit_words(int N) {
     return (size_t)pm_ceil_div(N, kFmK) * kFmK / 16 * 8 * kQmDigits * 64;
 }
-static size_t bound_words(int N) { return 2 * (size_t)N + 1; }
+static size_t bound_words(int N) { return 2 * (size_t)N + 2; }
 
 size_t pm_ffmm_bytes(int N) { return (digit_words(N) + bound_words(N) + kFmCols) * sizeof(int); }
 
@@ -415,33 +478,52 @@ void pm_ffmm_free(PmFfmmWork* W) {
     pm_dfree(W->bound);
 }
 
-// Buffers and the geometry's bounds; PM_ERR_OOM leaves W empty and no error behind, and the
-// caller takes the sums without buffers -- as it does on a stream under capture, where nothing
-// can be allocated
-static pm_status ffmm_ready(pm_surface* s, PmFfmmWork* W, cudaStream_t st) {
+// Buffers and the geometry's bounds (waits for them, once a workspace).  *room false: no room for
+// the buffers, or a stream under capture, where nothing can be allocated; no error is left behind.
+static pm_status ffmm_ready(pm_surface* s, PmFfmmWork* W, bool* room, cudaStream_t st) {
+    *room = true;
     if (W->S) return PM_OK;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     PM_CUDA_TRY(cudaStreamIsCapturing(st, &capture));
-    if (capture != cudaStreamCaptureStatusNone) return PM_ERR_OOM;
-    pm_status r = pm_dmalloc(&W->S, digit_words(s->N));
+    *room = capture == cudaStreamCaptureStatusNone;
+    if (!*room) return PM_OK;
+    const int N = s->N;
+    pm_status r = pm_dmalloc(&W->S, digit_words(N));
     if (r == PM_OK) r = pm_dmalloc(&W->top, kFmCols);
-    if (r == PM_OK) r = pm_dmalloc(&W->bound, bound_words(s->N));
+    if (r == PM_OK) r = pm_dmalloc(&W->bound, bound_words(N));
     if (r == PM_OK) {
-        cudaMemsetAsync(W->bound, 0, bound_words(s->N) * sizeof(int), st);
-        const int blocks = pm_ceil_div(s->N, 128);
-        k_fm_top<<<dim3(blocks, std::max(1, std::min(blocks, 4 * s->ctx->num_sms / blocks))), 128, 0, st>>>(
-            s->x, s->n, s->H, s->N, W->bound);
-        if (cudaGetLastError() != cudaSuccess) r = PM_ERR_CUDA;
+        const int blocks = pm_ceil_div(N, 128);
+        const int ns = std::max(1, std::min({blocks, 16 * s->ctx->num_sms / blocks, 24}));
+        const int chunk = pm_ceil_div(pm_ceil_div(N, ns), 128) * 128;
+        // 6 ns N values in the digits' room of 192 N and more
+        float *part = reinterpret_cast<float*>(W->S), *area = part + (size_t)5 * ns * N;
+        cudaMemsetAsync(W->bound, 0, bound_words(N) * sizeof(int), st);
+        k_fm_rows<<<dim3(blocks, ns), 128, 0, st>>>(s->src_ff, s->n, s->H, s->w, N, chunk, part, area);
+        k_fm_bounds<<<blocks, 128, 0, st>>>(N, ns, part, area, W->bound);
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&W->spread, W->bound + 2 * (size_t)N + 1, sizeof(float), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) {
+            pm_set_error("bounds of the float-float sums: %s", cudaGetErrorString(e));
+            r = PM_ERR_CUDA;
+        }
     }
     if (r != PM_OK) pm_ffmm_free(W);
-    if (r == PM_ERR_OOM) cudaGetLastError();
+    if (r == PM_ERR_OOM) {
+        cudaGetLastError();
+        *room = false;
+        return PM_OK;
+    }
     return r;
 }
 
 pm_status pm_ffmm_sum(pm_surface* s, PmFfmmWork* W, int kind, int nops, pm_surface* const* ops,
                       const int* ncols, const double* const* sigma, long long ld, int nsplit,
-                      float2* partial, cudaStream_t st) {
-    PM_TRY(ffmm_ready(s, W, st));
+                      float2* partial, bool* summed, cudaStream_t st) {
+    PM_TRY(ffmm_ready(s, W, summed, st));
+    *summed = *summed && W->spread <= (kind == kK ? 1e30f : kFmSpread);
+    if (!*summed) return PM_OK;
     // launches of at most kFmCols columns of at most PM_FFMM_OPS operators
     int q = 0, done = 0;                 // operator, its columns already taken
     size_t out = 0;                      // first column of the launch

@@ -314,14 +314,16 @@ struct PmFfmmWork {
     unsigned int* S = nullptr;      // the strengths' digits
     int* top = nullptr;             // per column: exponent of the largest strength
     unsigned int* bound = nullptr;  // the geometry's largest kernel values by target
+    float spread = 0.f;             // a target's largest value over its mean, at worst
 };
 void pm_ffmm_free(PmFfmmWork* W);
 size_t pm_ffmm_bytes(int N);        // device bytes of its buffers
 // partial[(column nsplit + split) N + i] for the columns of ops[0..nops) (all on s's geometry;
-// PM_FFMM_R: one operator), sigma[q] + r ld operator q's column r
+// PM_FFMM_R: one operator), sigma[q] + r ld operator q's column r.  *summed false: nothing was
+// done, for the geometry's nodes lie too unevenly or there is no room for the buffers
 pm_status pm_ffmm_sum(pm_surface* s, PmFfmmWork* W, int kind, int nops, pm_surface* const* ops,
                       const int* ncols, const double* const* sigma, long long ld, int nsplit,
-                      float2* partial, cudaStream_t st);
+                      float2* partial, bool* summed, cudaStream_t st);
 
 // free device memory now (cudaMemGetInfo), or the value of the environment variable
 // PM_FAKE_HBM_BYTES when set (a host-side stand-in for a full device) (pm_api.cu)
