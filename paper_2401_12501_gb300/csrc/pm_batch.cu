@@ -483,7 +483,12 @@ static int batch_splits(const pm_surface* s, int nrhs, int rb, int bps) {
 
 // Float-float sums of this many columns and more go to the tensor cores (pm_ffmm.cu): there a
 // pair costs about the same from 1 to 64 columns, in k_direct_multi_ff 12 instructions a column.
-constexpr int kFfmmMin = 8;
+// The products take 128 sources at a time, and below one such stage there is nothing to share.
+// Applies of 8 columns, us, k_direct_multi_ff -> tensor cores: R 32 -> 37, K 24 -> 34 at 54 nodes;
+// R 63 -> 37, K 45 -> 34 at 150; R 115 -> 66 at 1,536; R 228 -> 206 at 3,456; R 505 -> 431 at
+// 6,144; R 3,485 -> 3,252 at 18,150.
+constexpr int kFfmmMin = 8, kFfmmNodes = 128;
+static bool ffmm_takes(const pm_surface* s, int cols) { return cols >= kFfmmMin && s->N >= kFfmmNodes; }
 
 // Source splits of the tensor-core sums, one block an SM: the split whose blocks of `targets`
 // rows fill whole rounds best.
@@ -563,7 +568,7 @@ pm_status pm_apply_batch(pm_surface* s, int kernel_K, const double* sigma, long 
         const int rbff = nrhs <= 8 ? 8 : kRBff;
         int ns = ffmm_splits(s, 64);
         bool summed = false;
-        if (nrhs >= kFfmmMin) {
+        if (ffmm_takes(s, nrhs)) {
             PhaseTimer t(s, kernel_K ? PM_PHASE_DIRECT64_K : PM_PHASE_DIRECT64, st);
             PM_TRY(pm_ffmm_sum(s, &B.fm, kernel_K ? PM_FFMM_K : PM_FFMM_R, 1, &s, &nrhs, &sigma, ld_sigma,
                                ns, B.part, &summed, st));
@@ -1134,7 +1139,7 @@ size_t pm_batch_need_bytes(const pm_surface* s, int nrhs) {
     if (!(s->batch && s->batch->cap >= nrhs))
         need += R * N * (sizeof(float) + sizeof(float2) + 8 * sizeof(float2)) +
                 R * (size_t)s->npatch * s->ppad * sizeof(float);
-    if (nrhs >= kFfmmMin && !(s->batch && s->batch->cap >= nrhs && s->batch->fm.S))
+    if (ffmm_takes(s, nrhs) && !(s->batch && s->batch->cap >= nrhs && s->batch->fm.S))
         need += pm_ffmm_bytes(s->N);
     return need;
 }
@@ -2141,7 +2146,7 @@ pm_status multi_representation_ff(pm_surface* const* ops, int nops, const int* n
             const int rbff = cols <= 8 ? 8 : kRBff;
             int ns = ffmm_splits(s0, 64), c = 0;
             bool summed = false;
-            if (cols >= kFfmmMin) {
+            if (ffmm_takes(s0, cols)) {
                 std::vector<const double*> sg;
                 for (int q = k; q < k1; c += nrhs[q++]) sg.push_back(sig + (size_t)(c0 + c) * ld);
                 PM_TRY(pm_ffmm_sum(s0, &B.fm, PM_FFMM_K, k1 - k, ops + k, nrhs + k, sg.data(), ld, ns, B.part,
@@ -2204,7 +2209,7 @@ pm_status multi_remainder_ff(pm_surface* const* ops, int nops, const int* nrhs,
         while (k1 < nops && which[k1] && ops[k1]->x == ops[k]->x) ++k1;
         pm_surface* s0 = ops[k];
         bool summed = false;
-        if (k1 - k >= kRGMin) {
+        if (k1 - k >= kRGMin && s0->N >= kFfmmNodes) {
             PM_TRY(batch_ensure(s0, col[k1] - col[k]));
             PmBatchWork& B = *s0->batch;
             const int ns = ffmm_splits(s0, 16);
