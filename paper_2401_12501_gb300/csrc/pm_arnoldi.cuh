@@ -132,7 +132,6 @@ struct Steps {
     double* nrm = nullptr;
     cudaEvent_t ev[2] = {nullptr, nullptr};
 
-    static double positive(double v) { return v > 0.0 ? v : 0.0; }      // an undefined norm ends a cycle
     size_t slot() const { return 2 * (size_t)(m + 1) + 1; }
     pm_status create(int n_, int m_) {
         n = n_;
@@ -157,14 +156,15 @@ struct Steps {
             e = nullptr;
         }
     }
-    // V_0 = r / |r|, and |r| (waits for it)
+    // V_0 = r / |r|, and |r| (waits for it), NaN or infinite where r is or its squares overflow: a
+    // solve that met one has not converged
     pm_status begin(T* r, T* V0, cudaStream_t st, double* beta) {
         k_subtract<T><<<nblk, kThreads, 0, st>>>(nullptr, 0, 0, nullptr, 0, nullptr, r, n, nrm);
         k_next<T><<<nblk, kThreads, 0, st>>>(r, n, nrm, nblk, V0, reinterpret_cast<double*>(dev));
         PM_CUDA_TRY(cudaGetLastError());
         PM_CUDA_TRY(cudaMemcpyAsync(host, dev, sizeof(double), cudaMemcpyDeviceToHost, st));
         PM_CUDA_TRY(cudaStreamSynchronize(st));
-        *beta = positive(*reinterpret_cast<const double*>(host));
+        *beta = *reinterpret_cast<const double*>(host);
         return PM_OK;
     }
     // x += sum_{j < k} V_j y_j with y on the host (the stream's earlier steps have been waited for,
@@ -194,11 +194,13 @@ struct Steps {
         PM_CUDA_TRY(cudaEventRecord(ev[k & 1], st));
         return PM_OK;
     }
-    // wait for step k; its coefficients h_j = c[j] + c[k + 1 + j] and |w|
+    // wait for step k; its coefficients h_j = c[j] + c[k + 1 + j] and |w|, 0 where it is undefined,
+    // which ends the cycle
     pm_status wait(int k, const T** c, double* hn) {
         PM_CUDA_TRY(cudaEventSynchronize(ev[k & 1]));
         *c = host + (k & 1) * slot();
-        *hn = positive(*reinterpret_cast<const double*>(*c + 2 * (k + 1)));
+        const double norm = *reinterpret_cast<const double*>(*c + 2 * (k + 1));
+        *hn = norm > 0.0 ? norm : 0.0;
         return PM_OK;
     }
 };

@@ -932,9 +932,9 @@ extern "C" pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_ga
     double bnorm = 0.0;
     if ((st = steps.begin(rhs, V, b->st, &bnorm)) != PM_OK) { cleanup(); return st; }   // x = 0: r = rhs
     int iters = 0;
-    double relres = bnorm > 0 ? 1.0 : 0.0;
+    double relres = bnorm == 0.0 ? 0.0 : std::isfinite(bnorm) ? 1.0 : NAN;
     std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
-    if (bnorm > 0) {
+    if (relres > tol) {
         size_t fr = 0, total = 0;
         const size_t need = sizeof(double) * (size_t)n * n;
         if (cudaMemGetInfo(&fr, &total) == cudaSuccess &&
@@ -951,7 +951,7 @@ extern "C" pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_ga
         PM_TRY(apply_any(b, A, V + (size_t)k * n, w));
         return steps.step(V, n, k, w, b->st);
     };
-    while (st == PM_OK && bnorm > 0 && relres > tol && iters < maxit) {
+    while (st == PM_OK && relres > tol && iters < maxit) {       // an undefined residual ends it
         std::fill(g.begin(), g.end(), 0.0);
         g[0] = beta;
         int k = 0, started = 0;

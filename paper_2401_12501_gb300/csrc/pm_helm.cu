@@ -523,9 +523,9 @@ extern "C" pm_status pm_solve_c(pm_surface* s, const double* f, double* u, doubl
     double fnorm = 0.0;
     PM_TRY(W.steps.begin(W.f, W.V, st, &fnorm));          // x = 0: the first residual is f
     int iters = 0, cycles = 0;
-    double relres = 0.0;
+    double relres = fnorm == 0.0 ? 0.0 : NAN;
     pm_status result = PM_OK;
-    if (fnorm > 0.0) {
+    if (fnorm > 0.0 && std::isfinite(fnorm)) {
         PM_TRY(S.D.fill(s));
         std::vector<cplx> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
         const long long ldv = N;
@@ -538,7 +538,7 @@ extern "C" pm_status pm_solve_c(pm_surface* s, const double* f, double* u, doubl
         double beta = fnorm;
         for (;;) {
             relres = beta / fnorm;
-            if (relres <= tol || iters >= maxit) break;
+            if (!(relres > tol) || iters >= maxit) break;       // an undefined residual ends it
             // one cycle of GMRES(m) on A d = r, x += d; V_0 = r / |r|
             std::fill(g.begin(), g.end(), cplx(0.0));
             g[0] = beta;
@@ -601,11 +601,11 @@ extern "C" pm_status pm_solve_c(pm_surface* s, const double* f, double* u, doubl
                 break;
             }
         }
-        if (!(relres <= tol)) {
-            pm_set_error("pm_solve_c: relative residual %.3e above %.3e after %d iterations",
-                         relres, tol, iters);
-            result = PM_ERR_NOT_CONVERGED;
-        }
+    }
+    if (!(relres <= tol)) {
+        pm_set_error("pm_solve_c: relative residual %.3e above %.3e after %d iterations", relres, tol,
+                     iters);
+        result = PM_ERR_NOT_CONVERGED;
     }
     // u = K~ sigma (eq. representation; no projection for c != 0)
     if (S.D.MR) PM_TRY(S.dense(S.D.MK, W.x, 0, W.u));

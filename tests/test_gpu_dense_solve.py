@@ -89,3 +89,38 @@ def edge_solve(ctx, monkeypatch, kind, n, p, M, F):
     both(monkeypatch, solve)
     b.close()
     S.close()
+
+
+# data whose norm is undefined or overflows: no relative residual can be met, whichever way the
+# operator is applied
+@pytest.mark.parametrize("bad", [np.inf, np.nan, 1e200])
+@pytest.mark.parametrize("hbm", [None, "0"])
+def test_undefined_data_do_not_converge(ctx, monkeypatch, bad, hbm):
+    import paper_2401_12501_gb300 as pm
+    from paper_2401_12501_gb300._lib import PmError
+    if hbm is not None:
+        monkeypatch.setenv("PM_FAKE_HBM_BYTES", hbm)
+    s = cubed_sphere(1, 4, axes=(1.0, 1.5, 2.0))
+    S = pm.Surface.from_fixture(ctx, s)
+    S.set_coeff_c(np.ones(s.N), None, np.full(s.N, 3.0))
+    f = np.ones(s.N)
+    f[5] = bad
+    with pytest.raises(PmError, match="NOT_CONVERGED"):
+        S.solve_c(f)
+    S.close()
+
+    band = bands.torus_band(2, 3, 5, 6, 4)
+    co = bands.constant_band_coefficient(band)
+    S = pm.Surface.from_fixture(ctx, band.surface)
+    S.set_coeff(co.a, co.grad_a)
+    patch, uv = bands.edge_patches(band)
+    b = pm.BoundaryValueProblem(S, band.curves, np.ones(band.M), np.ones(4 * band.M), patch, uv,
+                                kind="dirichlet")
+    f, fg = np.ones(S.N), np.ones(b.Me)
+    for v in (f, fg):
+        v[2] = bad
+        with pytest.raises(PmError, match="NOT_CONVERGED"):
+            b.solve(f, fg)
+        v[2] = 1.0
+    b.close()
+    S.close()
