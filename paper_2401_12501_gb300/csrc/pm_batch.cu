@@ -1352,10 +1352,11 @@ struct MGroup {                // instances on one geometry (a surface and its c
 // g_k' = grad a_k / (2 a_k): q (q - H) and r / r^2 once a pair (15 operations), three FMAs a field,
 // one a right-hand side; a_k/pi multiplies the finished sums.  Bound by the FMA pipe: 59
 // operations for 4 fields x 8 right-hand sides, where A, B and g in the pair cost 78 in
-// two halves of 2 fields (24,576 nodes, 8 x 8 columns: a batch solve's sums 75.2 -> 51.8 ms).
+// two halves of 2 fields (24,576 nodes, 8 x 8 columns: a batch solve's sums 75.2 -> 52 ms).
 // The compensated sums lie in shared memory (they are touched every
-// 288 sources), which leaves the registers to four blocks an SM at FB = 4.
-constexpr int kGeoSt = 96;               // sources a stage
+// kTile sources), which leaves the registers to four blocks an SM at FB = 4.
+constexpr int kGeoSt = 64;               // sources a stage
+static_assert(kTile % kGeoSt == 0, "a plain float32 run is as long as in the other sums, kTile sources");
 template <int FB, int RB>
 __global__ void __launch_bounds__(kThreads, 4)
 k_mgeo32(const MGroup* __restrict__ G, const MInst* __restrict__ I,
@@ -1464,7 +1465,7 @@ k_mgeo32(const MGroup* __restrict__ G, const MInst* __restrict__ I,
             if (nf == FB) pairs(len, std::true_type{});
             else pairs(len, std::false_type{});
             fill += len;
-            if (fill > 256) flush();
+            if (fill == kTile) flush();
         }
         flush();
         if (i < N) {
