@@ -463,6 +463,12 @@ pm_status pm_selftest_fflog(pm_surface* s, const float* xh, const float* xl, int
                             double* out);
 
 /*
+ * Diagnostic: the float64 reciprocal and logarithm of the library's float64 sums at n host
+ * values (x >= 0, infinite or NaN), written to rcp and lg (host).
+ */
+pm_status pm_selftest_fast64(const double* x, int n, double* rcp, double* lg);
+
+/*
  * Self-test of the FMM's M2L offset classes (host code only, no device call):
  * for the 343 box offsets d = (dx, dy, dz) in [-3, 3]^3, entry
  * k = ((dx + 3) * 7 + (dy + 3)) * 7 + (dz + 3) of cls[343] receives the class

@@ -36,7 +36,7 @@ EXPORTS = ["pm_default_opts", "pm_ctx_create", "pm_ctx_destroy", "pm_surface_cre
            "pm_surface_destroy", "pm_surface_info", "pm_surface_set_coeff", "pm_apply_R",
            "pm_apply_K", "pm_apply_part", "pm_surface_get_near", "pm_solve",
            "pm_status_str", "pm_last_error", "pm_profile_enable", "pm_profile_read",
-           "pm_surface_tune", "pm_selftest_fflog", "pm_smooth_remainder_f32_noalloc",
+           "pm_surface_tune", "pm_selftest_fflog", "pm_selftest_fast64", "pm_smooth_remainder_f32_noalloc",
            "pm_surface_fmm_stats", "pm_server_create", "pm_server_destroy", "pm_server_submit",
            "pm_server_poll", "pm_server_wait", "pm_server_stats", "pm_server_submit_desc",
            "pm_server_wait_ex", "pm_server_stats_ex", "pm_server_configure", "pm_solve_multi", "pm_surface_set_knobs",
@@ -146,6 +146,7 @@ def load(path: str = LIB_PATH) -> C.CDLL:
     lib.pm_server_stats_ex.argtypes = [P, C.POINTER(C.c_longlong), C.POINTER(C.c_size_t),
                                        C.POINTER(C.c_size_t), C.POINTER(C.c_int)]
     lib.pm_selftest_fflog.argtypes = [P, P, P, C.c_int, P]
+    lib.pm_selftest_fast64.argtypes = [P, C.c_int, P, P]
     lib.pm_smooth_remainder_f32_noalloc.argtypes = [C.c_int, P, P, P, P, P, P, P, P]
     lib.pm_surface_info.argtypes = [P, C.POINTER(C.c_int), C.POINTER(C.c_int)]
     lib.pm_surface_set_coeff.argtypes = [P, P, P]

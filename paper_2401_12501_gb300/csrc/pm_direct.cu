@@ -384,6 +384,14 @@ k_direct_64(const pm_d4* __restrict__ src, const double* __restrict__ x,
     if (i < N) partial[(size_t)blockIdx.y * N + i] = KERNEL_K ? acc / (4.0 * M_PI) : acc;
 }
 
+__global__ void k_fast64_test(const double* __restrict__ x, int n, double* __restrict__ rcp,
+                              double* __restrict__ lg) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    rcp[k] = pm_rcp64(x[k]);
+    lg[k] = pm_log64(x[k]);
+}
+
 }  // namespace
 
 // Targets per thread of the float32 sums: the knob when set, else 2 for the
@@ -589,5 +597,28 @@ extern "C" pm_status pm_smooth_remainder_f32_noalloc(int N, const float* x, cons
     k_direct_R32<2><<<grid, kThreads, 0, st>>>(src, tgt, N, chunk, eps2, part, nullptr, Fresh{});
     k_noalloc_reduce<<<pm_ceil_div(N, 256), 256, 0, st>>>(N, nsplit, part, out);
     PM_CUDA_TRY(cudaGetLastError());
+    return PM_OK;
+}
+
+extern "C" pm_status pm_selftest_fast64(const double* x, int n, double* rcp, double* lg) {
+    if (!x || !rcp || !lg || n < 1) {
+        pm_set_error("pm_selftest_fast64: NULL argument or n < 1");
+        return PM_ERR_INVALID_ARG;
+    }
+    double* d = nullptr;                 // x, 1/x, log x
+    PM_TRY(pm_dmalloc(&d, 3 * (size_t)n));
+    const size_t bytes = sizeof(double) * n;
+    cudaError_t e = cudaMemcpy(d, x, bytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        k_fast64_test<<<pm_ceil_div(n, 256), 256>>>(d, n, d + n, d + 2 * (size_t)n);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(rcp, d + n, bytes, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(lg, d + 2 * (size_t)n, bytes, cudaMemcpyDeviceToHost);
+    pm_dfree(d);
+    if (e != cudaSuccess) {
+        pm_set_error("pm_selftest_fast64: %s", cudaGetErrorString(e));
+        return PM_ERR_CUDA;
+    }
     return PM_OK;
 }
