@@ -402,7 +402,8 @@ pm_status pm_bvp_apply(pm_bvp* b, const double* sigma, const double* mu, double*
  * K_gamma mu; sigma [N] and mu [Me] are written when not NULL.  info as for pm_solve
  * (refinements 0).  PM_ERR_NOT_CONVERGED (u, sigma, mu still written) when tol is
  * not reached.  While it runs a solve holds the system's matrix, 8 (N + Me)^2 bytes,
- * where it leaves max(1 GiB, 2 %) of the device free; else it goes pair by pair. */
+ * where that is at most half of the free device memory and leaves max(1 GiB, 2 %) of
+ * the device free; else it goes pair by pair. */
 pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_gamma, double tol,
                        int maxit, double* u, double* sigma, double* mu, pm_solve_info* info);
 
@@ -649,8 +650,9 @@ pm_status pm_apply_c(pm_surface* s, int which_K, const double* sigma, double* ou
  * relative residual, removed_mean = 0.  PM_ERR_NOT_CONVERGED (u and info still
  * written) when the tolerance is not met; PM_ERR_NO_COEFF if the surface is not
  * in c mode; PM_ERR_INVALID_ARG for NULL f or u, tol <= 0 or maxit < 1.  While it
- * runs a solve holds the operators as dense matrices, 32 N^2 bytes, where they leave
- * max(1 GiB, 2 %) of the device free; else it goes pair by pair.
+ * runs a solve holds the operators as dense matrices, 32 N^2 bytes, where they take at
+ * most half of the free device memory and leave max(1 GiB, 2 %) of the device free;
+ * else it goes pair by pair.
  */
 pm_status pm_solve_c(pm_surface* s, const double* f, double* u, double tol, int maxit,
                      double* sigma_out, pm_solve_info* info);

@@ -298,6 +298,13 @@ size_t pm_free_hbm_bytes() {
     return fr;
 }
 
+bool pm_matrix_fits(size_t need) {
+    size_t fr = 0, total = 0;
+    if (cudaMemGetInfo(&fr, &total) != cudaSuccess) return false;
+    fr = pm_free_hbm_bytes();
+    return need <= fr / 2 && need + std::max<size_t>(1ull << 30, total / 50) <= fr;
+}
+
 static void free_surface(pm_surface* s) {
     if (!s) return;
     if (s->ctx) cudaSetDevice(s->ctx->device);

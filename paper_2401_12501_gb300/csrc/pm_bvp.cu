@@ -935,11 +935,8 @@ extern "C" pm_status pm_bvp_solve(pm_bvp* b, const double* f, const double* f_ga
     double relres = bnorm == 0.0 ? 0.0 : std::isfinite(bnorm) ? 1.0 : NAN;
     std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
     if (relres > tol) {
-        size_t fr = 0, total = 0;
         const size_t need = sizeof(double) * (size_t)n * n;
-        if (cudaMemGetInfo(&fr, &total) == cudaSuccess &&
-            need + std::max<size_t>(1ull << 30, total / 50) <= pm_free_hbm_bytes() &&
-            cudaMallocAsync((void**)&A, need, b->st) != cudaSuccess)
+        if (pm_matrix_fits(need) && cudaMallocAsync((void**)&A, need, b->st) != cudaSuccess)
             A = nullptr;
         cudaGetLastError();
         if (A && (st = fill_sys(b, A)) != PM_OK) { cleanup(); return st; }

@@ -355,9 +355,7 @@ struct HelmDense {
     // (7.1 and 2.0 ms with the kernels from tables and the steps of pm_arnoldi.cuh).
     pm_status fill(pm_surface* s) {
         const size_t N = s->N, need = 2 * sizeof(double2) * N * N;
-        size_t fr = 0, total = 0;
-        PM_CUDA_TRY(cudaMemGetInfo(&fr, &total));
-        if (need + std::max<size_t>(1ull << 30, total / 50) > pm_free_hbm_bytes()) return PM_OK;
+        if (!pm_matrix_fits(need)) return PM_OK;
         if (cudaMallocAsync((void**)&MR, need, st) != cudaSuccess) {
             cudaGetLastError();
             MR = nullptr;

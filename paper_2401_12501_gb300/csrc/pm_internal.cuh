@@ -328,6 +328,10 @@ pm_status pm_ffmm_sum(pm_surface* s, PmFfmmWork* W, int kind, int nops, pm_surfa
 // free device memory now (cudaMemGetInfo), or the value of the environment variable
 // PM_FAKE_HBM_BYTES when set (a host-side stand-in for a full device) (pm_api.cu)
 size_t pm_free_hbm_bytes();
+// may a solve hold a matrix of this many bytes while it runs: half of what is free at most, and
+// not the last max(1 GiB, 2 %) of the device.  The rest stays for the program's other threads,
+// whose allocations, unlike the solve, have no smaller way (pm_api.cu)
+bool pm_matrix_fits(size_t need);
 
 // Chebyshev FMM (pm_fmm.cu)
 pm_status pm_fmm_build(pm_surface* s);

@@ -124,3 +124,20 @@ def test_undefined_data_do_not_converge(ctx, monkeypatch, bad, hbm):
         v[2] = 1.0
     b.close()
     S.close()
+
+
+# matrices of 6.1 GB with 12.1 GB free: more than half, so the pairs are summed at every step;
+# with 64 GB free they are evaluated once
+@pytest.mark.parametrize("free,dense", [(12.1e9, False), (64e9, True)])
+def test_matrix_takes_half_of_the_free_memory_at_most(ctx, monkeypatch, free, dense):
+    import paper_2401_12501_gb300 as pm
+    from paper_2401_12501_gb300._lib import PM_PHASE_DIRECT64
+    s = cubed_sphere(6, 8, axes=(1.0, 1.5, 2.0))
+    S = pm.Surface.from_fixture(ctx, s)
+    S.set_coeff_c(np.ones(s.N), None, np.full(s.N, 3.0))
+    monkeypatch.setenv("PM_FAKE_HBM_BYTES", str(int(free)))
+    S.profile()
+    _, info = S.solve_c(s.nodes[:, 0] + 0j, tol=1e-3)
+    _, sums = S.profile_read(PM_PHASE_DIRECT64)
+    assert info.iterations > 1 and (sums == 1) == dense
+    S.close()
