@@ -56,3 +56,33 @@ def test_pairs(surface, c):
         tol = 4e-14 * (1.0 + abs(k[j]) * np.linalg.norm(x[far] - x[j], axis=1))
         assert (np.abs(K[far] - wK) <= tol * np.abs(wK)).all()
         assert np.abs(R[far] - wR).max() <= 10 * tol.max() * np.abs(wR).max()
+
+
+# R entry by entry, with a gradient of a: each of its terms is g, g' or q g times factors good to a
+# few 2^-53, so an entry may be off by twice K's tolerance (the derivative's and the oracle's) of
+# the sum of its terms' moduli, the cosines taken as 1
+@pytest.mark.parametrize("c", CS)
+def test_remainder_entries(surface, c):
+    from oracle.kernels import green_scaled, scaled_pair_c, wavenumber
+    sf, S = surface
+    x, n, H = sf.nodes, sf.normals, sf.curvature
+    a = 1.0 + 0.2 * x[:, 0]
+    ga = 0.2 * (np.array([1.0, 0.0, 0.0]) - n * n[:, :1])
+    cv = c * (1.0 + 0.1 * x[:, 1])
+    S.set_coeff_c(a, ga, cv)
+    rp, bp, _, _ = S.get_near(corrections=False)
+    k = wavenumber(cv, a)
+    for j in (0, 57, 140, sf.N - 1):
+        e = np.zeros(sf.N)
+        e[j] = 1.0
+        R = S.apply_c(e, "R")
+        far = np.flatnonzero([j // 9 not in bp[rp[i]:rp[i + 1]] for i in range(sf.N)])
+        r = np.linalg.norm(x[far] - x[j], axis=1)
+        g, g1, _ = (np.abs(v) for v in green_scaled(r, k[j]))
+        want = np.array([scaled_pair_c(x[i], n[i], H[i], a[i], ga[i], cv[i], x[j], k[j])[0] for i in far])
+        q = abs(k[j]) ** 2
+        terms = ((np.linalg.norm(ga[far], axis=1) + 2.0 * a[far] * np.abs(H[far]) + 2.0 * a[far] / r) * g1
+                 + (np.abs(cv[far]) + 2.0 * a[far] * q) * g)
+        tol = 4e-14 * (1.0 + abs(k[j]) * r)
+        weight = sf.weights[j] / a[j]
+        assert (np.abs(R[far] - weight * want) <= 2.0 * tol * weight * terms).all()
