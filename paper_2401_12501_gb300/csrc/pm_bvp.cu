@@ -82,7 +82,6 @@ struct pm_bvp {
 namespace {
 
 constexpr int kT = 256;
-constexpr int kTile = 256;
 
 // mu_o[j] = sum_k I_c[j][k] mu[off_c + k] for the curve c of oversampled point j
 __global__ void k_bvp_interp(const double* __restrict__ I, const int* __restrict__ ioff,

@@ -221,14 +221,6 @@ struct FloatDigits {
     }
 };
 
-__device__ __forceinline__ void mma_f16(float* c, const unsigned int* a, uint2 b) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
-}
-
 // entries of the pair (target record t, source at (A, B) hi and lo) into e[0 .. NM)
 template <int KIND>
 __device__ __forceinline__ void entries(const float* t, float4 A, float4 B, const float4* stab, ff* e) {
@@ -380,7 +372,7 @@ k_ffmm(const float4* __restrict__ src, const float4* __restrict__ tg, const doub
 #pragma unroll
                 for (int da = 0; da < kQmDigits; ++da)
 #pragma unroll
-                    for (int db = 0; da + db < kSums && db < kQmDigits; ++db) mma_f16(acc[da + db], a[da], bb[db]);
+                    for (int db = 0; da + db < kSums && db < kQmDigits; ++db) qm_mma(acc[da + db], a[da], bb[db]);
             }
 #pragma unroll
             for (int c = 0; c < 4; ++c) {

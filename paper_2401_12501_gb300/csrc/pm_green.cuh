@@ -365,54 +365,6 @@ __host__ __device__ inline void green_scaled_any(double r, double q, double* out
     out[1] = out[3] = out[5] = 0.0;
 }
 
-// One source's a(y) R and a(y) K for real q(y) = c(y)/a(y), as (re, im) pairs
-// out[0..1] = a(y) R, out[2..3] = a(y) K (eq. explicit_remainder with
-// a(y) G = g(r; k(y)), k(y)^2 = q(y)), r = x - y:
-//   a(y) R = (gb . r^) g' - a(x) (g'' - g'/r) (n.r^)^2 - 2 a(x) H(x) (n.r^) g'
-//            + (c(x) - a(x) q(y)) g,          a(y) K = g,
-// gb = grad_G a(x), n and H the target's normal and mean curvature.
-__host__ __device__ inline void pair_rk_c(double rx, double ry, double rz, double nx, double ny,
-                                          double nz, double H, double a, double gbx, double gby,
-                                          double gbz, double c, double q, double* out)
-{
-    const double r = sqrt(rx * rx + ry * ry + rz * rz);
-    const double inv_r = 1.0 / r;
-    double g[6];
-    green_scaled_any(r, q, g);
-    const double nr = (nx * rx + ny * ry + nz * rz) * inv_r;
-    const double gr = (gbx * rx + gby * ry + gbz * rz) * inv_r;
-    const double t2 = a * nr * nr;
-    const double t1 = gr - 2.0 * a * H * nr;
-    const double t0 = c - a * q;
-    out[0] = t1 * g[2] - t2 * (g[4] - g[2] * inv_r) + t0 * g[0];
-    out[1] = t1 * g[3] - t2 * (g[5] - g[3] * inv_r) + t0 * g[1];
-    out[2] = g[0];
-    out[3] = g[1];
-}
-
-// pair_rk_c with complex c(x) and q(y) (out as in pair_rk_c): the real-q path when
-// q is real, the complex kernels otherwise.
-__host__ __device__ inline void pair_rk_cz(double rx, double ry, double rz, double nx, double ny,
-                                           double nz, double H, double a, double gbx, double gby,
-                                           double gbz, cplx_d c, cplx_d q, const double* g16t,
-                                           const double* g16w, double* out)
-{
-    const double r = sqrt(rx * rx + ry * ry + rz * rz);
-    const double inv_r = 1.0 / r;
-    double g[6];
-    if (q.im == 0.0) green_scaled_any(r, q.re, g);
-    else green_scaled_cz(r, q, g16t, g16w, g);
-    const double nr = (nx * rx + ny * ry + nz * rz) * inv_r;
-    const double gr = (gbx * rx + gby * ry + gbz * rz) * inv_r;
-    const double t2 = a * nr * nr;
-    const double t1 = gr - 2.0 * a * H * nr;
-    const cplx_d t0 = {c.re - a * q.re, c.im - a * q.im};       // c(x) - a(x) q(y)
-    out[0] = t1 * g[2] - t2 * (g[4] - g[2] * inv_r) + (t0.re * g[0] - t0.im * g[1]);
-    out[1] = t1 * g[3] - t2 * (g[5] - g[3] * inv_r) + (t0.re * g[1] + t0.im * g[0]);
-    out[2] = g[0];
-    out[3] = g[1];
-}
-
 #ifdef __CUDACC__
 // ---------------------------------------------------------------------------
 // Device evaluation by tables.  The functions above cost 500 (J, Y), 170 (K) and some 10,000
@@ -559,7 +511,11 @@ __device__ __forceinline__ void green_by_tables(double r, double inv_r, const Gr
     green_off_tables(r, G.q, g16t, g16w, out);
 }
 
-// pair_rk_cz by the tables
+// One source's a(y) R and a(y) K with q(y) = c(y)/a(y), as (re, im) pairs out[0..1] = a(y) R,
+// out[2..3] = a(y) K (eq. explicit_remainder with a(y) G = g(r; k(y)), k(y)^2 = q(y)), r = x - y:
+//   a(y) R = (gb . r^) g' - a(x) (g'' - g'/r) (n.r^)^2 - 2 a(x) H(x) (n.r^) g'
+//            + (c(x) - a(x) q(y)) g,          a(y) K = g,
+// gb = grad_G a(x), n and H the target's normal and mean curvature.
 __device__ __forceinline__ void pair_rk_tab(double rx, double ry, double rz, double nx, double ny,
                                             double nz, double H, double a, double gbx, double gby,
                                             double gbz, cplx_d c, const GreenQ& G, const GreenTab& T,

@@ -73,7 +73,6 @@ constexpr int PM_MAX_P_API = 11;     // quadrature kernels give one basis entry 
 constexpr int PM_GL16 = 16;          // points per quadrature panel
 constexpr int PM_TRI_MAX_P = 8;      // triangle patches: order p <= 8, p (p + 1) / 2 <= 36 nodes
 constexpr int PM_TRI_MAX_NT = 36;
-constexpr int PM_RADIAL_PANELS = 4;  // self rule: [0,L/8],[L/8,L/4],[L/4,L/2],[L/2,L]
 
 // Host-computed tables for the quadrature kernels (constant memory).
 struct QuadTables {

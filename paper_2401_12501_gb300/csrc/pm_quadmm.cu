@@ -62,14 +62,6 @@ struct QmShape {
     static constexpr int per_warp = (tiles2 + 7) / 8;
 };
 
-__device__ __forceinline__ void mma_f16(float* c, const unsigned int* a, unsigned int b0, unsigned int b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 template <bool TRANS>
 __device__ __forceinline__ void ldmatrix4(unsigned int* r, const __half* p) {
     const unsigned int a = (unsigned int)__cvta_generic_to_shared(p);
@@ -188,7 +180,7 @@ k_qm(const int4* __restrict__ items, const int4* __restrict__ cols, const __half
                 for (int da = 0; da < kQmDigits; ++da)
 #pragma unroll
                     for (int db = 0; da + db < kQmSums && db < kQmDigits; ++db)
-                        mma_f16(acc[da + db], a[da], b[db].x, b[db].y);
+                        qm_mma(acc[da + db], a[da], b[db]);
             }
             // sum over the digits' weights in units 512^-5, then to double: two exact steps
             const int c0 = nt * 8 + 2 * t4;
@@ -268,7 +260,7 @@ k_qm(const int4* __restrict__ items, const int4* __restrict__ cols, const __half
                     for (int da = 0; da < kQmDigits; ++da)
 #pragma unroll
                         for (int db = 0; da + db < kQmSums && db < kQmDigits; ++db)
-                            mma_f16(acc[da + db], a[da], b[db].x, b[db].y);
+                            qm_mma(acc[da + db], a[da], b[db]);
                 }
                 // a tile's sum to 2^-52 of its largest term (58 bits), two exact steps
 #pragma unroll

@@ -48,6 +48,15 @@ __device__ __forceinline__ unsigned int qm_digit2(unsigned long long a, unsigned
     return *reinterpret_cast<const unsigned int*>(&h);               // 0x6500 = 1280
 }
 
+// c += a b: 16 x 16 digits by 16 x 8
+__device__ __forceinline__ void qm_mma(float* c, const unsigned int* a, uint2 b) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
+}
+
 // Two neighbouring basis values k, k + 1 (k even) of a point into the table.
 __device__ __forceinline__ void qm_put(const QmTable& T, size_t tile, int point, int k, double a,
                                        double b) {
