@@ -69,8 +69,9 @@ __global__ void k_prep32(const double* __restrict__ sigma, const double* __restr
 // Strengths formed where the sums stage their sources, from the density itself (sigma null: src
 // holds them, k_prep32).  One launch less an apply: 2.5-3 us of host time and as much of the
 // device's, against a multiplication and a conversion on the float64 pipe for every source a
-// block stages, about 3 % of the sums.  Worth it up to kFreshNodes.  The first block column
-// leaves sig32 for the near field.
+// block stages, about 3 % of the sums.  Worth it up to kFreshNodes: a remainder apply 71.8 ->
+// 67.7 us at 9,600 nodes, 132.7 -> 130.0 at 13,824, 157.9 -> 155.5 at 15,000 (parametrix 49.1 ->
+// 45.1, 76.1 -> 72.2, 94.9 -> 90.9).  The first block column leaves sig32 for the near field.
 constexpr int kFreshNodes = 16384;
 struct Fresh {
     const double *sigma = nullptr, *wa = nullptr;

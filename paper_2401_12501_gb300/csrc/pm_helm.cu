@@ -352,7 +352,8 @@ struct HelmDense {
     // 32 N^2 bytes.  One evaluation of the pairs serves every step, residual and the
     // representation; the pair sums evaluate all of them each time.  A solve to 1e-12 on the
     // GB300: 3,456 nodes with c/a > 0 206 -> 14.7 ms, 864 nodes with complex c 878 -> 28.7 ms
-    // (7.1 and 2.0 ms with the kernels from tables and the steps of pm_arnoldi.cuh).
+    // (7.2 to 8.0 and 2.0 to 2.4 ms, by the number of steps the data take, with the kernels from
+    // tables and the steps of pm_arnoldi.cuh).
     pm_status fill(pm_surface* s) {
         const size_t N = s->N, need = 2 * sizeof(double2) * N * N;
         if (!pm_matrix_fits(need)) return PM_OK;

@@ -27,7 +27,7 @@
 // Weights of an item (a range of tiles) go to a slot of `partial`; k_qm_reduce adds the slots of
 // a block in a fixed order, so the results do not depend on the grouping.
 // Two blocks an SM up to n = 64 (their shared memory is 113 KB), one above.
-// GB300: a near field of 2,400 nodes (n = 100) 294 -> 71 ms with everything around it, 2,880
+// GB300: a near field of 2,400 nodes (n = 100) 286 -> 59 ms with everything around it, 2,880
 // nodes of triangles (n = 36) 705 -> 53 ms, against blocks that kept both contractions on the
 // float64 pipe; that pipe is 73 % busy at n = 36 and n = 64, 45 % at n = 100, where one block
 // an SM leaves it idle in the tensor phases.
