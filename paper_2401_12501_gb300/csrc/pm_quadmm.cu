@@ -25,7 +25,7 @@
 // Block: 256 threads, kQmCols columns, tiles of 64 points.  Warp w evaluates the integrands of
 // column w (a lane two points), so a column's largest |F| of a tile is a warp reduction.
 // Weights of an item (a range of tiles) go to a slot of `partial`; k_qm_reduce adds the slots of
-// a block in a fixed order, so the results do not depend on the grouping.
+// a block in a fixed order, so the results do not depend on which columns share a block.
 // Two blocks an SM up to n = 64 (their shared memory is 113 KB), one above.
 // GB300: a near field of 2,400 nodes (n = 100) 286 -> 59 ms with everything around it, 2,880
 // nodes of triangles (n = 36) 705 -> 53 ms, against blocks that kept both contractions on the
@@ -391,7 +391,8 @@ struct Buffers {
 
 // Room for a batch's table and slots.  Larger batches leave fewer half-empty last waves; these
 // keep what a build takes beside its results below 0.4 GB.  On a device without that much left
-// the batches are halved, up to five times; the weights do not depend on it.
+// the batches are halved, up to five times, which cuts the self rules into other pieces: the weights
+// change by rounding alone (2e-15 of the largest).
 constexpr size_t kTableBytes = 192u << 20, kSlotBytes = 128u << 20;
 
 }  // namespace
