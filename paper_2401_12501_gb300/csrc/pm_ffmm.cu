@@ -30,11 +30,12 @@
 // (5.7) and with 16 6.5 (9.6), RG with 8 operators of 8 columns 24.4 (eight times 5.7).  An
 // m16n8k16 takes two clocks an SM: RG keeps the tensor pipe 55 % busy; R1 and K are bound by the
 // entries' latency.  Errors against float64 are at most 0.7 of
-// k_direct_multi_ff's on even patches (kFfmSpread).
+// k_direct_multi_ff's on even patches (kFmSpread).
 #include "pm_ff.cuh"
 #include "pm_quadmm.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
 namespace {
@@ -48,13 +49,14 @@ constexpr int kFmCols = 64;
 constexpr size_t kBufWords = (size_t)4 * kKS * kQmDigits * 4 * 32;
 constexpr int kRecord = 20;                // floats of a target in shared memory
 // The remainder's fixed point serves while no row's largest |q^2 - H q| or 1/r stands more than
-// this factor above the row's mean over the surface: every entry of a row is rounded to some 2^-54
-// of its largest, a typical one to S 2^-54 of itself at a factor S, and float-float arithmetic
-// rounds each to about 2^-44.  Surfaces of even patches have 2^5 to 2^10.5 (1,500 to 400,000
-// nodes); patches halved towards a point pass 2^11 at a size of 2^-8.  Errors against float64
-// over those of k_direct_multi_ff, 8 columns: 0.1 to 0.2 at 2^8 (24,576 nodes of a torus), 0.4 to
-// 0.7 at 2^10.7 (flat ellipsoid, 21,600), 0.7 to 1.3 at 2^15.5 and 49 to 53 at 2^21.5 (patches
-// halved 12 and 18 times).  log r^2 has no such rows and is taken whenever it is defined.
+// this factor above the row's root mean square.  Every entry of a row is rounded to some 2^-54 of
+// its largest, which is S 2^-54 of their root mean square at a factor S, and float-float
+// arithmetic rounds each to about 2^-44 of itself.  Surfaces of even patches have 2^5 to 2^10.3
+// (1,500 to 400,000 nodes; 2^8.3 with the two kinks of a star); patches halved towards a point pass
+// 2^11 at a size of 2^-8.  Errors against float64 over those of k_direct_multi_ff, 8 columns: 0.1
+// to 0.2 at 2^7.4 (torus, 24,576 nodes), 0.04 to 0.1 at 2^8.3 (star, 24,576), 0.4 to 0.7 at 2^10.3
+// (flat ellipsoid, 21,600), 0.7 to 1.3 at 2^15.4 and 49 to 53 at 2^21.4 (patches halved 12 and 18
+// times).  log r^2 has no such rows and is taken whenever it is defined.
 constexpr float kFmSpread = 2048.f;
 
 // Columns of one launch: operators in order, first[q] <= column < first[q + 1]
@@ -70,28 +72,30 @@ __device__ __forceinline__ int op_of(const Cols& C, int col) {
 }
 
 // What the fixed point of a row is laid out for, by target i: its pairs' largest |q^2 - H q| and
-// 1/r, their means over the surface and the largest |log r^2|, of the sources of one split;
-// part[(split 5 + k) N + i] in the order max, max, sum, sum, max, and the sources' weights in
-// area[split N + i].  The differences and n.r are those of the sums (float-float): n.r is of the
+// 1/r, the sums of their squares over the sources, weighted as the strengths are by the quadrature,
+// and the largest |log r^2|, of the sources of one split; part[(split 5 + k) N + i] in the order
+// max, max, sum, sum, max, and the sum of the squared weights in sw[split N + i].  The sums are
+// free of the surface's size L, L^2 its area: |q^2 - H q| L^2, L / r, weights N w / L^2.  The differences and n.r are those of the sums (float-float): n.r is of the
 // order r^2, and of coordinates rounded to float32 its error grows past it where nodes are close.
 __global__ void __launch_bounds__(128)
 k_fm_rows(const float4* __restrict__ src, const double* __restrict__ nrm, const double* __restrict__ H,
-          const double* __restrict__ w, int N, int chunk, float* __restrict__ part,
-          float* __restrict__ area) {
+          const double* __restrict__ w, int N, int chunk, double area, float* __restrict__ part,
+          float* __restrict__ sw) {
     __shared__ float4 sa[128], sb[128];
     const int i = blockIdx.x * 128 + threadIdx.x, ii = min(i, N - 1);
     const float4 ta = src[2 * (size_t)ii], tb = src[2 * (size_t)ii + 1];
     ff n[3];
     for (int d = 0; d < 3; ++d) n[d] = ff_from_double(nrm[3 * (size_t)ii + d]);
     const float h = (float)H[ii];
-    float top0 = 0.f, top1 = 0.f, toplog = 0.f, sum0 = 0.f, sum1 = 0.f, sw = 0.f;
+    const float size2 = (float)area, size = sqrtf(size2);
+    float top0 = 0.f, top1 = 0.f, toplog = 0.f, sum0 = 0.f, sum1 = 0.f, sumw = 0.f;
     const int s0 = blockIdx.y * chunk, s1 = min(s0 + chunk, N);
     for (int base = s0; base < s1; base += 128) {
         __syncthreads();
         const int j = min(base + (int)threadIdx.x, N - 1);
         sa[threadIdx.x] = src[2 * (size_t)j];
         sb[threadIdx.x] = src[2 * (size_t)j + 1];
-        sb[threadIdx.x].w = (float)w[j];
+        sb[threadIdx.x].w = (float)(w[j] * N / area);
         __syncthreads();
         const int len = min(128, s1 - base);
         for (int k = 0; k < len; ++k) {
@@ -103,9 +107,10 @@ k_fm_rows(const float4* __restrict__ src, const double* __restrict__ nrm, const 
             const ff nr = ff_norm(ff_add_lazy(ff_add_lazy(ff_mul_lazy(n[0], dx), ff_mul_lazy(n[1], dy)),
                                               ff_mul_lazy(n[2], dz)));
             const float q = nr.h * inv, e0 = fabsf(q * (q - h)), e1 = sqrtf(inv);
-            sum0 = fmaf(b.w, e0, sum0);          // an undefined pair leaves the sums undefined
-            sum1 = fmaf(b.w, e1, sum1);
-            sw += b.w;
+            const float f0 = b.w * size2 * e0, f1 = b.w * size * e1;
+            sum0 = fmaf(f0, f0, sum0);           // an undefined pair leaves the sums undefined
+            sum1 = fmaf(f1, f1, sum1);
+            sumw = fmaf(b.w, b.w, sumw);
             top0 = fmaxf(top0, e0);
             top1 = fmaxf(top1, e1);
             toplog = fmaxf(toplog, fabsf(__logf(r2)));
@@ -118,16 +123,16 @@ k_fm_rows(const float4* __restrict__ src, const double* __restrict__ nrm, const 
     p[2 * (size_t)N] = sum0;
     p[3 * (size_t)N] = sum1;
     p[4 * (size_t)N] = toplog;
-    area[(size_t)blockIdx.y * N + i] = sw;
+    sw[(size_t)blockIdx.y * N + i] = sumw;
 }
 
 // bound[i], bound[N + i], bound[2 N]: the largest |q^2 - H q| and 1/r of target i and the largest
-// |log r^2| of all; bound[2 N + 1]: how far a row's largest entry stands above the row's mean, at
-// worst (infinity where a pair is undefined)
-__global__ void k_fm_bounds(int N, int nsplit, const float* __restrict__ part,
-                            const float* __restrict__ area, unsigned int* __restrict__ bound) {
+// |log r^2| of all; bound[2 N + 1]: how far a row's largest entry stands above the row's root mean
+// square, at worst (infinity where a pair is undefined)
+__global__ void k_fm_bounds(int N, int nsplit, double area, const float* __restrict__ part,
+                            const float* __restrict__ sw, unsigned int* __restrict__ bound) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float top0 = 0.f, top1 = 0.f, toplog = 0.f, sum0 = 0.f, sum1 = 0.f, sw = 0.f;
+    float top0 = 0.f, top1 = 0.f, toplog = 0.f, sum0 = 0.f, sum1 = 0.f, sumw = 0.f;
     for (int s = 0; s < nsplit && i < N; ++s) {
         const float* p = part + (size_t)s * 5 * N + i;
         top0 = fmaxf(top0, p[0]);
@@ -135,15 +140,17 @@ __global__ void k_fm_bounds(int N, int nsplit, const float* __restrict__ part,
         sum0 += p[2 * (size_t)N];
         sum1 += p[3 * (size_t)N];
         toplog = fmaxf(toplog, p[4 * (size_t)N]);
-        sw += area[(size_t)s * N + i];
+        sumw += sw[(size_t)s * N + i];
     }
     float over = 0.f;
     if (i < N) {
         bound[i] = __float_as_uint(top0);
         bound[N + i] = __float_as_uint(top1);
-        const bool defined = sum0 < 3e38f && sum1 < 3e38f && sw > 0.f;
+        const float size2 = (float)area, size = sqrtf(size2);
+        const bool defined = sum0 < 3e38f && sum1 < 3e38f && sumw > 0.f && sumw < 3e38f;
         over = !defined && N > 1 ? __int_as_float(0x7f800000)
-                                 : fmaxf(top0 > 0.f ? top0 * sw / sum0 : 0.f, top1 > 0.f ? top1 * sw / sum1 : 0.f);
+                                 : fmaxf(top0 > 0.f ? top0 * size2 * sqrtf(sumw / sum0) : 0.f,
+                                         top1 > 0.f ? top1 * size * sqrtf(sumw / sum1) : 0.f);
     }
     for (int o = 16; o > 0; o >>= 1) {
         over = fmaxf(over, __shfl_xor_sync(0xffffffffu, over, o));
@@ -489,10 +496,12 @@ static pm_status ffmm_ready(pm_surface* s, PmFfmmWork* W, bool* room, cudaStream
         const int ns = std::max(1, std::min({blocks, 16 * s->ctx->num_sms / blocks, 24}));
         const int chunk = pm_ceil_div(pm_ceil_div(N, ns), 128) * 128;
         // 6 ns N values in the digits' room of 192 N and more
-        float *part = reinterpret_cast<float*>(W->S), *area = part + (size_t)5 * ns * N;
+        float *part = reinterpret_cast<float*>(W->S), *sw = part + (size_t)5 * ns * N;
+        double area = 0.0;
+        for (double v : s->h_w) area += std::fabs(v);
         cudaMemsetAsync(W->bound, 0, bound_words(N) * sizeof(int), st);
-        k_fm_rows<<<dim3(blocks, ns), 128, 0, st>>>(s->src_ff, s->n, s->H, s->w, N, chunk, part, area);
-        k_fm_bounds<<<blocks, 128, 0, st>>>(N, ns, part, area, W->bound);
+        k_fm_rows<<<dim3(blocks, ns), 128, 0, st>>>(s->src_ff, s->n, s->H, s->w, N, chunk, area, part, sw);
+        k_fm_bounds<<<blocks, 128, 0, st>>>(N, ns, area, part, sw, W->bound);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(&W->spread, W->bound + 2 * (size_t)N + 1, sizeof(float), cudaMemcpyDeviceToHost, st);

@@ -313,7 +313,7 @@ struct PmFfmmWork {
     unsigned int* S = nullptr;      // the strengths' digits
     int* top = nullptr;             // per column: exponent of the largest strength
     unsigned int* bound = nullptr;  // the geometry's largest kernel values by target
-    float spread = 0.f;             // a target's largest value over its mean, at worst
+    float spread = 0.f;             // a target's largest value over its root mean square, at worst
 };
 void pm_ffmm_free(PmFfmmWork* W);
 size_t pm_ffmm_bytes(int N);        // device bytes of its buffers
